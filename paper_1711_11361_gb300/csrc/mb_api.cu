@@ -40,7 +40,7 @@ template <class T>
 int bulk_blocks_per_sm(int);
 double fp64_probe_rate(cudaStream_t st);
 template <class T>
-void launch_axisym_source(const InstDesc *, InstDyn *, int, int, int, cudaStream_t);
+void launch_axisym_source(const InstDesc *, InstDyn *, int, size_t, int, cudaStream_t);
 template <class T, class H>
 void launch_write_state(const InstDesc *, InstDyn *, const H *const *, const H *, int, int, int, int, cudaStream_t);
 template <class T, class H>
@@ -231,6 +231,24 @@ static const char *check_instance(const mb_grid &g, const mb_body &b, int prec, 
     return nullptr;
 }
 
+// bulk work items.  The FP32 Euler kernels: x sweep one warp per row, y sweep
+// one warp per 64 columns (two per thread) and yseg rows.  The scalar
+// kernels: units of 30 cells (x: one warp each; y: one CTA per 8 columns and
+// 30 rows)
+static void bulk_items(int prec, int yseg, InstDesc &I) {
+    if (prec == MB_FP32 && I.eq == MB_EULER) {
+        I.tiles_x[0] = 1;
+        I.tiles_x[1] = (I.nx + 63) / 64;
+        I.yseg = yseg;
+    } else {
+        I.tiles_x[0] = (I.nx + 29) / 30;
+        I.tiles_x[1] = (I.nx + 7) / 8;
+        I.yseg = 30;
+    }
+    I.ntiles[0] = I.tiles_x[0] * I.ny;
+    I.ntiles[1] = I.tiles_x[1] * ((I.ny + I.yseg - 1) / I.yseg);
+}
+
 // descriptor of one instance (device pointers and offsets into the shared
 // arrays are set by make_instance and relayout)
 static void describe_instance(int prec, int yseg, const mb_grid &g, double gamma, const mb_body &b,
@@ -290,15 +308,7 @@ static void describe_instance(int prec, int yseg, const mb_grid &g, double gamma
     }
     if (I.nv == 0) gcols = 0;
     I.gcol_max = gcols;
-    // bulk work items: x sweep one warp per row; y sweep one warp per 32
-    // columns (64 for the FP32 Euler kernel that carries two columns per
-    // thread) and 64-row segment
-    I.tiles_x[0] = 1;
-    I.ntiles[0] = g.ny;
-    const int ycols = (prec == MB_FP32 && base_equation(g.equation) == MB_EULER) ? 64 : 32;
-    I.tiles_x[1] = (g.nx + ycols - 1) / ycols;
-    I.yseg = yseg;
-    I.ntiles[1] = I.tiles_x[1] * ((g.ny + yseg - 1) / yseg);
+    bulk_items(prec, yseg, I);
 }
 
 // descriptor and device buffers of one instance
@@ -643,7 +653,10 @@ static mb_status do_sweep(mb_sim *s, int dir, double dt) {
             launch_bulk<double>(dir, eq, s->dd, s->dy, s->rec, s->n, s->total_tiles[dir], src, dst, last,
                                 s->tune_cta[dir], mode, dl, any_dall ? 1 : 0, st);
     };
-    const bool two_pass = s->prec == MB_FP32 && eq == MB_EULER;
+    // the FP32 Euler kernels always run in two passes (mb_set_overlap acts
+    // through defer_all); the scalar ones in one when the overlap is off
+    const bool packed = s->prec == MB_FP32 && eq == MB_EULER;
+    const bool two_pass = packed || s->overlap;
     if (two_pass && !s->timing) {
         // geometry and band fluxes (FP64 pipe, latency) on the side stream
         // while the bulk pass that needs no band data (FP32 pipe, HBM) runs
@@ -664,8 +677,12 @@ static mb_status do_sweep(mb_sim *s, int dir, double dt) {
             cudaEventCreate(&e1);
             cudaEventRecord(e0, st);
         }
-        bulk(0);
-        bulk(1);
+        if (packed) {
+            bulk(0);
+            bulk(1);
+        } else {
+            bulk(2);   // every unit in one launch
+        }
         if (s->timing) {
             cudaEventRecord(e1, st);
             s->evs.push_back({e0, e1});
@@ -679,8 +696,10 @@ static mb_status do_sweep(mb_sim *s, int dir, double dt) {
         bool axi = false;
         for (const auto &I : s->hd) axi = axi || I.axisym;
         if (axi) {
-            if (s->prec == MB_FP32) launch_axisym_source<float>(s->dd, s->dy, s->n, s->total_tiles[0], dst, st);
-            else launch_axisym_source<double>(s->dd, s->dy, s->n, s->total_tiles[0], dst, st);
+            size_t cells = 0;
+            for (const auto &I : s->hd) cells = std::max(cells, (size_t)I.pitch * I.ny);
+            if (s->prec == MB_FP32) launch_axisym_source<float>(s->dd, s->dy, s->n, cells, dst, st);
+            else launch_axisym_source<double>(s->dd, s->dy, s->n, cells, dst, st);
         }
     }
     if (s->sidx == 1) {
@@ -1080,10 +1099,7 @@ mb_status mb_merge_count(mb_sim *sim, int inst, long long *cells) {
 static cudaError_t set_yseg(mb_sim *s, int yseg) {
     if (yseg == s->tune_yseg) return cudaSuccess;
     s->tune_yseg = yseg;
-    for (auto &I : s->hd) {
-        I.yseg = yseg;
-        I.ntiles[1] = I.tiles_x[1] * ((I.ny + yseg - 1) / yseg);
-    }
+    for (auto &I : s->hd) bulk_items(s->prec, yseg, I);
     std::vector<int> from(s->n);
     for (int k = 0; k < s->n; ++k) from[k] = k;
     return relayout(s, s->n, from);

@@ -16,7 +16,14 @@
 //   k_finalize    Q = content / alpha at the end pose, class byte update
 #include "mb_internal.cuh"
 
+#include <algorithm>
+#include <type_traits>
+
+#include "mb_fp64.cuh"
+
 namespace mb {
+
+using namespace mbfp;
 
 // ---------------------------------------------------------------------------
 // helpers
@@ -394,6 +401,92 @@ __global__ void k_band_prep_o(const InstDesc *__restrict__ D, InstDyn *__restric
 }
 
 // ---------------------------------------------------------------------------
+// FP64 Euler flow arithmetic of the band faces and the scalar bulk kernels
+// ---------------------------------------------------------------------------
+// a face's side: state, 1/rho and pressure
+struct S64 { double q[4], ir, p; };
+__device__ __forceinline__ double press64(double g1, const double *q, double ir) {
+    const double m2 = __fma_rn(q[1], q[1], q[2] * q[2]);
+    return g1 * __fma_rn(-0.5 * m2, ir, q[3]);
+}
+// MUSCL-Hancock evolved states of one cell (the function evolve above; one
+// reciprocal of the product of two densities serves both sides, and the
+// positivity tests use the pressures the Riemann solver takes)
+template <int D>
+__device__ __forceinline__ void evolve64(double g1, double hl, const double *qm, const double *q0, const double *qp,
+                                         bool lim, S64 &L, S64 &R) {
+    constexpr int in = 1 + D, it = 2 - D;
+    double l[4], r[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const double dm = q0[k] - qm[k], dp = qp[k] - q0[k], pr = dm * dp;
+        double h = 0.0;   // half the van Leer slope
+        if (lim && pos64(pr)) h = pr * rcp64(dm + dp);
+        l[k] = q0[k] - h;
+        r[k] = q0[k] + h;
+    }
+    double rr = rcp64(l[0] * r[0]);
+    const double il = r[0] * rr, ig = l[0] * rr;
+    const double pl = press64(g1, l, il), pg = press64(g1, r, ig);
+    const double ul = l[in] * il, ug = r[in] * ig;
+    double df[4];
+    df[0] = l[in] - r[in];
+    df[in] = __fma_rn(l[in], ul, pl) - __fma_rn(r[in], ug, pg);
+    df[it] = l[it] * ul - r[it] * ug;
+    df[3] = ul * (l[3] + pl) - ug * (r[3] + pg);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        L.q[k] = __fma_rn(hl, df[k], l[k]);
+        R.q[k] = __fma_rn(hl, df[k], r[k]);
+    }
+    rr = rcp64(L.q[0] * R.q[0]);
+    L.ir = R.q[0] * rr;
+    R.ir = L.q[0] * rr;
+    L.p = press64(g1, L.q, L.ir);
+    R.p = press64(g1, R.q, R.ir);
+    if (!(pos64(L.q[0]) && pos64(R.q[0]) && pos64(L.p) && pos64(R.p))) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) L.q[k] = R.q[k] = q0[k];
+        L.ir = R.ir = rcp64(q0[0]);
+        L.p = R.p = press64(g1, q0, L.ir);
+    }
+}
+// HLLC flux (the function hllc above), the star flux in the form
+// [S* (S Q - F) + S p* (0, n, S*)] / (S - S*) with p* = p + rho (S - u)(S* - u)
+// of the side that holds the face (Toro, ch. 10)
+template <int D>
+__device__ __forceinline__ void hllc64(double g, const S64 &L, const S64 &R, double *F) {
+    constexpr int in = 1 + D, it = 2 - D;
+    const double uL = L.q[in] * L.ir, uR = R.q[in] * R.ir;
+    const double cL = sqrt64(g * (L.p * L.ir)), cR = sqrt64(g * (R.p * R.ir));
+    const double SL = min64(uL - cL, uR - cR), SR = max64(uL + cL, uR + cR);
+    const bool supL = nonneg64(SL), supR = !pos64(SR);
+    if (supL || supR) {
+        const S64 &s = supL ? L : R;
+        const double u = supL ? uL : uR;
+        F[0] = s.q[in];
+        F[in] = __fma_rn(s.q[in], u, s.p);
+        F[it] = s.q[it] * u;
+        F[3] = u * (s.q[3] + s.p);
+        return;
+    }
+    const double vL = SL - uL, vR = SR - uR;
+    const double aL = L.q[0] * vL, aR = R.q[0] * vR;
+    const double num = __fma_rn(uL, aL, __fma_rn(-uR, aR, R.p - L.p));
+    const double Ss = num * rcp64(aL - aR);
+    const bool left = nonneg64(Ss);
+    const double S = left ? SL : SR, u = left ? uL : uR, v = left ? vL : vR, a = left ? aL : aR;
+    const double p = left ? L.p : R.p;
+    const double mn = left ? L.q[in] : R.q[in], mt = left ? L.q[it] : R.q[it], E = left ? L.q[3] : R.q[3];
+    const double k = rcp64(S - Ss), kS = k * Ss;
+    const double Sp = S * __fma_rn(a, Ss - u, p);
+    F[0] = a * kS;
+    F[in] = __fma_rn(kS, __fma_rn(mn, v, -p), k * Sp);
+    F[it] = mt * v * kS;
+    F[3] = kS * (__fma_rn(E, v, -(u * p)) + Sp);
+}
+
+// ---------------------------------------------------------------------------
 // stabilised flux of one face: aperture times F2D (eqs. Klein2shieldedFluxMethod2
 // and Klein2DtotalfluxaMethod2 with the one- or two-sided shielded parts).
 // Not inlined, so that a face shared by two band cells gets identical bits.
@@ -410,10 +503,25 @@ __device__ __noinline__ void face_stab(int eq, T g, int dir, T lamT, T av0, T av
                                        const FaceIn *in, double *out) {
     for (int q = 0; q < MAXC; ++q) out[q] = 0.0;
     if (!(w[1].fluid && w[2].fluid && in->btF > 0.0)) return;
-    T QLa[MAXC], QRa[MAXC], QLb[MAXC], QRb[MAXC], F[MAXC];
-    evolve(eq, g, dir, lamT, av0, av1, w[0].q, w[1].q, w[2].q, w[0].fluid && w[2].fluid, QLa, QRa);
-    evolve(eq, g, dir, lamT, av0, av1, w[1].q, w[2].q, w[3].q, w[1].fluid && w[3].fluid, QLb, QRb);
-    riemann_flux(eq, g, dir, av0, av1, QRa, QLb, F);
+    T F[MAXC];
+    const bool limA = w[0].fluid && w[2].fluid, limB = w[1].fluid && w[3].fluid;
+    if (sizeof(T) == 8 && eq == 0) {
+        auto fluxes = [&](auto dc) {
+            constexpr int DC = decltype(dc)::value;
+            S64 x, a, b;
+            const double g1 = (double)g - 1.0, hl = 0.5 * (double)lamT;
+            evolve64<DC>(g1, hl, (const double *)w[0].q, (const double *)w[1].q, (const double *)w[2].q, limA, x, a);
+            evolve64<DC>(g1, hl, (const double *)w[1].q, (const double *)w[2].q, (const double *)w[3].q, limB, b, x);
+            hllc64<DC>((double)g, a, b, (double *)F);
+        };
+        if (dir == 0) fluxes(std::integral_constant<int, 0>());
+        else fluxes(std::integral_constant<int, 1>());
+    } else {
+        T QLa[MAXC], QRa[MAXC], QLb[MAXC], QRb[MAXC];
+        evolve(eq, g, dir, lamT, av0, av1, w[0].q, w[1].q, w[2].q, limA, QLa, QRa);
+        evolve(eq, g, dir, lamT, av0, av1, w[1].q, w[2].q, w[3].q, limB, QLb, QRb);
+        riemann_flux(eq, g, dir, av0, av1, QRa, QLb, F);
+    }
     double bf = in->btF;
     double sR = in->hasR ? fmax(0.0, bf - in->btR) : 0.0;
     double sL = in->hasL ? fmax(0.0, bf - in->btL) : 0.0;
@@ -520,103 +628,11 @@ __global__ void k_band_sweep(const InstDesc *__restrict__ D, InstDyn *__restrict
 // holds (computed once by k_band_sweep), so every face flux is computed once.
 // ---------------------------------------------------------------------------
 
-template <class T, int NC>
-struct QV { T q[NC]; };
-
-template <class T, int NC>
-__device__ __forceinline__ void load_cell(const T *__restrict__ Q, size_t plane, int ci, bool flip, int in,
-                                          QV<T, NC> &v) {
-#pragma unroll
-    for (int k = 0; k < NC; ++k) v.q[k] = __ldg(Q + k * plane + ci);
-    if (NC == 4 && flip) v.q[in] = -v.q[in];
-}
-
-template <class T, int NC>
-__device__ __forceinline__ void shfl_up(QV<T, NC> &o, const QV<T, NC> &v) {
-#pragma unroll
-    for (int k = 0; k < NC; ++k) o.q[k] = __shfl_up_sync(0xffffffffu, v.q[k], 1);
-}
-template <class T, int NC>
-__device__ __forceinline__ void shfl_dn(QV<T, NC> &o, const QV<T, NC> &v) {
-#pragma unroll
-    for (int k = 0; k < NC; ++k) o.q[k] = __shfl_down_sync(0xffffffffu, v.q[k], 1);
-}
-template <class T, int NC>
-__device__ __forceinline__ void shfl_idx(QV<T, NC> &o, const QV<T, NC> &v, int src) {
-#pragma unroll
-    for (int k = 0; k < NC; ++k) o.q[k] = __shfl_sync(0xffffffffu, v.q[k], src);
-}
-
-// face flux between cells (a-1, a) of a line: stabilised record value if a
-// band cell is adjacent, zero next to a solid cell, HLLC otherwise
-template <class T, int NC, int EQ, int DIR>
-__device__ __forceinline__ void face_flux(const InstDesc &I, const BandRec *__restrict__ R, int line, int a, int n,
-                                          uint8_t cl, uint8_t cr, T g, T av0, T av1, const QV<T, NC> &QRl,
-                                          const QV<T, NC> &QLr, QV<T, NC> &F) {
-    if ((cl | cr) & CLS_BAND) {
-        bool fl;
-        const int bclo = I.bc[2 * DIR], bchi = I.bc[2 * DIR + 1];
-        const int pb = ghost_map(a, n, bclo, bchi, &fl), pa = ghost_map(a - 1, n, bclo, bchi, &fl);
-        const int cib = DIR == 0 ? line * I.pitch + pb : pb * I.pitch + line;
-        const int cia = DIR == 0 ? line * I.pitch + pa : pa * I.pitch + line;
-        const bool b_real = a < n || bchi == 2;
-        const bool a_real = a - 1 >= 0 || bclo == 2;
-        if ((cr & CLS_BAND) && (b_real || !a_real || !(cl & CLS_BAND))) {
-            const BandRec &rb = R[I.rec[cib]];
-#pragma unroll
-            for (int k = 0; k < NC; ++k) F.q[k] = (T)rb.Flo[k];
-        } else {
-            const BandRec &ra = R[I.rec[cia]];
-#pragma unroll
-            for (int k = 0; k < NC; ++k) F.q[k] = (T)ra.Fhi[k];
-        }
-        return;
-    }
-    if ((cl | cr) & CLS_SOLID) {
-#pragma unroll
-        for (int k = 0; k < NC; ++k) F.q[k] = T(0);
-        return;
-    }
-    riemann_flux(EQ, g, DIR, av0, av1, QRl.q, QLr.q, F.q);
-}
-
 // a non-band cell whose updated state is not physical: listed for the
 // positivity safeguard (k_mix)
 __device__ __forceinline__ void list_bulk_bad(InstDyn &y, int cell) {
     const int k = atomicAdd(&y.nbulk, 1);
     if (k < NBULK) y.bulkbad[k] = cell;
-}
-
-// new state of a non-band cell; wave speeds and positivity for the CFL step
-template <class T, int NC, int EQ>
-__device__ __forceinline__ void update_cell(T *__restrict__ Qo, size_t plane, int ci, uint8_t c0, T lam, T g, T av0,
-                                            T av1, const QV<T, NC> &q, const QV<T, NC> &Flo, const QV<T, NC> &Fhi,
-                                            bool last, T &s0, T &s1, InstDyn &y) {
-    if (c0 & CLS_BAND) return;
-    if (c0 & CLS_SOLID) {
-#pragma unroll
-        for (int k = 0; k < NC; ++k) Qo[k * plane + ci] = T(NAN);
-        return;
-    }
-    T qn[NC];
-#pragma unroll
-    for (int k = 0; k < NC; ++k) {
-        qn[k] = q.q[k] + lam * (Flo.q[k] - Fhi.q[k]);
-        Qo[k * plane + ci] = qn[k];
-    }
-    if (EQ == 0) {
-        T ir = fdiv(T(1), qn[0]);
-        T p = (g - T(1)) * (qn[NC - 1] - T(0.5) * (qn[1 % NC] * qn[1 % NC] + qn[2 % NC] * qn[2 % NC]) * ir);
-        if (!(qn[0] > T(0)) || !(p > T(0))) list_bulk_bad(y, ci);
-        if (last) {
-            T c = tsqrt(g * p * ir);
-            s0 = fmax(s0, fabs(qn[1 % NC] * ir) + c);
-            s1 = fmax(s1, fabs(qn[2 % NC] * ir) + c);
-        }
-    } else if (last) {
-        s0 = fabs(av0);
-        s1 = fabs(av1);
-    }
 }
 
 template <class T>
@@ -633,6 +649,24 @@ __device__ __forceinline__ void finish_warp(InstDyn &y, bool last, T s0, T s1) {
     }
 }
 
+// (doubles: the maxima of positive values by their bits, off the FP64 pipe; a
+// NaN counts as 0, as in fmax)
+template <>
+__device__ __forceinline__ void finish_warp<double>(InstDyn &y, bool last, double s0, double s1) {
+    if (last) {
+        unsigned long long m0 = pos64(s0) ? (unsigned long long)__double_as_longlong(s0) : 0ull;
+        unsigned long long m1 = pos64(s1) ? (unsigned long long)__double_as_longlong(s1) : 0ull;
+        for (int o = 16; o > 0; o >>= 1) {
+            m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, o));
+            m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, o));
+        }
+        if ((threadIdx.x & 31) == 0) {
+            atomicMax(&y.S[0], m0);
+            atomicMax(&y.S[1], m1);
+        }
+    }
+}
+
 __device__ __forceinline__ int find_inst_warp(const InstDesc *D, int n_inst, int gw, int dir) {
     int lo = 0, hi = n_inst - 1;
     while (lo < hi) {
@@ -642,177 +676,282 @@ __device__ __forceinline__ int find_inst_warp(const InstDesc *D, int n_inst, int
     return lo;
 }
 
-// x sweep: one warp per row, lanes = 32 consecutive cells; the row is
-// processed chunk by chunk, the update trailing the flux computation by one
-// chunk so that the last lane finds its high face in the next chunk
+// Units of the scalar kernels (FP64 Euler, advection in both precisions): 30
+// consecutive cells of a line on the 32 lanes of a warp, lane l holding
+// position a0 - 1 + l, so that a unit evolves 32 cells, forms 31 fluxes and
+// updates 30 cells without looking past its own warp.  The FP64 pipe bounds
+// them (about 150 of its lane operations per cell), so what counts is that
+// every SM has some: one unit per warp spreads a 400 x 400 grid over 5600
+// warps, where a warp per row (x) or per 64 rows (y) left most SMs idle.
+// Measured per sweep, FP64 Euler, before -> after: 399 x 399, x 286 -> 76 us,
+// y 1380 -> 94 us (its two launches together); 9.8 M cells in 16 grids, x
+// 2950 -> 1604 us, y 4090 -> 1617 us, 0.85 of the FP64 pipe's rate for the 88
+// lane operations per cell this flow executes (with the division, square
+// root and comparisons of CUDA: 188 or more).
+constexpr int UNIT_CELLS = 30;
+constexpr int UNIT_COLS = 8;    // columns (lines) per CTA of the y sweep
+
+// the flow arithmetic of a unit by type and equation
 template <class T, int EQ>
-__global__ void __launch_bounds__(256) k_bulk_x(const InstDesc *__restrict__ D, InstDyn *__restrict__ Y,
-                                                const BandRec *__restrict__ R, int n_inst, int total_warps, int src,
-                                                int dst, int last) {
-    constexpr int NC = EQ == 0 ? 4 : 1;
+struct Flow {                     // advection
+    static constexpr int NC = 1;
+    struct S { T q[1]; };
+    T a, lam;
+    __device__ __forceinline__ Flow(const InstDesc &I, T l, int dir) : a((T)I.adv[dir]), lam(l) {}
+    template <int D>
+    __device__ __forceinline__ void states(const T *qm, const T *q0, const T *qp, bool lim, S &L, S &R) const {
+        evolve(1, T(0), D, lam, a, a, qm, q0, qp, lim, L.q, R.q);
+    }
+    template <int D>
+    __device__ __forceinline__ void flux(const S &L, const S &R, T *F) const {
+        F[0] = a > T(0) ? a * L.q[0] : a * R.q[0];
+    }
+};
+template <>
+struct Flow<double, 0> {          // Euler, FP64
+    static constexpr int NC = 4;
+    using S = S64;
+    double g, g1, lam, hl;
+    __device__ __forceinline__ Flow(const InstDesc &I, double l, int)
+        : g(I.gamma), g1(I.gamma - 1.0), lam(l), hl(0.5 * l) {}
+    template <int D>
+    __device__ __forceinline__ void states(const double *qm, const double *q0, const double *qp, bool lim, S &L,
+                                           S &R) const {
+        evolve64<D>(g1, hl, qm, q0, qp, lim, L, R);
+    }
+    template <int D>
+    __device__ __forceinline__ void flux(const S &L, const S &R, double *F) const { hllc64<D>(g, L, R, F); }
+};
+__device__ __forceinline__ void up_state(S64 &s) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s.q[k] = __shfl_up_sync(0xffffffffu, s.q[k], 1);
+    s.ir = __shfl_up_sync(0xffffffffu, s.ir, 1);
+    s.p = __shfl_up_sync(0xffffffffu, s.p, 1);
+}
+template <class S>
+__device__ __forceinline__ void up_state(S &s) { s.q[0] = __shfl_up_sync(0xffffffffu, s.q[0], 1); }
+
+// new state of a lane's cell (qn), with the positivity and wave-speed checks
+// of update_cell
+__device__ __forceinline__ void new_state(const Flow<double, 0> &f, const double *q, const double *Flo,
+                                          const double *Fhi, bool last, int ci, InstDyn &y, double *qn, double &s0,
+                                          double &s1) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) qn[k] = __fma_rn(f.lam, Flo[k] - Fhi[k], q[k]);
+    // p > 0 as 2 rho E > |m|^2; on the step's last sweep from the pressure
+    const double m2 = __fma_rn(qn[1], qn[1], qn[2] * qn[2]);
+    bool ok = pos64(qn[0]);
+    if (last) {
+        const double ir = rcp64(qn[0]), p = f.g1 * __fma_rn(-0.5 * m2, ir, qn[3]);
+        ok = ok && pos64(p);
+        const double c = sqrt64(f.g * (p * ir));
+        s0 = __fma_rn(abs64(qn[1]), ir, c);
+        s1 = __fma_rn(abs64(qn[2]), ir, c);
+    } else {
+        ok = ok && pos64(__fma_rn(twice64(qn[0]), qn[3], neg64(m2)));
+    }
+    if (!ok) list_bulk_bad(y, ci);
+}
+template <class T>
+__device__ __forceinline__ void new_state(const Flow<T, 1> &f, const T *q, const T *Flo, const T *Fhi, bool, int,
+                                          InstDyn &, T *qn, T &, T &) {
+    qn[0] = q[0] + f.lam * (Flo[0] - Fhi[0]);
+}
+
+// One unit: the states qm, q0, qp at this lane's position and its two
+// neighbours (classes cm, c0, cp) become the cell's new state qn; true where
+// the lane stores it (lanes 1 .. 30, positions 0 .. n-1, not a band cell;
+// NaN for a solid cell).  GEN: faces next to a band cell take the record's
+// stabilised flux.
+template <class T, int EQ, int DIR, bool GEN>
+__device__ __forceinline__ bool unit_update(const InstDesc &I, InstDyn &y, const BandRec *__restrict__ R,
+                                            const Flow<T, EQ> &f, int line, int pos, int n, const T *qm, const T *q0,
+                                            const T *qp, int cm, int c0, int cp, bool last, T *qn, T &s0, T &s1) {
+    constexpr int NC = Flow<T, EQ>::NC;
+    const int lane = threadIdx.x & 31;
+    typename Flow<T, EQ>::S L, S;
+    f.template states<DIR>(qm, q0, qp, !((cm | cp) & CLS_SOLID), L, S);
+    up_state(S);   // the right state of the lane below
+    T F[NC], Fhi[NC];
+    if (GEN && ((cm | c0) & CLS_BAND) && pos >= 0 && pos <= n) {
+        bool fl;
+        const int bclo = I.bc[2 * DIR], bchi = I.bc[2 * DIR + 1];
+        const int pb = ghost_map(pos, n, bclo, bchi, &fl), pa = ghost_map(pos - 1, n, bclo, bchi, &fl);
+        const int cib = DIR == 0 ? line * I.pitch + pb : pb * I.pitch + line;
+        const int cia = DIR == 0 ? line * I.pitch + pa : pa * I.pitch + line;
+        const bool b_real = pos < n || bchi == 2, a_real = pos >= 1 || bclo == 2;
+        const bool of_b = (c0 & CLS_BAND) && (b_real || !a_real || !(cm & CLS_BAND));
+        const double *rf = of_b ? R[I.rec[cib]].Flo : R[I.rec[cia]].Fhi;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) F[k] = (T)rf[k];
+    } else if ((cm | c0) & CLS_SOLID) {
+#pragma unroll
+        for (int k = 0; k < NC; ++k) F[k] = T(0);
+    } else {
+        f.template flux<DIR>(S, L, F);
+    }
+#pragma unroll
+    for (int k = 0; k < NC; ++k) Fhi[k] = __shfl_down_sync(0xffffffffu, F[k], 1);
+    if (lane == 0 || lane == 31 || pos >= n || (GEN && (c0 & CLS_BAND))) return false;
+    if (c0 & CLS_SOLID) {
+#pragma unroll
+        for (int k = 0; k < NC; ++k) qn[k] = T(NAN);
+        return true;
+    }
+    const int ci = DIR == 0 ? line * I.pitch + pos : pos * I.pitch + line;
+    new_state(f, q0, F, Fhi, last, ci, y, qn, s0, s1);
+    if (EQ == 1 && last) {
+        s0 = (T)fabs(I.adv[0]);
+        s1 = (T)fabs(I.adv[1]);
+    }
+    return true;
+}
+
+// Units that need no band data: no cell touched at the start pose within
+// three positions along the sweep of any of the unit's cells (as for the
+// deferred cells of the FP32 kernels below), or the whole unit outside the
+// body's extent over the sweep's poses.  They are updated concurrently with
+// the geometry and band fluxes (UNITS_FAR), the others after them
+// (UNITS_NEAR); both launches decide by the same test.  UNITS_ALL: one launch
+// over every unit, after the band fluxes.
+enum { UNITS_FAR = 0, UNITS_NEAR = 1, UNITS_ALL = 2 };
+
+// x sweep: one warp per unit; the three states a lane needs are plain loads
+// (the neighbours' come from L1)
+template <class T, int EQ>
+__global__ void __launch_bounds__(128, 4) k_unit_x(const InstDesc *__restrict__ D, InstDyn *__restrict__ Y,
+                                                   const BandRec *__restrict__ R, int n_inst, int total_units, int src,
+                                                   int dst, int last, int mode) {
+    constexpr int NC = Flow<T, EQ>::NC;
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (gw >= total_warps) return;
+    if (gw >= total_units) return;
     const int inst = find_inst_warp(D, n_inst, gw, 0);
     const InstDesc &I = D[inst];
     InstDyn &y = Y[inst];
-    const int j = gw - I.tile_off[0];
-    const int n = I.nx;
-    const T lam = sizeof(T) == 4 ? (T)y.lamf : (T)y.lam;
-    const T g = (T)I.gamma, av0 = (T)I.adv[0], av1 = (T)I.adv[1];
+    const int local = gw - I.tile_off[0], ncg = I.tiles_x[0];
+    const int j = local / ncg, a0 = (local - j * ncg) * UNIT_CELLS;
+    const int n = I.nx, bclo = I.bc[0], bchi = I.bc[1];
+    const uint8_t *__restrict__ cls = I.cls + (size_t)j * I.pitch;
+    bool fl;
+    if (mode != UNITS_ALL) {
+        bool far = j < y.row0 || j > y.row1 || (bclo != 2 && (a0 + UNIT_CELLS + 2 < y.col0 || a0 - 3 > y.col1));
+        if (!far && !y.defer_all) {
+            int t = cls[ghost_map(a0 - 3 + lane, n, bclo, bchi, &fl)];
+            if (lane < 4) t |= cls[ghost_map(a0 + 29 + lane, n, bclo, bchi, &fl)];
+            far = !__any_sync(0xffffffffu, t & CLS_TOUCH);
+        }
+        if (far != (mode == UNITS_FAR)) return;
+    }
     const size_t plane = (size_t)I.pitch * I.ny;
-    const T *__restrict__ Q = (const T *)I.Q[src];
-    T *__restrict__ Qo = (T *)I.Q[dst];
-    const int rowb = j * I.pitch;
-    const int bclo = I.bc[0], bchi = I.bc[1];
-    auto load = [&](int c, QV<T, NC> &v, uint8_t &cl) {
-        const int a = 32 * c + lane;
-        if (a < -2 || a > n + 1) {
+    const int pos = a0 - 1 + lane;
+    const T *__restrict__ Q = (const T *)I.Q[src] + (size_t)j * I.pitch;
+    T qm[NC], q0[NC], qp[NC], qn[NC];
+    int cm, c0, cp;
+    auto load = [&](int a, T *q, int &c) {
+        bool flip;
+        const int p = ghost_map(a, n, bclo, bchi, &flip);
+        c = cls[p];
 #pragma unroll
-            for (int k = 0; k < NC; ++k) v.q[k] = T(1);
-            cl = CLS_SOLID;
-            return;
-        }
-        bool fl;
-        const int p = ghost_map(a, n, bclo, bchi, &fl);
-        cl = I.cls[rowb + p];
-        load_cell<T, NC>(Q, plane, rowb + p, fl, 1, v);
+        for (int k = 0; k < NC; ++k) q[k] = __ldg(Q + k * plane + p);
+        if (NC == 4 && flip) q[1] = -q[1];
     };
-    const int c_last = (n + 1) >> 5;
-    QV<T, NC> Qm, Q0, Qp, QL, QR, F, Fprev, nb, nb2;
-    uint8_t cm, c0, cp;
-    load(-1, Qm, cm);
-    load(0, Q0, c0);
-    load(1, Qp, cp);
-    // evolved right state of cell -1 (lane 31 of chunk -1)
-    {
-        shfl_up(nb, Qm);
-        shfl_dn(nb2, Qm);
-        QV<T, NC> t;
-        shfl_idx(t, Q0, 0);
-        if (lane == 31) nb2 = t;
-        const int cmu = __shfl_up_sync(0xffffffffu, (int)cm, 1);
-        int cmd = __shfl_down_sync(0xffffffffu, (int)cm, 1);
-        const int c00 = __shfl_sync(0xffffffffu, (int)c0, 0);
-        if (lane == 31) cmd = c00;
-        const bool lim = !(cmu & CLS_SOLID) && !(cmd & CLS_SOLID);
-        evolve(EQ, g, 0, lam, av0, av1, nb.q, Qm.q, nb2.q, lim, QL.q, QR.q);
-    }
-    QV<T, NC> QRc;
-    shfl_idx(QRc, QR, 31);
-    int cRc = __shfl_sync(0xffffffffu, (int)cm, 31);
+    load(pos - 1, qm, cm);
+    load(pos, q0, c0);
+    load(pos + 1, qp, cp);
+    const Flow<T, EQ> f(I, sizeof(T) == 4 ? (T)y.lamf : (T)y.lam, 0);
     T s0 = T(0), s1 = T(0);
-    for (int c = 0; c <= c_last; ++c) {
-        // neighbours of chunk c
-        QV<T, NC> left, right, t;
-        shfl_up(left, Q0);
-        shfl_idx(t, Qm, 31);
-        if (lane == 0) left = t;
-        shfl_dn(right, Q0);
-        shfl_idx(t, Qp, 0);
-        if (lane == 31) right = t;
-        int cl_ = __shfl_up_sync(0xffffffffu, (int)c0, 1);
-        int cm31 = __shfl_sync(0xffffffffu, (int)cm, 31);
-        if (lane == 0) cl_ = cm31;
-        int cr_ = __shfl_down_sync(0xffffffffu, (int)c0, 1);
-        int cp0 = __shfl_sync(0xffffffffu, (int)cp, 0);
-        if (lane == 31) cr_ = cp0;
-        const bool lim = !(cl_ & CLS_SOLID) && !(cr_ & CLS_SOLID);
-        evolve(EQ, g, 0, lam, av0, av1, left.q, Q0.q, right.q, lim, QL.q, QR.q);
-        // face between cells a-1 and a
-        QV<T, NC> QRl;
-        shfl_up(QRl, QR);
-        if (lane == 0) QRl = QRc;
-        const int a = 32 * c + lane;
-        if (a >= 0 && a <= n) face_flux<T, NC, EQ, 0>(I, R, j, a, n, (uint8_t)cl_, c0, g, av0, av1, QRl, QL, F);
-        // update chunk c-1
-        if (c >= 1) {
-            QV<T, NC> Fhi;
-            shfl_dn(Fhi, Fprev);
-            shfl_idx(t, F, 0);
-            if (lane == 31) Fhi = t;
-            const int ap = a - 32;
-            if (ap >= 0 && ap < n)
-                update_cell<T, NC, EQ>(Qo, plane, rowb + ap, cm, lam, g, av0, av1, Qm, Fprev, Fhi, last, s0, s1, y);
-        }
-        shfl_idx(QRc, QR, 31);
-        Fprev = F;
-        Qm = Q0; cm = c0;
-        Q0 = Qp; c0 = cp;
-        load(c + 2, Qp, cp);
+    const bool st = mode == UNITS_FAR
+        ? unit_update<T, EQ, 0, false>(I, y, R, f, j, pos, n, qm, q0, qp, cm, c0, cp, last != 0, qn, s0, s1)
+        : unit_update<T, EQ, 0, true>(I, y, R, f, j, pos, n, qm, q0, qp, cm, c0, cp, last != 0, qn, s0, s1);
+    if (st) {
+        T *__restrict__ Qo = (T *)I.Q[dst] + (size_t)j * I.pitch + pos;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) Qo[k * plane] = qn[k];
     }
-    // the last chunk (its high faces were computed in the final iteration)
-    {
-        QV<T, NC> Fhi;
-        shfl_dn(Fhi, Fprev);
-        const int ap = 32 * c_last + lane;
-        if (ap >= 0 && ap < n && lane < 31)
-            update_cell<T, NC, EQ>(Qo, plane, rowb + ap, cm, lam, g, av0, av1, Qm, Fprev, Fhi, last, s0, s1, y);
-    }
-    (void)cRc;
     finish_warp<T>(y, last != 0, s0, s1);
 }
 
-// y sweep: one thread per column and segment of I.yseg rows, marching upward
-// with a register window; 32 consecutive columns per warp keep every load
-// and store coalesced
+// y sweep: one CTA per 8 columns and 30 rows, a warp per column with its
+// lanes along the rows; the CTA's 34 x 8 states pass through shared memory
+// both ways, so that global loads and stores are 8 consecutive columns
 template <class T, int EQ>
-__global__ void __launch_bounds__(256, 3) k_bulk_y(const InstDesc *__restrict__ D, InstDyn *__restrict__ Y,
-                                                const BandRec *__restrict__ R, int n_inst, int total_warps, int src,
-                                                int dst, int last) {
-    constexpr int NC = EQ == 0 ? 4 : 1;
-    const int lane = threadIdx.x & 31;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (gw >= total_warps) return;
-    const int inst = find_inst_warp(D, n_inst, gw, 1);
+__global__ void __launch_bounds__(256, 2) k_unit_y(const InstDesc *__restrict__ D, InstDyn *__restrict__ Y,
+                                                   const BandRec *__restrict__ R, int n_inst, int src, int dst,
+                                                   int last, int mode) {
+    constexpr int NC = Flow<T, EQ>::NC;
+    constexpr int ROWS = UNIT_CELLS + 4, LD = UNIT_COLS + 1;
+    __shared__ T sq[NC][ROWS][LD];
+    __shared__ uint8_t sc[ROWS][LD];
+    __shared__ uint8_t sst[UNIT_CELLS][LD];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int inst = find_inst_warp(D, n_inst, blockIdx.x, 1);
     const InstDesc &I = D[inst];
     InstDyn &y = Y[inst];
-    const int local = gw - I.tile_off[1];
-    const int ncg = I.tiles_x[1];
-    const int cg = local % ncg, sg = local / ncg;
-    const int i_raw = cg * 32 + lane;
-    const bool active = i_raw < I.nx;
-    const int i = active ? i_raw : I.nx - 1;
-    const int n = I.ny;
-    const int j0 = sg * I.yseg, j1 = min(n, j0 + I.yseg);
-    const T lam = sizeof(T) == 4 ? (T)y.lamf : (T)y.lam;
-    const T g = (T)I.gamma, av0 = (T)I.adv[0], av1 = (T)I.adv[1];
-    const size_t plane = (size_t)I.pitch * I.ny;
-    const T *__restrict__ Q = (const T *)I.Q[src];
-    T *__restrict__ Qo = (T *)I.Q[dst];
-    const int bclo = I.bc[2], bchi = I.bc[3];
-    auto load = [&](int r, QV<T, NC> &v, uint8_t &cl) {
-        bool fl;
-        const int p = ghost_map(r, n, bclo, bchi, &fl);
-        const int ci = p * I.pitch + i;
-        cl = I.cls[ci];
-        load_cell<T, NC>(Q, plane, ci, fl, 2, v);
-    };
-    QV<T, NC> qa, qm, qc, qp, qq, QL, QR, QRc, F, Fprev;
-    uint8_t ca, cm, cc, cp, cq;
-    load(j0 - 2, qa, ca);
-    load(j0 - 1, qm, cm);
-    load(j0, qc, cc);
-    load(j0 + 1, qp, cp);
-    load(j0 + 2, qq, cq);
-    // evolved top state of row j0-1
-    evolve(EQ, g, 1, lam, av0, av1, qa.q, qm.q, qc.q, !(ca & CLS_SOLID) && !(cc & CLS_SOLID), QL.q, QRc.q);
-    T s0 = T(0), s1 = T(0);
-    for (int f = j0; f <= j1; ++f) {
-        // window: qm = row f-1, qc = row f, qp = row f+1, qq = row f+2
-        evolve(EQ, g, 1, lam, av0, av1, qm.q, qc.q, qp.q, !(cm & CLS_SOLID) && !(cp & CLS_SOLID), QL.q, QR.q);
-        face_flux<T, NC, EQ, 1>(I, R, i, f, n, cm, cc, g, av0, av1, QRc, QL, F);
-        if (f > j0 && active)
-            update_cell<T, NC, EQ>(Qo, plane, (f - 1) * I.pitch + i, cm, lam, g, av0, av1, qm, Fprev, F, last, s0,
-                                   s1, y);
-        QRc = QR;
-        Fprev = F;
-        qm = qc; cm = cc;
-        qc = qp; cc = cp;
-        qp = qq; cp = cq;
-        if (f + 3 <= j1 + 1) load(f + 3, qq, cq);
+    const int local = blockIdx.x - I.tile_off[1], ncg = I.tiles_x[1];
+    const int sg = local / ncg, i0 = (local - sg * ncg) * UNIT_COLS, j0 = sg * UNIT_CELLS;
+    const int n = I.ny, bclo = I.bc[2], bchi = I.bc[3];
+    bool fl;
+    if (mode != UNITS_ALL) {
+        bool far = i0 + UNIT_COLS - 1 < y.col0 || i0 > y.col1 ||
+                   (bclo != 2 && (j0 + UNIT_CELLS + 2 < y.row0 || j0 - 3 > y.row1));
+        if (!far && !y.defer_all) {
+            int t = 0;
+            for (int e = threadIdx.x; e < (UNIT_CELLS + 6) * UNIT_COLS; e += 256) {
+                const int i = i0 + (e & (UNIT_COLS - 1));
+                if (i < I.nx) t |= I.cls[ghost_map(j0 - 3 + (e >> 3), n, bclo, bchi, &fl) * I.pitch + i];
+            }
+            far = !__syncthreads_or(t & CLS_TOUCH);
+        }
+        if (far != (mode == UNITS_FAR)) return;
     }
+    const size_t plane = (size_t)I.pitch * n;
+    const T *__restrict__ Q = (const T *)I.Q[src];
+    for (int e = threadIdx.x; e < ROWS * UNIT_COLS; e += 256) {
+        const int r = e >> 3, c = e & (UNIT_COLS - 1);
+        bool flip;
+        const int ci = ghost_map(j0 - 2 + r, n, bclo, bchi, &flip) * I.pitch + min(i0 + c, I.nx - 1);
+        sc[r][c] = I.cls[ci];
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            const T v = __ldg(Q + k * plane + ci);
+            sq[k][r][c] = NC == 4 && k == 2 && flip ? -v : v;
+        }
+    }
+    __syncthreads();
+    const int i = i0 + w, pos = j0 - 1 + lane;
+    T s0 = T(0), s1 = T(0);
+    T qm[NC], q0[NC], qp[NC], qn[NC];
+    bool st = false;
+    if (i < I.nx) {   // whole warps
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            qm[k] = sq[k][lane][w];
+            q0[k] = sq[k][lane + 1][w];
+            qp[k] = sq[k][lane + 2][w];
+        }
+        const int cm = sc[lane][w], c0 = sc[lane + 1][w], cp = sc[lane + 2][w];
+        const Flow<T, EQ> f(I, sizeof(T) == 4 ? (T)y.lamf : (T)y.lam, 1);
+        st = mode == UNITS_FAR
+            ? unit_update<T, EQ, 1, false>(I, y, R, f, i, pos, n, qm, q0, qp, cm, c0, cp, last != 0, qn, s0, s1)
+            : unit_update<T, EQ, 1, true>(I, y, R, f, i, pos, n, qm, q0, qp, cm, c0, cp, last != 0, qn, s0, s1);
+        __syncwarp();
+        if (st) {   // a warp's column is its own
+#pragma unroll
+            for (int k = 0; k < NC; ++k) sq[k][lane + 1][w] = qn[k];
+        }
+    }
+    if (lane >= 1 && lane <= UNIT_CELLS) sst[lane - 1][w] = st;
     finish_warp<T>(y, last != 0, s0, s1);
+    __syncthreads();
+    T *__restrict__ Qo = (T *)I.Q[dst];
+    for (int e = threadIdx.x; e < UNIT_CELLS * UNIT_COLS; e += 256) {
+        const int r = e >> 3, c = e & (UNIT_COLS - 1);
+        if (!sst[r][c]) continue;
+        const size_t ci = (size_t)(j0 + r) * I.pitch + i0 + c;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) Qo[k * plane + ci] = sq[k][r + 2][c];
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1938,28 +2077,28 @@ __global__ void __launch_bounds__(128, MINB) k_bulk_y_p(const InstDesc *__restri
 // Geometric source of the axisymmetric Euler equations after a y sweep (a
 // reading; Sec. III.E models its open-ended tube in axisymmetric form): with
 // x axial and y the radius from the axis y = y0 = 0, every fluid cell gets
-// Q -= dt (v / r) [rho, rho u, rho v, E + p], r at the cell centre.  One warp
-// per grid row; instances of the batch without the flag return at once.  In
+// Q -= dt (v / r) [rho, rho u, rho v, E + p], r at the cell centre.  One thread
+// per cell (grid: x over the largest instance's cells, y over the instances);
+// instances of the batch without the flag return at once.  In
 // FP64 every operation is rounded on its own (no contraction), in the order
 // of the plain definition.
 // ---------------------------------------------------------------------------
 template <class T>
 __global__ void __launch_bounds__(256) k_axisym_source(const InstDesc *__restrict__ D, InstDyn *__restrict__ Y,
-                                                       int n_inst, int total_warps, int buf) {
-    const int lane = threadIdx.x & 31;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (gw >= total_warps) return;
-    const int inst = find_inst_warp(D, n_inst, gw, 0);
+                                                       int buf) {
+    const int inst = blockIdx.y;
     const InstDesc &I = D[inst];
     if (!I.axisym || I.eq != 0) return;
     InstDyn &y = Y[inst];
-    const int j = gw - I.tile_off[0];
     const size_t plane = (size_t)I.pitch * I.ny;
-    T *__restrict__ Q = (T *)I.Q[buf] + (size_t)j * I.pitch;
-    const double r = __dmul_rn(__dadd_rn((double)j, 0.5), I.dy);
     const double dt = y.dt;
     bool bad = false;
-    for (int i = lane; i < I.nx; i += 32) {
+    // a warp's 32 positions lie in one row (the pitch is a multiple of 32)
+    for (size_t c = (size_t)blockIdx.x * 256 + threadIdx.x; c < plane; c += (size_t)gridDim.x * 256) {
+        const int j = (int)(c / I.pitch), i = (int)(c - (size_t)j * I.pitch);
+        if (i >= I.nx) continue;
+        const double r = __dmul_rn(__dadd_rn((double)j, 0.5), I.dy);
+        T *__restrict__ Q = (T *)I.Q[buf] + (size_t)j * I.pitch;
         const T q0 = Q[i], q1 = Q[plane + i], q2 = Q[2 * plane + i], q3 = Q[3 * plane + i];
         if (!(q0 == q0)) continue;   // solid
         T n0, n1, n2, n3, pn;
@@ -1990,12 +2129,13 @@ __global__ void __launch_bounds__(256) k_axisym_source(const InstDesc *__restric
         Q[3 * plane + i] = n3;
         if (!(n0 > (T)0) || !(pn > (T)0)) bad = true;
     }
-    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&y.err, ERR_UNSTABLE);
+    if (bad) atomicOr(&y.err, ERR_UNSTABLE);
 }
 
 template <class T>
-void launch_axisym_source(const InstDesc *D, InstDyn *Y, int n_inst, int total_rows, int buf, cudaStream_t st) {
-    if (total_rows > 0) k_axisym_source<T><<<(total_rows + 7) / 8, 256, 0, st>>>(D, Y, n_inst, total_rows, buf);
+void launch_axisym_source(const InstDesc *D, InstDyn *Y, int n_inst, size_t max_cells, int buf, cudaStream_t st) {
+    const unsigned bx = (unsigned)std::min<size_t>((max_cells + 255) / 256, 1u << 20);
+    if (bx > 0 && n_inst > 0) k_axisym_source<T><<<dim3(bx, n_inst), 256, 0, st>>>(D, Y, buf);
 }
 
 // ---------------------------------------------------------------------------
@@ -2280,12 +2420,6 @@ __global__ void __launch_bounds__(128, 5) k_bulk_def_y(const InstDesc *__restric
         }
         if (last) def_wave_speeds(Y, inst, st != 0, s0, s1);
     }
-}
-
-template <class T, int EQ>
-void bulk_attr_t(int dir) {
-    if (dir == 0) cudaFuncSetAttribute(k_bulk_x<T, EQ>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
-    else cudaFuncSetAttribute(k_bulk_y<T, EQ>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
 }
 
 // ---------------------------------------------------------------------------
@@ -2857,25 +2991,42 @@ void launch_band_stage(int stage, const InstDesc *D, InstDyn *Y, BandRec *R, con
     }
 }
 
+// the scalar kernels over total units (x: warps, y: CTAs), in the mode
+// UNITS_*
+template <class T>
+void launch_units(int dir, int eq, const InstDesc *D, InstDyn *Y, const BandRec *R, int n_inst, int total, int src,
+                  int dst, int last, int mode, cudaStream_t st) {
+    const unsigned bx = (unsigned)((total + 3) / 4);
+    if (eq == 1) {
+        if (dir == 0) k_unit_x<T, 1><<<bx, 128, 0, st>>>(D, Y, R, n_inst, total, src, dst, last, mode);
+        else k_unit_y<T, 1><<<total, 256, 0, st>>>(D, Y, R, n_inst, src, dst, last, mode);
+    } else if constexpr (sizeof(T) == 8) {
+        if (dir == 0) k_unit_x<T, 0><<<bx, 128, 0, st>>>(D, Y, R, n_inst, total, src, dst, last, mode);
+        else k_unit_y<T, 0><<<total, 256, 0, st>>>(D, Y, R, n_inst, src, dst, last, mode);
+    }
+}
+
 // bulk passes of one sweep.  FP32 Euler (the FP32x2 kernels): mode 0 is the
 // pass over the cells that need no band data (it lists the deferred cell
 // pairs in dl), mode 1 the deferred pairs and, when any instance may have
-// defer_all (any_defer_all), the streaming pass over those instances.  Other
-// kernels: one pass, launched for mode 0 only.
+// defer_all (any_defer_all), the streaming pass over those instances.  The
+// scalar kernels: mode is UNITS_*.
 template <class T>
 void launch_bulk(int dir, int eq, const InstDesc *D, InstDyn *Y, const BandRec *R, int n_inst, int total_warps,
                  int src, int dst, int last, int shape, int mode, DeferList dl, int any_defer_all, cudaStream_t st) {
     const int cta = shape & 1023;
     const int wpc = cta / 32;   // warps per CTA of the FP32x2 kernels
-    int blocks = (total_warps + 7) / 8;
-    if (blocks <= 0) return;
+    if (total_warps <= 0) return;
     const bool packed = sizeof(T) == 4 && eq == 0;   // FP32 Euler: the FP32x2 kernels
-    if (!packed && mode != 0) return;
+    if (!packed) {
+        launch_units<T>(dir, eq, D, Y, R, n_inst, total_warps, src, dst, last, mode, st);
+        return;
+    }
     const int pg = (total_warps + wpc - 1) / wpc;
     const bool m4 = (shape & SHAPE_MINB4) != 0, r8 = (shape & SHAPE_RING8) != 0;
     constexpr int DEF_BLOCKS = 760;   // 5 resident CTAs of 128 threads per SM, grid-stride over the list
     if (dir == 0) {
-        if (packed) {
+        {
             const size_t sm = wpc * (r8 ? sizeof(XRing<8>) : sizeof(XRing<4>));
             if (mode == 1) {
                 k_bulk_def_x<<<DEF_BLOCKS, 128, 0, st>>>(D, Y, R, src, dst, last, dl);
@@ -2885,10 +3036,9 @@ void launch_bulk(int dir, int eq, const InstDesc *D, InstDyn *Y, const BandRec *
             else if (m4) k_bulk_x_p<4, 4, 0><<<pg, cta, sm, st>>>(D, Y, R, n_inst, total_warps, src, dst, last, dl);
             else if (r8) k_bulk_x_p<5, 8, 0><<<pg, cta, sm, st>>>(D, Y, R, n_inst, total_warps, src, dst, last, dl);
             else k_bulk_x_p<5, 4, 0><<<pg, cta, sm, st>>>(D, Y, R, n_inst, total_warps, src, dst, last, dl);
-        } else if (eq == 0) k_bulk_x<T, 0><<<blocks, 256, 0, st>>>(D, Y, R, n_inst, total_warps, src, dst, last);
-        else k_bulk_x<T, 1><<<blocks, 256, 0, st>>>(D, Y, R, n_inst, total_warps, src, dst, last);
+        }
     } else {
-        if (packed) {
+        {
             const size_t sm = wpc * sizeof(YRing);
             if (mode == 1) {
                 k_bulk_def_y<<<DEF_BLOCKS, 128, 0, st>>>(D, Y, R, src, dst, last, dl);
@@ -2896,16 +3046,13 @@ void launch_bulk(int dir, int eq, const InstDesc *D, InstDyn *Y, const BandRec *
                     k_bulk_y_p<4, 1><<<pg, cta, sm, st>>>(D, Y, R, n_inst, total_warps, src, dst, last, dl);
             } else if (m4) k_bulk_y_p<4, 0><<<pg, cta, sm, st>>>(D, Y, R, n_inst, total_warps, src, dst, last, dl);
             else k_bulk_y_p<5, 0><<<pg, cta, sm, st>>>(D, Y, R, n_inst, total_warps, src, dst, last, dl);
-        } else if (eq == 0) k_bulk_y<T, 0><<<blocks, 256, 0, st>>>(D, Y, R, n_inst, total_warps, src, dst, last);
-        else k_bulk_y<T, 1><<<blocks, 256, 0, st>>>(D, Y, R, n_inst, total_warps, src, dst, last);
+        }
     }
 }
 
 template <class T>
 int bulk_blocks_per_sm(int dir) {
     cudaFuncSetAttribute(k_mix<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, MIX_SMEM);
-    bulk_attr_t<T, 0>(dir);
-    bulk_attr_t<T, 1>(dir);
     if (sizeof(T) == 4) {   // the FP32x2 kernels' shared-memory rings (4 warps per CTA at most)
         if (dir == 0) {
             const int s4 = (int)(4 * sizeof(XRing<4>)), s8 = (int)(4 * sizeof(XRing<8>));
@@ -2945,7 +3092,7 @@ void launch_read_state(const InstDesc *D, H *const *ptrs, H *p1, int inst0, int 
     template void launch_bulk<T>(int, int, const InstDesc *, InstDyn *, const BandRec *, int, int, int, int, int,  \
                                  int, int, DeferList, int, cudaStream_t);                                               \
     template int bulk_blocks_per_sm<T>(int);                                                                       \
-    template void launch_axisym_source<T>(const InstDesc *, InstDyn *, int, int, int, cudaStream_t);               \
+    template void launch_axisym_source<T>(const InstDesc *, InstDyn *, int, size_t, int, cudaStream_t);            \
     template void launch_write_state<T, double>(const InstDesc *, InstDyn *, const double *const *, const double *, \
                                                 int, int, int, int, cudaStream_t);                                 \
     template void launch_write_state<T, float>(const InstDesc *, InstDyn *, const float *const *, const float *,    \
