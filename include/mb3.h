@@ -84,12 +84,14 @@ mb_status mb3_last_sweep(mb3_sim *sim, double *wall, int *merged);
  * beside it).  Geometry, wall states and shielded fluxes, the update of the
  * contents, covering and uncovering, the safeguard and the state stay FP64,
  * and fluxes are stored in FP64, so the update stays conservative to FP64
- * rounding.  Allocates the copy (4 bytes x 5 per cell) on first use;
+ * rounding.  Allocates two copies (4 bytes x 5 per cell each: a sweep's old
+ * and new state) on first use;
  * MB_E_STATE in the middle of a step, MB_E_INVAL for another value. */
 mb_status mb3_set_precision(mb3_sim *sim, int precision);
-/* device time (ms) of the last sweep's face-flux kernel (MUSCL-Hancock +
- * HLLC + stabilised flux of every face along the sweep), from CUDA events
- * recorded around it on the simulation's stream */
+/* device time (ms) of the last sweep's flow kernels (MUSCL-Hancock + HLLC +
+ * stabilised flux of every face along the sweep, and the content update),
+ * from CUDA events recorded around their launches on the simulation's stream
+ * (the geometry kernels run beside the first) */
 mb_status mb3_flux_time(mb3_sim *sim, double *ms);
 
 #ifdef __cplusplus

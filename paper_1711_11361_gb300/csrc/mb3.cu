@@ -9,12 +9,13 @@
 //             apertures of the sweep's faces (R)
 //   k3_wall   flux-GCL provisional states, shielded distance, wall normal,
 //             wall state and flux of the band cells (R)
-//   k3_evolve MUSCL-Hancock evolved boundary states of every cell along d
-//   k3_flux   HLLC + stabilised flux of every d-face
-//   k3_update the conservative update alpha_B Q' of every cell
+//   k3_row, k3_march  MUSCL-Hancock states, HLLC + stabilised fluxes and the
+//             conservative update alpha_B Q' of every cell: the cells away
+//             from R beside the geometry, the others after k3_wall
 //   k3_events covering / uncovering, gathered per cell in cell order (R)
 //   k3_bad / k3_mix  the positivity safeguard (one block merges in shared memory)
-//   k3_final  Q = content / alpha_B, solid cells NaN, error checks
+//   k3_final  Q = content / alpha_B in R, solid cells NaN, error checks
+//             (elsewhere the content is the state)
 // Geometry: the volume of a box inside the body by the divergence theorem
 // over the faces of box ∩ body, each face the plane's polygon clipped by all
 // other half-spaces in its own plane; apertures by clipping the face
@@ -30,8 +31,11 @@
 #include <vector>
 
 #include "mb3.h"
+#include "mb_fp64.cuh"
 
 namespace mb3 {
+
+using namespace mbfp;
 
 constexpr int NC = 5;
 constexpr int MAXP = MB3_MAX_PLANES;
@@ -237,10 +241,11 @@ struct Desc {
     int d;                  // the sweep's direction
     double lam;             // dt / h_d
     int r0[3], rn[3];       // region R: first cell and extent per axis
-    double *Q, *Qn, *C, *Cn, *F;
-    double *E;              // evolved boundary states along d, 2 NC planes
-    int f32;                // FP32 flux option: Qf, and E read as floats
-    float *Qf;              // the state in FP32 (FP32 flux option)
+    double *Q, *Qn;         // the state at the sweep's and at the step's start
+    double *C;              // contents before the events (R; alpha on its way out of mb3_read_state)
+    double *Cn;             // new contents, then the new state
+    int f32;                // FP32 flux option
+    float *Qf, *Qfn;        // Q and the new state in FP32 (FP32 flux option)
     float gammaf, hlamf;    // gamma and lam / 2 in FP32 (no conversion per thread)
     double *aA, *aM, *aB;   // over R
     unsigned char *tA, *tB; // over R
@@ -254,7 +259,7 @@ struct Desc {
     unsigned char *evt;     // event type over R: 0 none, 1 covered, 2 uncovered donor, 3 covered, leaves
     unsigned *emask;        // recipients / donors (bit (dk+1)*9 + (dj+1)*3 + (di+1))
     double *easum;
-    unsigned char *upd;
+    unsigned char *upd;     // over R: the cell has a new content (elsewhere every cell has)
     int *err;
     double *wall;           // 5 summed wall terms
     int *seeds, *nseed;
@@ -293,6 +298,9 @@ __device__ __forceinline__ double alphaA(const Desc &D, int i, int j, int k) {
 __device__ __forceinline__ double alphaB(const Desc &D, int i, int j, int k) {
     return in_r(D, i, j, k) ? D.aB[ridx(D, i, j, k)] : 1.0;
 }
+__device__ __forceinline__ bool updated(const Desc &D, int i, int j, int k) {
+    return !in_r(D, i, j, k) || D.upd[ridx(D, i, j, k)];
+}
 __device__ __forceinline__ double swept(const Desc &D, int i, int j, int k) {
     return in_rf(D, D.d, i, j, k) ? D.bt[rfidx(D, D.d, i, j, k)] : 1.0;
 }
@@ -330,6 +338,9 @@ __device__ __forceinline__ double widen(double x) { return x; }
 __device__ __forceinline__ double node(const Desc &D, int a, int i) { return D.lo[a] + (double)i * D.h[a]; }
 // x is neither infinite nor NaN: its exponent field is not all ones (an
 // integer test, off GB300's narrow FP64 pipe)
+__device__ __forceinline__ bool isnan64(double x) {
+    return ((unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull) > 0x7ff0000000000000ull;
+}
 __device__ __forceinline__ bool finite64(double x) {
     return (__double_as_longlong(x) & 0x7ff0000000000000LL) != 0x7ff0000000000000LL;
 }
@@ -573,294 +584,472 @@ __global__ void k3_wall(Desc D) {
 __device__ __forceinline__ double pressure5(double g, const double *q) {
     return (g - 1.0) * (q[4] - 0.5 * (q[1] * q[1] + q[2] * q[2] + q[3] * q[3]) / q[0]);
 }
-// (GB300's FP64 pipe is narrow: each quotient costs a Newton sequence, so
-// the kernels share one reciprocal of rho where they can.  The flow
-// arithmetic below takes its type T as a template argument: double for the
-// FP64 path, float for the FP32 flux option; every literal is a T, so the
-// float instances stay in float and the double ones are the FP64 path's
-// arithmetic unchanged)
-// a b + c with one rounding (the file is built without contraction, so
-// the flow arithmetic fuses where it says so)
-__device__ __forceinline__ double fmad(double a, double b, double c) { return __fma_rn(a, b, c); }
+// The line kernels' flow arithmetic in the type T: double for the FP64 path
+// (mb_fp64.cuh), float for the FP32 flux option (below; the file is built
+// without contraction, so it fuses where it says so).
 __device__ __forceinline__ float fmad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-template <typename T> __device__ __forceinline__ T sq3(const T *m) { return fmad(m[0], m[0], fmad(m[1], m[1], m[2] * m[2])); }
+__device__ __forceinline__ float sq3(const float *m) { return fmad(m[0], m[0], fmad(m[1], m[1], m[2] * m[2])); }
 // the physical flux along d of a state with 1/rho given
-template <typename T>
-__device__ __forceinline__ void flux5(T g, int d, const T *q, T ir, T *f) {
-    const T rho = q[0], un = q[1 + d] * ir;
-    const T p = (g - T(1)) * fmad(T(-0.5) * sq3(q + 1), ir, q[4]);
+template <int d>
+__device__ __forceinline__ void flux5(float g, const float *q, float ir, float *f) {
+    const float rho = q[0], un = q[1 + d] * ir;
+    const float p = (g - 1.0f) * fmad(-0.5f * sq3(q + 1), ir, q[4]);
     f[0] = rho * un;
     for (int m = 0; m < 3; ++m) f[1 + m] = m == d ? fmad(q[1 + m], un, p) : q[1 + m] * un;
     f[4] = un * (q[4] + p);
 }
 // HLLC, Davis wave speeds (Toro, Riemann Solvers ch. 10)
-template <typename T>
-__device__ __forceinline__ void hllc5(T g, int d, const T *qL, const T *qR, T *F) {
-    const int in = 1 + d;
+template <int d>
+__device__ __forceinline__ void hllc5(float g, const float *qL, const float *qR, float *F) {
+    constexpr int in = 1 + d;
     // 1/rho of both states from one reciprocal of their product
-    const T rL = qL[0], rR = qR[0], rr2 = T(1) / (rL * rR), iL = rR * rr2, iR = rL * rr2;
-    const T uL = qL[in] * iL, uR = qR[in] * iR;
-    const T pL = (g - T(1)) * fmad(T(-0.5) * sq3(qL + 1), iL, qL[4]);
-    const T pR = (g - T(1)) * fmad(T(-0.5) * sq3(qR + 1), iR, qR[4]);
-    const T cL = sqrt(g * pL * iL), cR = sqrt(g * pR * iR);
-    const T SL = fmin(uL - cL, uR - cR), SR = fmax(uL + cL, uR + cR);
-    if (SL >= T(0)) { flux5(g, d, qL, iL, F); return; }
-    if (SR <= T(0)) { flux5(g, d, qR, iR, F); return; }
-    const T num = fmad(-(rR * uR), SR - uR, fmad(rL * uL, SL - uL, pR - pL));
-    const T den = fmad(rL, SL - uL, -(rR * (SR - uR)));
-    const T Ss = num / den;
-    const bool left = Ss >= T(0);
-    const T *q = left ? qL : qR;
-    const T r = left ? rL : rR, ir = left ? iL : iR, u = left ? uL : uR, p = left ? pL : pR;
-    const T S = left ? SL : SR;
-    T f[NC], qs[NC];
+    const float rL = qL[0], rR = qR[0], rr2 = 1.0f / (rL * rR), iL = rR * rr2, iR = rL * rr2;
+    const float uL = qL[in] * iL, uR = qR[in] * iR;
+    const float pL = (g - 1.0f) * fmad(-0.5f * sq3(qL + 1), iL, qL[4]);
+    const float pR = (g - 1.0f) * fmad(-0.5f * sq3(qR + 1), iR, qR[4]);
+    const float cL = sqrtf(g * pL * iL), cR = sqrtf(g * pR * iR);
+    const float SL = fminf(uL - cL, uR - cR), SR = fmaxf(uL + cL, uR + cR);
+    if (SL >= 0.0f) { flux5<d>(g, qL, iL, F); return; }
+    if (SR <= 0.0f) { flux5<d>(g, qR, iR, F); return; }
+    const float num = fmad(-(rR * uR), SR - uR, fmad(rL * uL, SL - uL, pR - pL));
+    const float den = fmad(rL, SL - uL, -(rR * (SR - uR)));
+    const float Ss = num / den;
+    const bool left = Ss >= 0.0f;
+    float q[NC];
+    for (int k = 0; k < NC; ++k) q[k] = left ? qL[k] : qR[k];
+    const float r = q[0], ir = left ? iL : iR, u = left ? uL : uR, p = left ? pL : pR;
+    const float S = left ? SL : SR;
+    float f[NC], qs[NC];
     f[0] = r * u;
     for (int m = 0; m < 3; ++m) f[1 + m] = m == d ? fmad(q[1 + m], u, p) : q[1 + m] * u;
     f[4] = u * (q[4] + p);
     // fac = a / dS and p / a with a = rho (S - u), dS = S - S*, from one
     // reciprocal of a dS
-    const T a = r * (S - u), dS = S - Ss, rr = T(1) / (a * dS);
-    const T fac = a * a * rr;
+    const float a = r * (S - u), dS = S - Ss, rr = 1.0f / (a * dS);
+    const float fac = a * a * rr;
     qs[0] = fac;
     for (int m = 0; m < 3; ++m) qs[1 + m] = m == d ? fac * Ss : fac * (q[1 + m] * ir);
     qs[4] = fac * fmad(q[4], ir, (Ss - u) * fmad(p * dS, rr, Ss));
     for (int k = 0; k < NC; ++k) F[k] = fmad(S, qs[k] - q[k], f[k]);
 }
-template <typename T>
-__device__ __forceinline__ T vanleer(T dm, T dp) {
-    const T pr = dm * dp;
-    return pr > T(0) ? T(2) * pr / (dm + dp) : T(0);
+__device__ __forceinline__ float vanleer(float dm, float dp) {
+    const float pr = dm * dp;
+    return pr > 0.0f ? 2.0f * pr / (dm + dp) : 0.0f;
 }
-// gamma and lam / 2 in the type T
-template <typename T> __device__ __forceinline__ T gam(const Desc &D);
-template <> __device__ __forceinline__ double gam<double>(const Desc &D) { return D.gamma; }
-template <> __device__ __forceinline__ float gam<float>(const Desc &D) { return D.gammaf; }
-template <typename T> __device__ __forceinline__ T halflam(const Desc &D);
-template <> __device__ __forceinline__ double halflam<double>(const Desc &D) { return 0.5 * D.lam; }
-template <> __device__ __forceinline__ float halflam<float>(const Desc &D) { return D.hlamf; }
-// the state and evolved-state arrays of the type T
+
+// MUSCL-Hancock evolved boundary states L, R of a cell from its state and its
+// neighbours' along d (conserved variables, van Leer, zero slope next to a
+// solid cell (!lim), first order where an evolved state is not physical),
+// and the HLLC flux of two of them, widened to FP64
+template <typename T, int d> struct Flow;
+template <int d> struct Flow<double, d> {
+    using S = Side<NC>;
+    double g, g1, hl;
+    __device__ __forceinline__ explicit Flow(const Desc &D) : g(D.gamma), g1(D.gamma - 1.0), hl(0.5 * D.lam) {}
+    __device__ __forceinline__ void states(const double *qm, const double *q0, const double *qp, bool lim, S &L,
+                                           S &R) const {
+        evolve64<NC, d>(g1, hl, qm, q0, qp, lim, L, R);
+    }
+    __device__ __forceinline__ void flux(const S &L, const S &R, double *F) const { hllc64<NC, d>(g, L, R, F); }
+};
+template <int d> struct Flow<float, d> {
+    struct S { float q[NC]; };
+    float g, hl;
+    __device__ __forceinline__ explicit Flow(const Desc &D) : g(D.gammaf), hl(D.hlamf) {}
+    __device__ __forceinline__ void states(const float *qm, const float *q0, const float *qp, bool lim, S &L,
+                                           S &R) const {
+        float qL[NC], qR[NC], fL[NC], fR[NC];
+        for (int k = 0; k < NC; ++k) {
+            const float sl = lim ? vanleer(q0[k] - qm[k], qp[k] - q0[k]) : 0.0f;
+            qL[k] = fmad(-0.5f, sl, q0[k]);
+            qR[k] = fmad(0.5f, sl, q0[k]);
+        }
+        const float rr2 = 1.0f / (qL[0] * qR[0]);   // 1/rho of both extrapolated states
+        flux5<d>(g, qL, qR[0] * rr2, fL);
+        flux5<d>(g, qR, qL[0] * rr2, fR);
+        for (int k = 0; k < NC; ++k) {
+            const float df = fL[k] - fR[k];
+            L.q[k] = fmad(hl, df, qL[k]);
+            R.q[k] = fmad(hl, df, qR[k]);
+        }
+        // physical: rho > 0 and p > 0, i.e. 2 rho E > |m|^2
+        auto ok = [](const float *Q) {
+            return Q[0] > 0.0f && 2.0f * Q[0] * Q[4] > Q[1] * Q[1] + Q[2] * Q[2] + Q[3] * Q[3];
+        };
+        if (!ok(L.q) || !ok(R.q))
+            for (int k = 0; k < NC; ++k) { L.q[k] = q0[k]; R.q[k] = q0[k]; }
+    }
+    // (fluxes are FP64 values either way, so that the update's differences
+    // F_lo - F_hi telescope as in the FP64 path)
+    __device__ __forceinline__ void flux(const S &L, const S &R, double *F) const {
+        float f[NC];
+        hllc5<d>(g, L.q, R.q, f);
+        for (int k = 0; k < NC; ++k) F[k] = widen(f[k]);
+    }
+};
+// the state array of the type T
 template <typename T> __device__ __forceinline__ const T *qsrc(const Desc &D);
 template <> __device__ __forceinline__ const double *qsrc<double>(const Desc &D) { return D.Q; }
 template <> __device__ __forceinline__ const float *qsrc<float>(const Desc &D) { return D.Qf; }
-template <typename T> __device__ __forceinline__ T *esrc(const Desc &D);
-template <> __device__ __forceinline__ double *esrc<double>(const Desc &D) { return D.E; }
-template <> __device__ __forceinline__ float *esrc<float>(const Desc &D) { return reinterpret_cast<float *>(D.E); }
-
-// the cell at position m along d of the line through (i, j, k) (the
-// coordinate along d replaced), with the boundary conditions' ghosts:
-// returns its cell index, *flip for a reflective mirror
-__device__ __forceinline__ int line_cell(const Desc &D, int d, const int *base, int m, int nal, bool *flip, int *pos) {
-    const int bc = D.bc[m < 0 ? 2 * d : 2 * d + 1];
-    int mm = m;
+// position m along a line of nal cells with the boundary conditions' ghosts:
+// the cell it is or mirrors, *flip for a reflective mirror
+__device__ __forceinline__ int line_pos(const Desc &D, int d, int m, int nal, bool *flip) {
     *flip = false;
-    if (m < 0 || m >= nal) {
-        if (bc == MB_BC_PERIODIC) { mm %= nal; if (mm < 0) mm += nal; }
-        else { mm = m < 0 ? -1 - m : 2 * nal - 1 - m; *flip = bc == MB_BC_REFLECTIVE; }
-    }
-    int ijk[3] = {base[0], base[1], base[2]};
-    ijk[d] = mm;
-    pos[0] = ijk[0]; pos[1] = ijk[1]; pos[2] = ijk[2];
-    return cidx(D, ijk[0], ijk[1], ijk[2]);
+    if (m >= 0 && m < nal) return m;
+    const int bc = D.bc[m < 0 ? 2 * d : 2 * d + 1];
+    if (bc == MB_BC_PERIODIC) { m %= nal; return m < 0 ? m + nal : m; }
+    *flip = bc == MB_BC_REFLECTIVE;
+    return m < 0 ? -1 - m : 2 * nal - 1 - m;
 }
 
-// MUSCL-Hancock evolved boundary states QL, QR of the cell at position m
-// along the line (conserved variables, van Leer, zero slope next to a solid
-// cell, first order where an evolved state is not physical)
-template <typename T>
-__device__ __forceinline__ void evolve5(const Desc &D, int d, const int *base, int m, int nal, T *QL, T *QR) {
-    const T *Q = qsrc<T>(D);
-    T q[3][NC];
-    bool fl[3];
-    for (int s = 0; s < 3; ++s) {
-        bool flip;
-        int pos[3];
-        const int c = line_cell(D, d, base, m - 1 + s, nal, &flip, pos);
-        fl[s] = fluid_a(D, pos[0], pos[1], pos[2]);
-        for (int k = 0; k < NC; ++k) q[s][k] = Q[(size_t)k * D.n + c];
-        if (flip) q[s][1 + d] = -q[s][1 + d];
-    }
-    const bool lim = fl[0] && fl[2];
-    const T g = gam<T>(D), hl = halflam<T>(D);
-    T qL[NC], qR[NC], fL[NC], fR[NC];
-    for (int k = 0; k < NC; ++k) {
-        const T sl = lim ? vanleer(q[1][k] - q[0][k], q[2][k] - q[1][k]) : T(0);
-        qL[k] = fmad(T(-0.5), sl, q[1][k]);
-        qR[k] = fmad(T(0.5), sl, q[1][k]);
-    }
-    const T rr2 = T(1) / (qL[0] * qR[0]);   // 1/rho of both extrapolated states
-    flux5(g, d, qL, qR[0] * rr2, fL);
-    flux5(g, d, qR, qL[0] * rr2, fR);
-    for (int k = 0; k < NC; ++k) {
-        const T df = fL[k] - fR[k];
-        QL[k] = fmad(hl, df, qL[k]);
-        QR[k] = fmad(hl, df, qR[k]);
-    }
-    // physical: rho > 0 and p > 0, i.e. 2 rho E > |m|^2
-    const bool okL = QL[0] > T(0) && T(2) * QL[0] * QL[4] > QL[1] * QL[1] + QL[2] * QL[2] + QL[3] * QL[3];
-    const bool okR = QR[0] > T(0) && T(2) * QR[0] * QR[4] > QR[1] * QR[1] + QR[2] * QR[2] + QR[3] * QR[3];
-    if (!okL || !okR)
-        for (int k = 0; k < NC; ++k) { QL[k] = q[1][k]; QR[k] = q[1][k]; }
-}
-
-// the d-faces form a grid like the cells' with nfl faces along d (x
-// fastest): the index of the face at (i, j, k), the low d-face of cell
-// (i, j, k) (its d-index may be nal: the high face of the last cell)
-__device__ __forceinline__ int fidx(const Desc &D, int nfl, int i, int j, int k) {
-    const int m0 = D.d == 0 ? nfl : D.nx, m1 = D.d == 1 ? nfl : D.ny;
-    return (k * m1 + j) * m0 + i;
-}
-
-// (the kernels of the sweep's line work take the direction d as a template
-// argument, so that the per-direction indexing is static)
-// the evolved boundary states of every fluid cell along d, once per cell:
-// E holds QL in planes 0..NC-1 and QR in planes NC..2NC-1
-template <int d, typename T>
-__global__ void k3_evolve(Desc D, int nal) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= D.n) return;
-    const int base[3] = {c % D.nx, (c / D.nx) % D.ny, c / (D.nx * D.ny)};
-    if (!fluid_a(D, base[0], base[1], base[2])) return;
-    T QL[NC], QR[NC];
-    evolve5(D, d, base, base[d], nal, QL, QR);
-    T *E = esrc<T>(D);
-    for (int q = 0; q < NC; ++q) {
-        E[(size_t)q * D.n + c] = QL[q];
-        E[(size_t)(NC + q) * D.n + c] = QR[q];
-    }
-}
-
-// the stabilised flux bf F2D of every d-face (eqs. Klein2DtotalfluxaMethod2,
-// Klein2shieldedFluxMethod2, with the two-sided shielded parts) into the
-// NC planes of F, face m of a line between its cells m-1 and m; the
-// evolved states of the cells come from E, those of a boundary's ghost
-// cells (a periodic ghost is the cell it wraps to) are evolved here
-template <int d, typename T>
-__global__ void k3_flux(Desc D, int nal, int nfl, int nlines) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int faces = nfl * nlines;
-    if (t >= faces) return;
-    const int m0 = d == 0 ? nfl : D.nx, m1 = d == 1 ? nfl : D.ny;
-    const int base[3] = {(int)(t % m0), (int)((t / m0) % m1), (int)(t / ((long long)m0 * m1))};
-    const int m = base[d];
-    const bool periodic = D.bc[2 * d] == MB_BC_PERIODIC;
-    double out[NC] = {0, 0, 0, 0, 0};
-    bool flipL, flipR;
-    int pL[3], pR[3];
-    const int cL = line_cell(D, d, base, m - 1, nal, &flipL, pL);
-    const int cR = line_cell(D, d, base, m, nal, &flipR, pR);
-    // face m's time-averaged aperture (the low face of cell m; m = nal: the
-    // high face of the last cell): 1 outside R
-    const bool fin = in_rf(D, d, base[0], base[1], base[2]);
-    const double bf = fin ? D.bt[rfidx(D, d, base[0], base[1], base[2])] : 1.0;
-    if (fluid_a(D, pL[0], pL[1], pL[2]) && fluid_a(D, pR[0], pR[1], pR[2]) && (!fin || bf > 0.0)) {
-        const T *E = esrc<T>(D);
-        T QRa[NC], QLb[NC], G[NC], F[NC];
-        if (m >= 1 || periodic) for (int q = 0; q < NC; ++q) QRa[q] = E[(size_t)(NC + q) * D.n + cL];
-        else evolve5(D, d, base, m - 1, nal, G, QRa);
-        if (m < nal) for (int q = 0; q < NC; ++q) QLb[q] = E[(size_t)q * D.n + cR];
-        else evolve5(D, d, base, m, nal, QLb, G);
-        hllc5(gam<T>(D), d, QRa, QLb, F);
-        const int mR = m < nal ? m : (periodic ? 0 : -1);
-        const int mL = m - 1 >= 0 ? m - 1 : (periodic ? nal - 1 : -1);
-        double sR = 0.0, sL = 0.0, dR = 0.0, dL = 0.0;
-        const double *FBR = nullptr, *FBL = nullptr;
-        bool wall = false;   // a neighbour has wall data (else sR = sL = 0, no test needed)
-        if (mR >= 0) {
-            int c3[3] = {base[0], base[1], base[2]};
-            c3[d] = mR;
-            int f3[3] = {base[0], base[1], base[2]};
-            f3[d] = mR + 1 < nal || !periodic ? mR + 1 : 0;
-            if (in_r(D, c3[0], c3[1], c3[2])) {
-                const int r = ridx(D, c3[0], c3[1], c3[2]);
-                if (D.whas[r]) {
-                    wall = true;
-                    sR = fmax(0.0, bf - swept(D, f3[0], f3[1], f3[2]));
-                    dR = D.wdist[r];
-                    FBR = &D.wFB[(size_t)NC * r];
-                }
+// The face f of a line in R's neighbourhood (f the low d-face of cell ijk[d] =
+// f, f = nal the high face of the last cell): its HLLC flux becomes the
+// stabilised flux bf F2D (eqs. Klein2DtotalfluxaMethod2,
+// Klein2shieldedFluxMethod2, with the two-sided shielded parts); both cells
+// are fluid and bf > 0
+template <typename T, int d>
+__device__ __forceinline__ void stabilise(const Desc &D, const int *ijk, int f, int nal, bool periodic, bool fin,
+                                          double bf, double *F) {
+    const int mR = f < nal ? f : -1, mL = f >= 1 ? f - 1 : (periodic ? nal - 1 : -1);
+    double sR = 0.0, sL = 0.0, dR = 0.0, dL = 0.0;
+    const double *FBR = nullptr, *FBL = nullptr;
+    bool wall = false;   // a neighbour has wall data (else sR = sL = 0)
+    int c3[3] = {ijk[0], ijk[1], ijk[2]};
+    if (mR >= 0) {
+        c3[d] = mR;
+        if (in_r(D, c3[0], c3[1], c3[2])) {
+            const int r = ridx(D, c3[0], c3[1], c3[2]);
+            if (D.whas[r]) {
+                wall = true;
+                c3[d] = mR + 1 < nal || !periodic ? mR + 1 : 0;
+                sR = fmax(0.0, bf - swept(D, c3[0], c3[1], c3[2]));
+                dR = D.wdist[r];
+                FBR = &D.wFB[(size_t)NC * r];
             }
         }
-        if (mL >= 0) {
-            int c3[3] = {base[0], base[1], base[2]};
-            c3[d] = mL;
-            if (in_r(D, c3[0], c3[1], c3[2])) {
-                const int r = ridx(D, c3[0], c3[1], c3[2]);
-                if (D.whas[r]) {
-                    wall = true;
-                    sL = fmax(0.0, bf - swept(D, c3[0], c3[1], c3[2]));
-                    dL = D.wdist[r];
-                    FBL = &D.wFB[(size_t)NC * r];
-                }
+    }
+    if (mL >= 0) {
+        c3[d] = mL;
+        if (in_r(D, c3[0], c3[1], c3[2])) {
+            const int r = ridx(D, c3[0], c3[1], c3[2]);
+            if (D.whas[r]) {
+                wall = true;
+                sL = fmax(0.0, bf - swept(D, c3[0], c3[1], c3[2]));
+                dL = D.wdist[r];
+                FBL = &D.wFB[(size_t)NC * r];
             }
-        }
-        if (wall && sR + sL > bf) {
-            const double sc = bf / (sR + sL);
-            sR *= sc;
-            sL *= sc;
-        }
-        if (wall && (sR > 0.0 || sL > 0.0)) {   // the shielded parts, in FP64
-            for (int q = 0; q < NC; ++q) {
-                const double Fq = F[q];
-                double v = (bf - sL - sR) * Fq;
-                if (sR > 0.0) v += sR * (FBR[q] + dR * (Fq - FBR[q]));
-                if (sL > 0.0) v += sL * (FBL[q] + dL * (Fq - FBL[q]));
-                out[q] = v;
-            }
-        } else {                                // (bf - 0 - 0) F
-            const T b = fin ? T(bf) : T(1);
-            for (int q = 0; q < NC; ++q) out[q] = widen(b * F[q]);
         }
     }
-    // fluxes are stored in FP64 either way, so that the update's
-    // differences F_lo - F_hi telescope as in the FP64 path
-    for (int q = 0; q < NC; ++q) D.F[(size_t)q * faces + t] = out[q];
-}
-
-// alpha_B Q' = alpha_A Q + lam (F_lo - F_hi) + lam (beta_hi - beta_lo)(F^B -
-// w_d Q^B) (eqs. Klein2DcompleteMovingMethod2a-c) into Cn (and C in R)
-template <int d>
-__global__ void k3_update(Desc D, int nal, int nfl) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= D.n) return;
-    const int i = c % D.nx, j = (c / D.nx) % D.ny, k = c / (D.nx * D.ny);
-    const bool periodic = D.bc[2 * d] == MB_BC_PERIODIC;
-    double v[NC] = {0, 0, 0, 0, 0};
-    unsigned char u = 0;
-    if (fluid_a(D, i, j, k)) {
-        const int ijk[3] = {i, j, k};
-        const int m = ijk[d];
-        const int faces = nfl * (D.n / nal);
-        int hi3[3] = {i, j, k};
-        hi3[d] = m + 1 < nal || !periodic ? m + 1 : 0;
-        const int flo = fidx(D, nfl, i, j, k), fhi = fidx(D, nfl, hi3[0], hi3[1], hi3[2]);
-        const double blo = swept(D, i, j, k), bhi = swept(D, hi3[0], hi3[1], hi3[2]);
-        const bool cin = in_r(D, i, j, k);
-        const double aA = cin ? D.aA[ridx(D, i, j, k)] : 1.0;
-        const bool w = cin && D.whas[ridx(D, i, j, k)] && blo != bhi;
-        const int r = w ? ridx(D, i, j, k) : 0;
+    if (wall && sR + sL > bf) {
+        const double sc = bf / (sR + sL);
+        sR *= sc;
+        sL *= sc;
+    }
+    if (wall && (sR > 0.0 || sL > 0.0)) {
         for (int q = 0; q < NC; ++q) {
-            const double Qq = D.Q[(size_t)q * D.n + c];   // alpha_A Q, which is Q outside R
-            double x = (cin ? aA * Qq : Qq) + D.lam * (D.F[(size_t)q * faces + flo] - D.F[(size_t)q * faces + fhi]);
-            if (w) {
-                const double wt = D.lam * (bhi - blo) * (D.wFB[(size_t)NC * r + q] - D.U[d] * D.wQB[(size_t)NC * r + q]);
-                x += wt;
-                atomicAdd(&D.wall[q], wt);
-            }
-            v[q] = x;
+            const double Fq = F[q];
+            double v = (bf - sL - sR) * Fq;
+            if (sR > 0.0) v += sR * (FBR[q] + dR * (Fq - FBR[q]));
+            if (sL > 0.0) v += sL * (FBL[q] + dL * (Fq - FBL[q]));
+            F[q] = v;
         }
-        u = 1;
+    } else if (fin && bf != 1.0) {
+        // (the FP32 option's product in FP32)
+        for (int q = 0; q < NC; ++q) F[q] = sizeof(T) == 4 ? widen((float)bf * (float)F[q]) : bf * F[q];
     }
-    // C keeps the content for the events, which read it in R only (event
-    // cells are cut at pose A or B, their neighbours within R)
-    const bool inr = in_r(D, i, j, k);
+}
+// flux of face f of the line through ijk between cells with states L (of the
+// low cell) and R; GEN: zero next to a solid cell, stabilised near the body
+template <typename T, int d, bool GEN>
+__device__ __forceinline__ void line_flux(const Desc &D, const Flow<T, d> &fl, const int *line, int f, int nal,
+                                          bool fluids, const typename Flow<T, d>::S &L, const typename Flow<T, d>::S &R,
+                                          double *F) {
+    if (GEN) {
+        const bool periodic = D.bc[2 * d] == MB_BC_PERIODIC;
+        int ijk[3] = {line[0], line[1], line[2]};
+        ijk[d] = periodic && f == nal ? 0 : f;
+        const bool fin = in_rf(D, d, ijk[0], ijk[1], ijk[2]);
+        const double bf = fin ? D.bt[rfidx(D, d, ijk[0], ijk[1], ijk[2])] : 1.0;
+        for (int q = 0; q < NC; ++q) F[q] = 0.0;
+        if (!fluids || (fin && !(bf > 0.0))) return;
+        fl.flux(L, R, F);
+        stabilise<T, d>(D, ijk, ijk[d], nal, periodic, fin, bf, F);
+    } else {
+        fl.flux(L, R, F);
+    }
+}
+
+// the content update x = Q + lam (F_lo - F_hi) of a cell away from the body
+// (fused for the FP64 path; the FP32 option rounds each operation) and its
+// FP32 copy
+__device__ __forceinline__ double content(double lam, double q, double flo, double fhi, double) {
+    return __fma_rn(lam, flo - fhi, q);
+}
+__device__ __forceinline__ double content(double lam, double q, double flo, double fhi, float) {
+    return q + lam * (flo - fhi);
+}
+// alpha_B Q' = alpha_A Q + lam (F_lo - F_hi) + lam (beta_hi - beta_lo)(F^B -
+// w_d Q^B) (eqs. Klein2DcompleteMovingMethod2a-c) of cell m of the line
+// through ijk, index c, into Cn (in R also C and upd; elsewhere the FP32 copy
+// and the safeguard's seed test: alpha_A = alpha_B = 1 there and no event
+// changes the content).  w: this thread's wall terms.
+template <typename T, int d, bool GEN>
+__device__ __forceinline__ void line_update(const Desc &D, const int *line, int m, int nal, int c, const double *Q,
+                                            const double *Flo, const double *Fhi, double *w) {
+    double v[NC];
+    if (GEN) {
+        int ijk[3] = {line[0], line[1], line[2]};
+        ijk[d] = m;
+        if (in_r(D, ijk[0], ijk[1], ijk[2])) {
+            const int r = ridx(D, ijk[0], ijk[1], ijk[2]);
+            const bool fl = fluid_a(D, ijk[0], ijk[1], ijk[2]);
+            const double aA = D.aA[r];
+            const double blo = swept(D, ijk[0], ijk[1], ijk[2]);
+            ijk[d] = m + 1 < nal || D.bc[2 * d] != MB_BC_PERIODIC ? m + 1 : 0;
+            const double bhi = swept(D, ijk[0], ijk[1], ijk[2]);
+            const bool wall = fl && D.whas[r] && blo != bhi;
+            for (int q = 0; q < NC; ++q) {
+                v[q] = 0.0;
+                if (fl) v[q] = aA * Q[q] + D.lam * (Flo[q] - Fhi[q]);
+                if (wall) {
+                    const double wt = D.lam * (bhi - blo) * (D.wFB[(size_t)NC * r + q] -
+                                                             D.U[d] * D.wQB[(size_t)NC * r + q]);
+                    v[q] += wt;
+                    w[q] += wt;
+                }
+                D.C[(size_t)q * D.n + c] = v[q];
+                D.Cn[(size_t)q * D.n + c] = v[q];
+            }
+            D.upd[r] = fl;
+            return;
+        }
+    }
     for (int q = 0; q < NC; ++q) {
-        if (inr) D.C[(size_t)q * D.n + c] = v[q];
+        v[q] = content(D.lam, Q[q], Flo[q], Fhi[q], T(0));
         D.Cn[(size_t)q * D.n + c] = v[q];
     }
-    D.upd[c] = u;
-    // a safeguard seed outside R (alpha_A = alpha_B = 1 there, no event
-    // changes the content): a non-physical content
-    if (u && !inr && content_bad(v)) add_seed(D, c);
+    if (sizeof(T) == 4) {
+        float x[NC];
+        for (int q = 0; q < NC; ++q) {
+            x[q] = narrow32(v[q]);
+            D.Qfn[(size_t)q * D.n + c] = x[q];
+        }
+        // the seed test in FP32 where that decides with a margin of 1e-5
+        const float t = 2.0f * x[0] * x[4];
+        if (!(x[0] > 0.0f && x[4] > 0.0f && t < 1e38f && t - sq3(x + 1) > 1e-5f * t) && content_bad(v))
+            add_seed(D, c);
+    } else if (!physical64<NC>(v)) {
+        if (content_bad(v)) add_seed(D, c);
+    }
+}
+// a warp's wall terms, one atomic per component
+__device__ __forceinline__ void add_wall(const Desc &D, const double *w) {
+    bool any = false;
+    for (int q = 0; q < NC; ++q) any = any || w[q] != 0.0;
+    if (!__any_sync(0xffffffffu, any)) return;
+    for (int q = 0; q < NC; ++q) {
+        double s = w[q];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((threadIdx.x & 31) == 0 && s != 0.0) atomicAdd(&D.wall[q], s);
+    }
+}
+
+// The near cells of a sweep along d: the lines through R's cross-section, from
+// two cells before R to two after its last d-face (over a periodic side too).
+// Only their update reads body data: k3_row and k3_march update all other
+// cells, beside the geometry, and k3_near_row and k3_near the near ones after
+// k3_wall (few, and FP64 chains: as many threads as there are cells).
+struct Near { int a, len; bool wrap; };   // positions a .. a + len - 1 (modulo a periodic line)
+__host__ __device__ inline Near near_range(const Desc &D, int d, int nal) {
+    Near N;
+    N.a = D.r0[d] - 2;
+    N.len = D.rn[d] > 0 ? D.rn[d] + 5 : 0;
+    N.wrap = D.bc[2 * d] == MB_BC_PERIODIC;
+    if (N.wrap) {
+        if (N.len > nal) N.len = nal;
+    } else {
+        const int e = N.a + N.len < nal ? N.a + N.len : nal;
+        if (N.a < 0) N.a = 0;
+        N.len = e > N.a ? e - N.a : 0;
+    }
+    return N;
+}
+__device__ __forceinline__ bool near_line(const Desc &D, int d, const int *ijk) {
+    bool in = D.rn[0] > 0;
+    for (int q = 0; q < 3; ++q) in = in && (q == d || (ijk[q] >= D.r0[q] && ijk[q] < D.r0[q] + D.rn[q]));
+    return in;
+}
+__device__ __forceinline__ bool near_pos(const Near &N, int m, int nal) {
+    int r = m - N.a;
+    if (N.wrap) r += r >= nal ? -nal : r < 0 ? nal : 0;
+    return r >= 0 && r < N.len;
+}
+
+// x sweep.  The line kernels keep the evolved states and the fluxes in
+// registers: per cell they read the state and write the new one (80 bytes; 120
+// with the FP32 copy), where a kernel each for the states, the fluxes, the
+// update and the new state moved 400.  FP64: bound by the FP64 pipe, 180 lane
+// operations per cell; 4 M cells per sweep, before -> after: x 2520 -> 1298
+// us, y 2400 -> 1395, z 2390 -> 1392 (0.85 of the pipe's rate).  FP32 option:
+// 15 FP64 lane operations per cell (the update) and about 700 instructions;
+// 32 M cells per sweep, 3790 -> 1002 us (x), 1104, 1133.  Rows are laid end
+// to end as slots, position -1 .. nx of every row, and a warp takes 32 slots
+// from slot 30 w on: it evolves 32 positions, forms 31 fluxes and updates 30
+// cells, whatever the row length.
+template <typename T, bool GEN>
+__device__ __forceinline__ void row_unit(const Desc &D, bool store, int p, int j, int k) {
+    const Flow<T, 0> fl(D);
+    const int line[3] = {0, j, k};
+    const int row = (k * D.ny + j) * D.nx;
+    const T *__restrict__ Q = qsrc<T>(D) + row;
+    T q[3][NC];
+    bool fu[3];
+    for (int s = 0; s < 3; ++s) {
+        bool flip;
+        const int c = line_pos(D, 0, p - 1 + s, D.nx, &flip);
+        for (int m = 0; m < NC; ++m) q[s][m] = Q[(size_t)m * D.n + c];
+        if (flip) q[s][1] = -q[s][1];
+        fu[s] = !GEN || fluid_a(D, c, j, k);
+    }
+    double Qd[NC];   // the cell's FP64 state
+    for (int m = 0; m < NC; ++m)
+        Qd[m] = sizeof(T) == 8 ? (double)q[1][m] : store ? D.Q[(size_t)m * D.n + row + p] : 0.0;
+    typename Flow<T, 0>::S L, R;
+    fl.states(q[0], q[1], q[2], fu[0] && fu[2], L, R);
+    {   // the right state of the slot below
+        T *x = reinterpret_cast<T *>(&R);
+        for (int m = 0; m < (int)(sizeof(R) / sizeof(T)); ++m) x[m] = __shfl_up_sync(0xffffffffu, x[m], 1);
+    }
+    double F[NC], Fhi[NC];
+    line_flux<T, 0, GEN>(D, fl, line, max(p, 0), D.nx, fu[0] && fu[1], R, L, F);
+    for (int m = 0; m < NC; ++m) Fhi[m] = __shfl_down_sync(0xffffffffu, F[m], 1);
+    double w[NC] = {0, 0, 0, 0, 0};
+    if (store) line_update<T, 0, GEN>(D, line, p, D.nx, row + p, Qd, F, Fhi, w);
+    if (GEN) add_wall(D, w);
+}
+// slot s of rows of len positions: its row, its position in it
+__device__ __forceinline__ unsigned row_slot(unsigned len, unsigned *s) {
+    *s = (unsigned)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 30u + (threadIdx.x & 31u);
+    const unsigned row = *s / len;
+    *s -= row * len;
+    return row;
+}
+__device__ __forceinline__ bool mid_lane() { return (threadIdx.x & 31u) - 1u < 30u; }
+template <typename T>
+__global__ void __launch_bounds__(128, 4) k3_row(Desc D) {
+    const unsigned rows = (unsigned)(D.ny * D.nz);
+    unsigned s;
+    const unsigned r = row_slot((unsigned)D.nx + 2u, &s), row = min(r, rows - 1u);
+    const int p = (int)s - 1, k = (int)(row / (unsigned)D.ny), j = (int)(row - (unsigned)k * (unsigned)D.ny);
+    const int ijk[3] = {0, j, k};
+    bool store = r < rows && p >= 0 && p < D.nx && mid_lane();
+    if (near_line(D, 0, ijk)) store = store && !near_pos(near_range(D, 0, D.nx), p, D.nx);
+    row_unit<T, false>(D, store, p, j, k);
+}
+template <typename T>
+__global__ void __launch_bounds__(128, 3) k3_near_row(Desc D, Near N) {
+    const unsigned rows = (unsigned)(D.rn[1] * D.rn[2]);
+    unsigned s;
+    const unsigned r = row_slot((unsigned)N.len + 2u, &s), row = min(r, rows - 1u);
+    const int k = D.r0[2] + (int)(row / (unsigned)D.rn[1]), j = D.r0[1] + (int)(row % (unsigned)D.rn[1]);
+    const bool store = r < rows && s >= 1u && s <= (unsigned)N.len && mid_lane();
+    int p = N.a + (int)s - 1;
+    if (D.bc[0] == MB_BC_PERIODIC) {   // a cell's own position (its neighbours' are mapped)
+        p %= D.nx;
+        if (p < 0) p += D.nx;
+    }
+    row_unit<T, true>(D, store, p, j, k);
+}
+
+// y and z sweeps: a thread marches along seg cells of its line with a
+// register window, 32 neighbouring lines per warp (along x, running on over
+// the row's end), so that loads and stores are whole rows
+template <typename T, int d, bool GEN>
+__device__ __forceinline__ void march(const Desc &D, bool in, bool nearl, const int *line, int base, int stride,
+                                      int m0, int m1, int nal) {
+    using S = typename Flow<T, d>::S;
+    const Flow<T, d> fl(D);
+    const T *__restrict__ Q = qsrc<T>(D) + base;
+    auto load = [&](int m, T *q, bool &fu) {
+        bool flip;
+        const int p = line_pos(D, d, m, nal, &flip);
+        for (int k = 0; k < NC; ++k) q[k] = Q[(size_t)k * D.n + (size_t)p * stride];
+        if (flip) q[1 + d] = -q[1 + d];
+        fu = true;
+        if (GEN) {
+            int ijk[3] = {line[0], line[1], line[2]};
+            ijk[d] = p;
+            fu = fluid_a(D, ijk[0], ijk[1], ijk[2]);
+        }
+    };
+    const Near N = near_range(D, d, nal);
+    T qm[NC], qc[NC], qp[NC], qq[NC];
+    bool um, uc, up, uq;
+    S L, R, Rc;
+    double F[NC], Fp[NC], w[NC] = {0, 0, 0, 0, 0};
+    {
+        T qa[NC];
+        bool ua;
+        load(m0 - 2, qa, ua);
+        load(m0 - 1, qm, um);
+        load(m0, qc, uc);
+        load(m0 + 1, qp, up);
+        fl.states(qa, qm, qc, ua && uc, L, Rc);
+    }
+    for (int f = m0; f <= m1; ++f) {
+        if (f < m1) load(f + 2, qq, uq);   // the next face's high neighbour
+        double Qd[NC];
+        const int c = base + (f - 1) * stride;
+        const bool store = f > m0 && in && (GEN || !(nearl && near_pos(N, f - 1, nal)));
+        if (sizeof(T) == 4) {
+            if (store)
+                for (int k = 0; k < NC; ++k) Qd[k] = D.Q[(size_t)k * D.n + c];
+        } else {
+            for (int k = 0; k < NC; ++k) Qd[k] = qm[k];
+        }
+        fl.states(qm, qc, qp, um && up, L, R);
+        line_flux<T, d, GEN>(D, fl, line, f, nal, um && uc, Rc, L, F);
+        if (store) line_update<T, d, GEN>(D, line, f - 1, nal, c, Qd, Fp, F, w);
+        Rc = R;
+        um = uc; uc = up; up = uq;
+        for (int k = 0; k < NC; ++k) {
+            Fp[k] = F[k];
+            qm[k] = qc[k];
+            qc[k] = qp[k];
+            qp[k] = qq[k];
+        }
+    }
+    if (GEN) add_wall(D, w);
+}
+template <typename T, int d>
+__global__ void __launch_bounds__(32, 12) k3_march(Desc D, int seg, unsigned nlb) {
+    const unsigned sg = blockIdx.x / nlb, lb = blockIdx.x - sg * nlb;
+    const int nal = d == 1 ? D.ny : D.nz, nlines = D.n / nal;
+    const int l = (int)(lb * 32u + threadIdx.x);
+    const bool in = l < nlines;
+    const int lc = in ? l : nlines - 1;
+    const int i = lc % D.nx, o = lc / D.nx;   // o: the line's other coordinate (z for d = 1, y for d = 2)
+    const int line[3] = {i, d == 1 ? 0 : o, d == 1 ? o : 0};
+    const int m0 = (int)sg * seg, m1 = min(nal, m0 + seg);
+    const int base = d == 1 ? o * D.ny * D.nx + i : lc, stride = d == 1 ? D.nx : D.nx * D.ny;
+    march<T, d, false>(D, in, near_line(D, d, line), line, base, stride, m0, m1, nal);
+}
+// the near cells of a y or z sweep, one per thread
+template <typename T, int d>
+__global__ void __launch_bounds__(128, 3) k3_near(Desc D, Near N) {
+    const int nal = d == 1 ? D.ny : D.nz, no = d == 1 ? D.rn[2] : D.rn[1];
+    const int t = (int)(blockIdx.x * 128u + threadIdx.x), tot = D.rn[0] * no * N.len;
+    const bool in = t < tot;
+    const int tc = in ? t : tot - 1;
+    const int i = D.r0[0] + tc % D.rn[0], o = D.r0[d == 1 ? 2 : 1] + (tc / D.rn[0]) % no;
+    int m = N.a + tc / (D.rn[0] * no);
+    if (D.bc[2 * d] == MB_BC_PERIODIC) {
+        m %= nal;
+        if (m < 0) m += nal;
+    }
+    const int line[3] = {i, d == 1 ? 0 : o, d == 1 ? o : 0};
+    const int base = d == 1 ? o * D.ny * D.nx + i : o * D.nx + i, stride = d == 1 ? D.nx : D.nx * D.ny;
+    march<T, d, true>(D, in, true, line, base, stride, m, m + 1, nal);
 }
 
 // covering / uncovering (Sec. II.C.5): each event cell of R finds its
@@ -933,7 +1122,7 @@ __global__ void k3_events(Desc D) {
             }
             D.Cn[(size_t)q * D.n + c] = sigma * tot;
         }
-        D.upd[c] = 1;
+        D.upd[t] = 1;
         return;
     }
     // a recipient or donor: the event cells among the 26 neighbours that
@@ -978,7 +1167,7 @@ __global__ void k3_bad(Desc D) {
     int i, j, k;
     r_cell(D, t, &i, &j, &k);
     const int c = cidx(D, i, j, k);
-    if (!D.upd[c]) return;
+    if (!D.upd[t]) return;
     const double aB = D.aB[t];
     if (!(aB > 0.0)) return;
     double q[NC];
@@ -998,6 +1187,11 @@ __device__ bool physical5(const Desc &D, int c) {
         if (!isfinite(q[m])) return false;
     }
     return q[0] > 0.0 && pressure5(D.gamma, q) > 0.0;
+}
+// a merged cell's content; its FP32 copy too (in R k3_final writes it again)
+__device__ __forceinline__ void put_share(const Desc &D, int c, int q, double v) {
+    D.Cn[(size_t)q * D.n + c] = v;
+    if (D.f32) D.Qfn[(size_t)q * D.n + c] = float(v);
 }
 // (one thread, over global lists: the form for clusters too large for the
 // shared-memory form in k3_mix; it continues from layer layer0 with the ns
@@ -1032,7 +1226,7 @@ __device__ void mix_serial(const Desc &D, int ns, int layer0, int mixed) {
             for (int m = 0; m < 6; ++m) {
                 int ii, jj, kk;
                 const int cc = nbr(D, i, j, k, off[m][0], off[m][1], off[m][2], &ii, &jj, &kk);
-                if (cc < 0 || !(alphaB(D, ii, jj, kk) > 0.0) || !D.upd[cc]) continue;
+                if (cc < 0 || !(alphaB(D, ii, jj, kk) > 0.0) || !updated(D, ii, jj, kk)) continue;
                 const int b = add(cc);
                 if (b < 0) break;
                 const int ra = root(a), rb = root(b);
@@ -1077,7 +1271,7 @@ __device__ void mix_serial(const Desc &D, int ns, int layer0, int mixed) {
             const int sr = slot(rootcell[x]);
             const double aB = alphaB(D, i, j, k);
             for (int q = 0; q < NC; ++q)
-                D.Cn[(size_t)q * D.n + c] = aB * (D.ntot[(NC + 1) * sr + q] / D.ntot[(NC + 1) * sr + NC]);
+                put_share(D, c, q, aB * (D.ntot[(NC + 1) * sr + q] / D.ntot[(NC + 1) * sr + NC]));
         }
         mixed += nn;
         // cells still non-physical, in cell order
@@ -1114,7 +1308,7 @@ __global__ void __launch_bounds__(MIXS_THREADS) k3_mix(Desc D) {
     __shared__ int snode[MIXS_SEEDS];       // the seed's node
     __shared__ int nodes[MIXS_NODES], lbl[MIXS_NODES];
     __shared__ double cache[MIXS_NODES][NC + 1], sums[MIXS_NODES][NC + 1];
-    __shared__ int s_wsum[MIXS_THREADS / 32], s_nn, s_changed, s_nb;
+    __shared__ int s_wsum[MIXS_THREADS / 32], s_changed, s_nb;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     int ns = *D.nseed;
     if (ns > SEEDCAP) {
@@ -1137,7 +1331,7 @@ __global__ void __launch_bounds__(MIXS_THREADS) k3_mix(Desc D) {
             for (int m = 0; m < 6; ++m) {
                 int ii, jj, kk;
                 const int cc = nbr(D, i, j, k, off[m][0], off[m][1], off[m][2], &ii, &jj, &kk);
-                const bool ok = cc >= 0 && alphaB(D, ii, jj, kk) > 0.0 && D.upd[cc];
+                const bool ok = cc >= 0 && alphaB(D, ii, jj, kk) > 0.0 && updated(D, ii, jj, kk);
                 cand[7 * s + 1 + m] = ok ? cc : INT_MAX;
                 enode[6 * s + m] = ok ? cc : -1;
             }
@@ -1229,7 +1423,7 @@ __global__ void __launch_bounds__(MIXS_THREADS) k3_mix(Desc D) {
         for (int x = tid; x < nn; x += MIXS_THREADS) {
             const int c = nodes[x], r = lbl[x];
             const double aB = cache[x][NC];
-            for (int q = 0; q < NC; ++q) D.Cn[(size_t)q * D.n + c] = aB * (sums[r][q] / sums[r][NC]);
+            for (int q = 0; q < NC; ++q) put_share(D, c, q, aB * (sums[r][q] / sums[r][NC]));
             if (!physical5(D, c)) D.seeds[atomicAdd(&s_nb, 1)] = c;
         }
         mixed += nn;
@@ -1246,32 +1440,29 @@ __global__ void __launch_bounds__(MIXS_THREADS) k3_mix(Desc D) {
 }
 
 // Q = content / alpha_B (NaN where alpha_B = 0 or the cell was not
-// updated), with the checks of the new state
-// (outside R alpha_B = 1 and the state is the content: its test was the
-// seed test, and the safeguard flags cells it leaves non-physical)
+// updated) in R, in place, with the checks of the new state.  Elsewhere
+// alpha_B = 1 and the content is the state: its test was the seed test, and
+// the safeguard flags cells it leaves non-physical.
 __global__ void k3_final(Desc D) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= D.n) return;
-    const int i = c % D.nx, j = (c / D.nx) % D.ny, k = c / (D.nx * D.ny);
-    if (!in_r(D, i, j, k)) {
-        for (int m = 0; m < NC; ++m) {
-            const double cn = D.Cn[(size_t)m * D.n + c];
-            D.Q[(size_t)m * D.n + c] = cn;
-            if (D.f32) D.Qf[(size_t)m * D.n + c] = float(cn);
-        }
-        return;
-    }
-    const double aB = alphaB(D, i, j, k);
-    const bool ok = aB > 0.0 && D.upd[c];
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= D.rn[0] * D.rn[1] * D.rn[2]) return;
+    int i, j, k;
+    r_cell(D, t, &i, &j, &k);
+    const int c = cidx(D, i, j, k);
+    const double aB = D.aB[t];
+    const bool ok = aB > 0.0 && D.upd[t];
     const double ia = ok ? (aB == 1.0 ? 1.0 : 1.0 / aB) : 0.0;
     double q[NC];
     for (int m = 0; m < NC; ++m) {
         const double cn = D.Cn[(size_t)m * D.n + c];
         q[m] = ok ? (ia == 1.0 ? cn : cn * ia) : NAN;
-        D.Q[(size_t)m * D.n + c] = q[m];
-        if (D.f32) D.Qf[(size_t)m * D.n + c] = float(q[m]);
+        D.Cn[(size_t)m * D.n + c] = q[m];
+        if (D.f32) D.Qfn[(size_t)m * D.n + c] = float(q[m]);
+        // the provisional state of a cell that was solid at pose A (k3_wall)
+        // leaves the step-start state
+        if (D.gcl && D.aA[t] == 0.0) D.Q[(size_t)m * D.n + c] = NAN;
     }
-    if (aB > 0.0 && !D.upd[c]) atomicOr(D.err, E_UNSTABLE);
+    if (aB > 0.0 && !D.upd[t]) atomicOr(D.err, E_UNSTABLE);
     if (ok) {
         bool bad = !(q[0] > 0.0) || !(2.0 * q[0] * q[4] > q[1] * q[1] + q[2] * q[2] + q[3] * q[3]);
         for (int m = 0; m < NC; ++m) if (!finite64(q[m])) bad = true;
@@ -1280,36 +1471,109 @@ __global__ void k3_final(Desc D) {
 }
 
 // maxima of |u_d| + c over the fluid cells (positive doubles compare as
-// their bit patterns)
-// (a grid-stride loop, 256-thread blocks: one atomic per block and axis;
-// in the type T of the flow arithmetic)
+// their bit patterns), in the type T of the flow arithmetic; 256-thread
+// blocks, one atomic per block and axis.
+// FP64: a block takes 2048 cells at a time and first forms their speeds in
+// FP32 (error below 4e-6 of the speed where p > E / 10); only a cell within
+// 1e-5 of the largest the block has seen along an axis, or with a smaller
+// pressure, goes through the FP64 formula, so that the result is that
+// formula's over every cell.  4 M cells: 267 us with the FP64 formula
+// throughout.
+constexpr int SPEED_CELLS = 8;   // cells per thread and turn (FP64)
 template <typename T>
-__global__ void k3_speeds(Desc D) {
-    __shared__ double red[3][8];
-    const T *Q = qsrc<T>(D);
-    const T g = gam<T>(D);
-    T s[3] = {T(0), T(0), T(0)};
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < D.n; c += gridDim.x * blockDim.x) {
-        if (isnan(Q[c])) continue;
-        T q[NC];
-        for (int m = 0; m < NC; ++m) q[m] = Q[(size_t)m * D.n + c];
-        const T ir = T(1) / q[0];
-        const T p = (g - T(1)) * (q[4] - T(0.5) * (q[1] * q[1] + q[2] * q[2] + q[3] * q[3]) * ir);
-        const T cs = sqrt(g * p * ir);
-        for (int a = 0; a < 3; ++a) s[a] = fmax(s[a], fabs(q[1 + a] * ir) + cs);
-    }
-    const int w = threadIdx.x >> 5;
+__device__ __forceinline__ void block_max3(const T *s, T (*red)[8], T *m) {
     for (int a = 0; a < 3; ++a) {
-        double v = double(s[a]);
+        T v = s[a];
         for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-        if ((threadIdx.x & 31) == 0) red[a][w] = v;
+        if ((threadIdx.x & 31) == 0) red[a][threadIdx.x >> 5] = v;
     }
     __syncthreads();
-    if (threadIdx.x < 3) {
-        double v = 0.0;
-        for (int q = 0; q < 8; ++q) v = fmax(v, red[threadIdx.x][q]);
-        if (v > 0.0) atomicMax((unsigned long long *)&D.smax[threadIdx.x], (unsigned long long)__double_as_longlong(v));
+    for (int a = 0; a < 3; ++a) {
+        m[a] = red[a][0];
+        for (int q = 1; q < 8; ++q) m[a] = fmax(m[a], red[a][q]);
     }
+    __syncthreads();
+}
+__device__ __forceinline__ void put_speeds(const Desc &D, const double *v) {
+    const int a = threadIdx.x;
+    if (a < 3 && v[a] > 0.0)
+        atomicMax((unsigned long long *)&D.smax[a], (unsigned long long)__double_as_longlong(v[a]));
+}
+__global__ void __launch_bounds__(256) k3_speeds64(Desc D) {
+    __shared__ float redf[3][8];
+    __shared__ double red[3][8];
+    const double g = D.gamma;
+    const float gf = D.gammaf;
+    double s[3] = {0.0, 0.0, 0.0};
+    float lead[3] = {0.0f, 0.0f, 0.0f};
+    for (long long c0 = (long long)blockIdx.x * 256 * SPEED_CELLS; c0 < D.n; c0 += (long long)gridDim.x * 256 * SPEED_CELLS) {
+        float v[SPEED_CELLS][3], m[3] = {0.0f, 0.0f, 0.0f};
+        unsigned want = 0u;
+#pragma unroll
+        for (int u = 0; u < SPEED_CELLS; ++u) {
+            const long long c = c0 + u * 256 + threadIdx.x;
+            v[u][0] = v[u][1] = v[u][2] = -1.0f;
+            if (c >= D.n) continue;
+            bool ok = true;
+            float x[NC];
+            bool fluid = true;
+            for (int k = 0; k < NC; ++k) {
+                const double q = D.Q[(size_t)k * D.n + c];
+                if (k == 0) fluid = !isnan64(q);
+                x[k] = near32(q, ok);
+            }
+            if (!fluid) continue;
+            const float ir = __fdividef(1.0f, x[0]);
+            const float p = (gf - 1.0f) * (x[4] - 0.5f * sq3(x + 1) * ir);
+            if (!(ok && x[0] > 1e-30f && x[4] < 1e30f && p > 0.1f * x[4])) { want |= 1u << u; continue; }
+            const float cs = sqrtf(gf * p * ir);
+            for (int a = 0; a < 3; ++a) {
+                v[u][a] = fabsf(x[1 + a] * ir) + cs;
+                m[a] = fmaxf(m[a], v[u][a]);
+            }
+        }
+        float bm[3];
+        block_max3<float>(m, redf, bm);
+        for (int a = 0; a < 3; ++a) lead[a] = fmaxf(lead[a], bm[a]);
+#pragma unroll
+        for (int u = 0; u < SPEED_CELLS; ++u) {
+            for (int a = 0; a < 3; ++a)
+                if (v[u][a] >= lead[a] * (1.0f - 1e-5f)) want |= 1u << u;
+        }
+        while (want) {
+            const int u = __ffs(want) - 1;
+            want &= want - 1;
+            const long long c = c0 + u * 256 + threadIdx.x;
+            double q[NC];
+            for (int k = 0; k < NC; ++k) q[k] = D.Q[(size_t)k * D.n + c];
+            const double ir = rcp64(q[0]), p = press64<NC>(g - 1.0, q, ir), cs = sqrt64(g * (p * ir));
+            for (int a = 0; a < 3; ++a) {
+                const double x = __fma_rn(abs64(q[1 + a]), ir, cs);
+                if (pos64(x)) s[a] = max64(s[a], x);
+            }
+        }
+    }
+    double bm[3];
+    block_max3<double>(s, red, bm);
+    put_speeds(D, bm);
+}
+__global__ void __launch_bounds__(256) k3_speeds32(Desc D) {
+    __shared__ float red[3][8];
+    const float g = D.gammaf;
+    float s[3] = {0.0f, 0.0f, 0.0f};
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < D.n; c += gridDim.x * blockDim.x) {
+        float q[NC];
+        for (int m = 0; m < NC; ++m) q[m] = D.Qf[(size_t)m * D.n + c];
+        if (isnan(q[0])) continue;
+        const float ir = 1.0f / q[0];
+        const float p = (g - 1.0f) * (q[4] - 0.5f * (q[1] * q[1] + q[2] * q[2] + q[3] * q[3]) * ir);
+        const float cs = sqrtf(g * p * ir);
+        for (int a = 0; a < 3; ++a) s[a] = fmaxf(s[a], fabsf(q[1 + a] * ir) + cs);
+    }
+    float bm[3];
+    block_max3<float>(s, red, bm);
+    const double v[3] = {(double)bm[0], (double)bm[1], (double)bm[2]};
+    put_speeds(D, v);
 }
 
 // solid cells (alpha = 0 in R at the current pose) read NaN; alpha of every
@@ -1347,15 +1611,17 @@ struct mb3_sim {
     int sidx = 0;
     double dt_step = 0.0, cfl = 0.5;
     cudaStream_t st = nullptr;
-    cudaStream_t gs[2] = {nullptr, nullptr};      // face apertures and swept apertures beside k3_cells
-    cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};
+    // the geometry (k3_cells, k3_faces, k3_swept side by side, then k3_wall)
+    // beside the cells away from the body
+    cudaStream_t gs[3] = {nullptr, nullptr, nullptr};
+    cudaEvent_t fork = nullptr, join[3] = {nullptr, nullptr, nullptr};
     std::string err;
     size_t rcap = 0, rfcap = 0;
     bool prev_ok = false;        // aB / tB hold the current pose over the region q0, qn
     int q0[3] = {0, 0, 0}, qn[3] = {0, 0, 0};
     double wall_host[NC] = {0, 0, 0, 0, 0};
     int merged = 0;
-    cudaEvent_t ev0 = nullptr, ev1 = nullptr;   // around the last sweep's k3_flux
+    cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};   // around the last sweep's two line launches
     float flux_ms = 0.0f;
     std::vector<void *> owned;
 };
@@ -1426,7 +1692,7 @@ static cudaError_t ensure_r(mb3_sim *s, size_t rc, size_t rf) {
         dfree(s, D.aA); dfree(s, D.aM); dfree(s, D.aB); dfree(s, D.tA); dfree(s, D.tB); dfree(s, D.whas);
         dfree(s, D.aP); dfree(s, D.tP);
         s->prev_ok = false;
-        dfree(s, D.wdist); dfree(s, D.wFB); dfree(s, D.wQB); dfree(s, D.evt); dfree(s, D.emask); dfree(s, D.easum);
+        dfree(s, D.wdist); dfree(s, D.wFB); dfree(s, D.wQB); dfree(s, D.evt); dfree(s, D.upd); dfree(s, D.emask); dfree(s, D.easum);
         const size_t c = rc + rc / 4;
         if (e == cudaSuccess) e = dalloc(s, &D.aA, c);
         if (e == cudaSuccess) e = dalloc(s, &D.aM, c);
@@ -1440,6 +1706,7 @@ static cudaError_t ensure_r(mb3_sim *s, size_t rc, size_t rf) {
         if (e == cudaSuccess) e = dalloc(s, &D.wFB, NC * c);
         if (e == cudaSuccess) e = dalloc(s, &D.wQB, NC * c);
         if (e == cudaSuccess) e = dalloc(s, &D.evt, c);
+        if (e == cudaSuccess) e = dalloc(s, &D.upd, c);
         if (e == cudaSuccess) e = dalloc(s, &D.emask, c);
         if (e == cudaSuccess) e = dalloc(s, &D.easum, c);
         s->rcap = e == cudaSuccess ? c : 0;
@@ -1515,23 +1782,19 @@ mb_status mb3_create(const mb3_grid *g, double gamma, double cfl, const mb3_body
     }
     for (int q = 0; q < 6; ++q) s->bb[q] = b->bbox[q];
     cudaError_t e = cudaStreamCreateWithFlags(&s->st, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreate(&s->ev0);
-    if (e == cudaSuccess) e = cudaEventCreate(&s->ev1);
-    for (int q = 0; q < 2 && e == cudaSuccess; ++q) {
-        e = cudaStreamCreateWithFlags(&s->gs[q], cudaStreamNonBlocking);
+    for (int q = 0; q < 4 && e == cudaSuccess; ++q) e = cudaEventCreate(&s->ev[q]);
+    int plo = 0, phi = 0;
+    if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&plo, &phi);
+    for (int q = 0; q < 3 && e == cudaSuccess; ++q) {
+        e = cudaStreamCreateWithPriority(&s->gs[q], cudaStreamNonBlocking, phi);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->join[q], cudaEventDisableTiming);
     }
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming);
     const size_t n = D.n;
-    size_t fmax_ = 0;
-    for (int a = 0; a < 3; ++a) fmax_ = std::max(fmax_, (size_t)(nn[a] + 1) * (n / nn[a]));
     if (e == cudaSuccess) e = dalloc(s, &D.Q, NC * n);
     if (e == cudaSuccess) e = dalloc(s, &D.Qn, NC * n);
     if (e == cudaSuccess) e = dalloc(s, &D.C, NC * n);
     if (e == cudaSuccess) e = dalloc(s, &D.Cn, NC * n);
-    if (e == cudaSuccess) e = dalloc(s, &D.F, NC * fmax_);
-    if (e == cudaSuccess) e = dalloc(s, &D.E, 2 * NC * n);
-    if (e == cudaSuccess) e = dalloc(s, &D.upd, n);
     if (e == cudaSuccess) e = dalloc(s, &D.err, 1);
     if (e == cudaSuccess) e = dalloc(s, &D.wall, NC);
     if (e == cudaSuccess) e = dalloc(s, &D.seeds, mb3::SEEDCAP + mb3::NODECAP);
@@ -1558,12 +1821,11 @@ mb_status mb3_create(const mb3_grid *g, double gamma, double cfl, const mb3_body
 void mb3_destroy(mb3_sim *s) {
     if (!s) return;
     if (s->st) cudaStreamSynchronize(s->st);
-    for (int q = 0; q < 2; ++q) if (s->gs[q]) cudaStreamSynchronize(s->gs[q]);
+    for (int q = 0; q < 3; ++q) if (s->gs[q]) cudaStreamSynchronize(s->gs[q]);
     for (void *p : s->owned) cudaFree(p);
-    if (s->ev0) cudaEventDestroy(s->ev0);
-    if (s->ev1) cudaEventDestroy(s->ev1);
+    for (int q = 0; q < 4; ++q) if (s->ev[q]) cudaEventDestroy(s->ev[q]);
     if (s->fork) cudaEventDestroy(s->fork);
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < 3; ++q) {
         if (s->join[q]) cudaEventDestroy(s->join[q]);
         if (s->gs[q]) cudaStreamDestroy(s->gs[q]);
     }
@@ -1623,14 +1885,49 @@ mb_status mb3_read_state(mb3_sim *s, double *Q, double *alpha, double *clock) {
     return err_status(s, w);
 }
 
+// the line kernels of a sweep along D.d: over all but the near cells, or over
+// those (near)
+extern "C++" {
+template <typename T>
+static void line_sweep_t(const Desc &D, bool near, cudaStream_t st) {
+    const int nal = D.d == 0 ? D.nx : D.d == 1 ? D.ny : D.nz;
+    if (near) {
+        const mb3::Near N = mb3::near_range(D, D.d, nal);
+        if (N.len == 0) return;
+        const long long cells = (long long)N.len * D.rn[0] * D.rn[1] * D.rn[2] / D.rn[D.d];
+        const long long slots = (long long)(N.len + 2) * D.rn[1] * D.rn[2];
+        if (D.d == 0) mb3::k3_near_row<T><<<nblk((slots + 29) / 30 * 32, 128), 128, 0, st>>>(D, N);
+        else if (D.d == 1) mb3::k3_near<T, 1><<<nblk(cells, 128), 128, 0, st>>>(D, N);
+        else mb3::k3_near<T, 2><<<nblk(cells, 128), 128, 0, st>>>(D, N);
+        return;
+    }
+    if (D.d == 0) {
+        const long long slots = (long long)(D.nx + 2) * D.ny * D.nz;
+        mb3::k3_row<T><<<nblk((slots + 29) / 30 * 32, 128), 128, 0, st>>>(D);
+        return;
+    }
+    // cells per thread: a segment costs two evolved states and a flux more
+    // than its cells, so as long as leaves 32 warps per SM (8 per quarter,
+    // each with its share of the FP64 pipe), from 64 down to 8, in CTAs of one
+    // warp.  200 x 200 x 100 cells, FP64: 1.51 ms with 16 warps per SM
+    const unsigned nlb = nblk(D.n / nal, 32);
+    int seg = 64;
+    while (seg > 8 && (long long)nlb * ((nal + seg - 1) / seg) < 152 * 32) seg /= 2;
+    const int nseg = (nal + seg - 1) / seg;
+    seg = (nal + nseg - 1) / nseg;
+    if (D.d == 1) mb3::k3_march<T, 1><<<nlb * (unsigned)nseg, 32, 0, st>>>(D, seg, nlb);
+    else mb3::k3_march<T, 2><<<nlb * (unsigned)nseg, 32, 0, st>>>(D, seg, nlb);
+}
+static void line_sweep(const Desc &D, bool near, cudaStream_t st) {
+    if (D.f32) line_sweep_t<float>(D, near, st);
+    else line_sweep_t<double>(D, near, st);
+}
+}
+
 mb_status mb3_sweep(mb3_sim *s, int d, double dt) {
     if (!s || d < 0 || d > 2 || !(dt > 0.0)) return MB_E_INVAL;
     if (s->sidx > 0 && dt != s->dt_step) return fail3(s, MB_E_STATE, "the sweeps of a step must share dt");
     cudaError_t e = cudaSuccess;
-    if (s->sidx == 0) {
-        s->dt_step = dt;
-        e = cudaMemcpyAsync(s->D.Qn, s->D.Q, NC * (size_t)s->D.n * sizeof(double), cudaMemcpyDeviceToDevice, s->st);
-    }
     const double delta = s->D.U[d] * dt;
     double TA[3] = {s->T[0], s->T[1], s->T[2]}, TM[3] = {TA[0], TA[1], TA[2]}, TB[3] = {TA[0], TA[1], TA[2]};
     TB[d] += delta;
@@ -1650,15 +1947,15 @@ mb_status mb3_sweep(mb3_sim *s, int d, double dt) {
         for (int a = 0; a < 3; ++a) { s->D.p0[a] = s->q0[a]; s->D.pn[a] = s->qn[a]; }
     }
     s->prev_ok = false;
+    // three state buffers rotate: the step-start state stays in its own (Qn),
+    // each sweep writes the new state into the free one (Cn)
+    if (s->sidx == 0) s->dt_step = dt;
     Desc D = s->D;
+    if (s->sidx == 0) D.Qn = D.Q;
     for (int a = 0; a < 3; ++a) { D.r0[a] = r0[a]; D.rn[a] = rn[a]; }
     D.d = d;
     D.lam = dt / D.h[d];
     D.hlamf = 0.5f * (float)D.lam;
-    const int nn[3] = {D.nx, D.ny, D.nz};
-    const int nal = nn[d], nlines = D.n / nal;
-    const bool periodic = D.bc[2 * d] == MB_BC_PERIODIC;
-    const int nfl = periodic ? nal : nal + 1;
     if (e == cudaSuccess) e = cudaMemsetAsync(D.wall, 0, NC * sizeof(double), s->st);
     if (e == cudaSuccess) e = cudaMemsetAsync(D.nseed, 0, sizeof(int), s->st);
     if (e == cudaSuccess) e = cudaMemsetAsync(D.mixed, 0, sizeof(int), s->st);
@@ -1667,48 +1964,49 @@ mb_status mb3_sweep(mb3_sim *s, int d, double dt) {
     if (rc > 0) {
         // the three geometry kernels are independent (each writes its own
         // arrays); the cut cells near a body's corners make each of them a
-        // long tail on few SMs, so they run side by side on three streams
+        // long tail on few SMs, so they run side by side on three streams,
+        // and beside the cells that need no body data
         cudaEventRecord(s->fork, s->st);
-        cudaStreamWaitEvent(s->gs[0], s->fork, 0);
-        cudaStreamWaitEvent(s->gs[1], s->fork, 0);
-        mb3::k3_cells<<<nblk(32LL * (reuse ? 2 : 3) * (long long)rc), 256, 0, s->st>>>(
+        for (int q = 0; q < 3; ++q) cudaStreamWaitEvent(s->gs[q], s->fork, 0);
+        mb3::k3_cells<<<nblk(32LL * (reuse ? 2 : 3) * (long long)rc), 256, 0, s->gs[0]>>>(
             D, BA, BM, BB, reuse ? mb3::CELLS_REUSE_A : mb3::CELLS_ALL);
         long long nfaces = 0;
         for (int a = 0; a < 4; ++a) {
             const int ax = a < 3 ? a : d;
             nfaces += (long long)(rn[0] + (ax == 0)) * (rn[1] + (ax == 1)) * (rn[2] + (ax == 2));
         }
-        mb3::k3_faces<<<nblk(nfaces), 256, 0, s->gs[0]>>>(D, BM, BA, delta);
+        mb3::k3_faces<<<nblk(nfaces), 256, 0, s->gs[1]>>>(D, BM, BA, delta);
         if (delta != 0.0) {
             const long long nsw = (long long)(rn[0] + (d == 0)) * (rn[1] + (d == 1)) * (rn[2] + (d == 2));
-            mb3::k3_swept<<<nblk(32LL * nsw), 256, 0, s->gs[1]>>>(D, BA, delta);
+            mb3::k3_swept<<<nblk(32LL * nsw), 256, 0, s->gs[2]>>>(D, BA, delta);
         }
-        for (int q = 0; q < 2; ++q) {
+        for (int q = 1; q < 3; ++q) {
             cudaEventRecord(s->join[q], s->gs[q]);
-            cudaStreamWaitEvent(s->st, s->join[q], 0);
+            cudaStreamWaitEvent(s->gs[0], s->join[q], 0);
         }
-        mb3::k3_wall<<<nblk((long long)rc), 256, 0, s->st>>>(D);
+        mb3::k3_wall<<<nblk((long long)rc), 256, 0, s->gs[0]>>>(D);
+        cudaEventRecord(s->join[0], s->gs[0]);
     }
-    const bool f = D.f32;
-    const auto evolve = d == 0 ? (f ? mb3::k3_evolve<0, float> : mb3::k3_evolve<0, double>)
-                      : d == 1 ? (f ? mb3::k3_evolve<1, float> : mb3::k3_evolve<1, double>)
-                               : (f ? mb3::k3_evolve<2, float> : mb3::k3_evolve<2, double>);
-    const auto flux = d == 0 ? (f ? mb3::k3_flux<0, float> : mb3::k3_flux<0, double>)
-                    : d == 1 ? (f ? mb3::k3_flux<1, float> : mb3::k3_flux<1, double>)
-                             : (f ? mb3::k3_flux<2, float> : mb3::k3_flux<2, double>);
-    const auto update = d == 0 ? mb3::k3_update<0> : d == 1 ? mb3::k3_update<1> : mb3::k3_update<2>;
-    evolve<<<nblk(D.n), 256, 0, s->st>>>(D, nal);
-    cudaEventRecord(s->ev0, s->st);
-    flux<<<nblk((long long)nfl * nlines), 256, 0, s->st>>>(D, nal, nfl, nlines);
-    cudaEventRecord(s->ev1, s->st);
-    update<<<nblk(D.n), 256, 0, s->st>>>(D, nal, nfl);
+    cudaEventRecord(s->ev[0], s->st);
+    line_sweep(D, false, s->st);
+    cudaEventRecord(s->ev[1], s->st);
     if (rc > 0) {
+        cudaStreamWaitEvent(s->st, s->join[0], 0);
+        cudaEventRecord(s->ev[2], s->st);
+        line_sweep(D, true, s->st);
+        cudaEventRecord(s->ev[3], s->st);
         mb3::k3_evprep<<<nblk((long long)rc), 256, 0, s->st>>>(D);
         mb3::k3_events<<<nblk((long long)rc), 256, 0, s->st>>>(D);
+        mb3::k3_bad<<<nblk((long long)rc), 256, 0, s->st>>>(D);
     }
-    if (rc > 0) mb3::k3_bad<<<nblk((long long)rc), 256, 0, s->st>>>(D);
     mb3::k3_mix<<<1, mb3::MIXS_THREADS, 0, s->st>>>(D);
-    mb3::k3_final<<<nblk(D.n), 256, 0, s->st>>>(D);
+    if (rc > 0) mb3::k3_final<<<nblk((long long)rc), 256, 0, s->st>>>(D);
+    // the new state's buffer becomes the state's; the next sweep writes into
+    // the one left over
+    s->D.Cn = s->sidx == 0 ? s->D.Qn : D.Q;
+    s->D.Qn = D.Qn;
+    s->D.Q = D.Cn;
+    std::swap(s->D.Qf, s->D.Qfn);
     int w = 0;
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(s->wall_host, D.wall, NC * sizeof(double), cudaMemcpyDeviceToHost, s->st);
@@ -1718,7 +2016,10 @@ mb_status mb3_sweep(mb3_sim *s, int d, double dt) {
     if (e != cudaSuccess) return cuda3(s, e, "mb3_sweep");
     s->prev_ok = true;
     for (int a = 0; a < 3; ++a) { s->q0[a] = r0[a]; s->qn[a] = rn[a]; }
-    cudaEventElapsedTime(&s->flux_ms, s->ev0, s->ev1);
+    float near_ms = 0.0f;
+    cudaEventElapsedTime(&s->flux_ms, s->ev[0], s->ev[1]);
+    if (rc > 0) cudaEventElapsedTime(&near_ms, s->ev[2], s->ev[3]);
+    s->flux_ms += near_ms;
     s->T[d] = TB[d];
     if (++s->sidx == 3) {
         s->sidx = 0;
@@ -1733,8 +2034,9 @@ mb_status mb3_cfl_dt(mb3_sim *s, double *dt) {
     double sm[3] = {0, 0, 0};
     cudaError_t e = cudaMemsetAsync(s->D.smax, 0, 3 * sizeof(double), s->st);
     const unsigned nb = std::min(nblk(s->D.n), 152u * 8u);
-    if (e == cudaSuccess && s->D.f32) mb3::k3_speeds<float><<<nb, 256, 0, s->st>>>(s->D);
-    else if (e == cudaSuccess) mb3::k3_speeds<double><<<nb, 256, 0, s->st>>>(s->D);
+    if (e == cudaSuccess && s->D.f32) mb3::k3_speeds32<<<nb, 256, 0, s->st>>>(s->D);
+    else if (e == cudaSuccess)
+        mb3::k3_speeds64<<<std::min(nblk(s->D.n, 256 * mb3::SPEED_CELLS), 152u * 8u), 256, 0, s->st>>>(s->D);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpyAsync(sm, s->D.smax, 3 * sizeof(double), cudaMemcpyDeviceToHost, s->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
@@ -1780,6 +2082,7 @@ mb_status mb3_set_precision(mb3_sim *s, int precision) {
     if (s->sidx != 0) return fail3(s, MB_E_STATE, "mb3_set_precision in the middle of a step");
     cudaError_t e = cudaSuccess;
     if (precision == MB_FP32 && !s->D.Qf) e = dalloc(s, &s->D.Qf, NC * (size_t)s->D.n);
+    if (e == cudaSuccess && precision == MB_FP32 && !s->D.Qfn) e = dalloc(s, &s->D.Qfn, NC * (size_t)s->D.n);
     if (e != cudaSuccess) return cuda3(s, e, "mb3_set_precision");
     s->D.f32 = precision == MB_FP32;
     if (s->D.f32) mb3::k3_to_f32<<<nblk(s->D.n), 256, 0, s->st>>>(s->D);

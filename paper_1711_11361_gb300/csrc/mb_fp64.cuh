@@ -76,13 +76,143 @@ __device__ __forceinline__ double max64(double a, double b) { return key64(a) < 
 __device__ __forceinline__ double abs64(double x) {
     return __hiloint2double(__double2hiint(x) & 0x7fffffff, __double2loint(x));
 }
-__device__ __forceinline__ double neg64(double x) {
-    return __hiloint2double(__double2hiint(x) ^ (int)0x80000000, __double2loint(x));
+// x rounded to float (to nearest, ties to even) by integer instructions where
+// the result is a normal float or zero, else by the conversion
+__device__ __forceinline__ float narrow32(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned m = hi & 0x7fffffffu;
+    if (m - 0x38100000u < 0x0fd00000u) {   // exponent field 897 .. 1149
+        const unsigned long long r = ((unsigned long long)(m - 0x38000000u) << 32 | lo) + 0x0fffffffull +
+                                     ((lo >> 29) & 1u);
+        return __uint_as_float((unsigned)(r >> 29) | (hi & 0x80000000u));
+    }
+    if ((m | lo) == 0u) return __uint_as_float(hi);
+    return (float)x;
 }
-// x / 2 and 2 x of normal numbers by the exponent field (0 stays 0)
-__device__ __forceinline__ double twice64(double x) {
-    const int hi = __double2hiint(x);
-    return (hi & 0x7ff00000) ? __hiloint2double(hi + 0x100000, __double2loint(x)) : x + x;
+// a float that is x to 2^-22 where *ok stays true (tiny values become 0)
+__device__ __forceinline__ float near32(double x, bool &ok) {
+    const unsigned hi = (unsigned)__double2hiint(x), m = hi & 0x7fffffffu;
+    ok = ok && m < 0x47e00000u;
+    const unsigned f = __funnelshift_l((unsigned)__double2loint(x), m - 0x38000000u, 3);
+    return m < 0x38100000u ? 0.0f : __uint_as_float(f | (hi & 0x80000000u));
+}
+
+// ---------------------------------------------------------------------------
+// FP64 Euler arithmetic, conserved variables q[NC] = rho, momenta, E; D: the
+// momentum normal to the faces
+// ---------------------------------------------------------------------------
+// a face's side: state, 1/rho and pressure
+template <int NC>
+struct Side { double q[NC], ir, p; };
+template <int NC>
+__device__ __forceinline__ double msq64(const double *q) {   // |m|^2
+    double s = q[NC - 2] * q[NC - 2];
+#pragma unroll
+    for (int k = NC - 3; k >= 1; --k) s = __fma_rn(q[k], q[k], s);
+    return s;
+}
+template <int NC>
+__device__ __forceinline__ double press64(double g1, const double *q, double ir) {
+    return g1 * __fma_rn(-0.5 * msq64<NC>(q), ir, q[NC - 1]);
+}
+// rho > 0 and 2 rho E > |m|^2, in FP32 where that decides with a margin of
+// 1e-5 (its error is below 2e-6), else in FP64
+template <int NC>
+__device__ __forceinline__ bool physical64(const double *q) {
+    bool ok = true;
+    const float r = near32(q[0], ok), E = near32(q[NC - 1], ok);
+    float m2 = 0.0f;
+#pragma unroll
+    for (int k = 1; k < NC - 1; ++k) {
+        const float m = near32(q[k], ok);
+        m2 = fmaf(m, m, m2);
+    }
+    const float t = 2.0f * r * E;
+    if (ok && r > 0.0f && E > 0.0f && t < 1e38f && t - m2 > 1e-5f * t) return true;
+    return pos64(q[0]) && 2.0 * q[0] * q[NC - 1] > msq64<NC>(q) && q[NC - 1] - q[NC - 1] == 0.0;
+}
+// MUSCL-Hancock evolved states of one cell: van Leer slopes in conserved
+// variables (none where !lim), half-step evolution (hl = dt / 2h), first order
+// where an evolved state is not physical.  One reciprocal of the product of
+// two densities serves both sides; the positivity tests use the pressures
+// that the Riemann solver takes.
+template <int NC, int D>
+__device__ __forceinline__ void evolve64(double g1, double hl, const double *qm, const double *q0, const double *qp,
+                                         bool lim, Side<NC> &L, Side<NC> &R) {
+    constexpr int in = 1 + D, E = NC - 1;
+    double l[NC], r[NC];
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        // half the slope: dm dp / (dm + dp)
+        const double dm = q0[k] - qm[k], dp = qp[k] - q0[k];
+        double pr = dm * dp, y = 0.0;
+        if (lim && pos64(pr)) y = rcp64(dm + dp);
+        else pr = 0.0;
+        l[k] = __fma_rn(-pr, y, q0[k]);
+        r[k] = __fma_rn(pr, y, q0[k]);
+    }
+    double rr = rcp64(l[0] * r[0]);
+    const double il = r[0] * rr, ig = l[0] * rr;
+    const double pl = press64<NC>(g1, l, il), pg = press64<NC>(g1, r, ig);
+    const double ul = l[in] * il, ug = r[in] * ig;
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        double df;   // flux of the low side less that of the high side
+        if (k == 0) df = l[in] - r[in];
+        else if (k == in) df = __fma_rn(l[in], ul, pl) - __fma_rn(r[in], ug, pg);
+        else if (k == E) df = __fma_rn(ul, l[E] + pl, -(ug * (r[E] + pg)));
+        else df = __fma_rn(l[k], ul, -(r[k] * ug));
+        L.q[k] = __fma_rn(hl, df, l[k]);
+        R.q[k] = __fma_rn(hl, df, r[k]);
+    }
+    rr = rcp64(L.q[0] * R.q[0]);
+    L.ir = R.q[0] * rr;
+    R.ir = L.q[0] * rr;
+    L.p = press64<NC>(g1, L.q, L.ir);
+    R.p = press64<NC>(g1, R.q, R.ir);
+    if (!(pos64(L.q[0]) && pos64(R.q[0]) && pos64(L.p) && pos64(R.p))) {
+#pragma unroll
+        for (int k = 0; k < NC; ++k) L.q[k] = R.q[k] = q0[k];
+        L.ir = R.ir = rcp64(q0[0]);
+        L.p = R.p = press64<NC>(g1, q0, L.ir);
+    }
+}
+// HLLC flux with Davis wave speeds (Toro, ch. 10), the star flux in the form
+// [S* (S Q - F) + S p* (0, n, S*)] / (S - S*) with p* = p + rho (S - u)(S* - u)
+// of the side that holds the face
+template <int NC, int D>
+__device__ __forceinline__ void hllc64(double g, const Side<NC> &L, const Side<NC> &R, double *F) {
+    constexpr int in = 1 + D, E = NC - 1;
+    const double uL = L.q[in] * L.ir, uR = R.q[in] * R.ir;
+    const double cL = sqrt64(g * (L.p * L.ir)), cR = sqrt64(g * (R.p * R.ir));
+    const double SL = min64(uL - cL, uR - cR), SR = max64(uL + cL, uR + cR);
+    const bool supL = nonneg64(SL), supR = !pos64(SR);
+    if (supL || supR) {
+        const double u = supL ? uL : uR, p = supL ? L.p : R.p;
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            const double q = supL ? L.q[k] : R.q[k], m = supL ? L.q[in] : R.q[in];
+            F[k] = k == 0 ? m : k == in ? __fma_rn(q, u, p) : k == E ? u * (q + p) : q * u;
+        }
+        return;
+    }
+    const double vL = SL - uL, vR = SR - uR;
+    const double aL = L.q[0] * vL, aR = R.q[0] * vR;
+    const double num = __fma_rn(uL, aL, __fma_rn(-uR, aR, R.p - L.p));
+    const double Ss = num * rcp64(aL - aR);
+    const bool left = nonneg64(Ss);
+    const double S = left ? SL : SR, u = left ? uL : uR, v = left ? vL : vR, a = left ? aL : aR;
+    const double p = left ? L.p : R.p;
+    const double k1 = rcp64(S - Ss), kS = k1 * Ss;
+    const double Sp = S * __fma_rn(a, Ss - u, p);
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        const double q = left ? L.q[k] : R.q[k];
+        if (k == 0) F[k] = a * kS;
+        else if (k == in) F[k] = __fma_rn(kS, __fma_rn(q, v, -p), k1 * Sp);
+        else if (k == E) F[k] = kS * (__fma_rn(q, v, -(u * p)) + Sp);
+        else F[k] = q * v * kS;
+    }
 }
 
 }  // namespace mbfp

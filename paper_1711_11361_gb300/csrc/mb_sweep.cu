@@ -401,92 +401,6 @@ __global__ void k_band_prep_o(const InstDesc *__restrict__ D, InstDyn *__restric
 }
 
 // ---------------------------------------------------------------------------
-// FP64 Euler flow arithmetic of the band faces and the scalar bulk kernels
-// ---------------------------------------------------------------------------
-// a face's side: state, 1/rho and pressure
-struct S64 { double q[4], ir, p; };
-__device__ __forceinline__ double press64(double g1, const double *q, double ir) {
-    const double m2 = __fma_rn(q[1], q[1], q[2] * q[2]);
-    return g1 * __fma_rn(-0.5 * m2, ir, q[3]);
-}
-// MUSCL-Hancock evolved states of one cell (the function evolve above; one
-// reciprocal of the product of two densities serves both sides, and the
-// positivity tests use the pressures the Riemann solver takes)
-template <int D>
-__device__ __forceinline__ void evolve64(double g1, double hl, const double *qm, const double *q0, const double *qp,
-                                         bool lim, S64 &L, S64 &R) {
-    constexpr int in = 1 + D, it = 2 - D;
-    double l[4], r[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const double dm = q0[k] - qm[k], dp = qp[k] - q0[k], pr = dm * dp;
-        double h = 0.0;   // half the van Leer slope
-        if (lim && pos64(pr)) h = pr * rcp64(dm + dp);
-        l[k] = q0[k] - h;
-        r[k] = q0[k] + h;
-    }
-    double rr = rcp64(l[0] * r[0]);
-    const double il = r[0] * rr, ig = l[0] * rr;
-    const double pl = press64(g1, l, il), pg = press64(g1, r, ig);
-    const double ul = l[in] * il, ug = r[in] * ig;
-    double df[4];
-    df[0] = l[in] - r[in];
-    df[in] = __fma_rn(l[in], ul, pl) - __fma_rn(r[in], ug, pg);
-    df[it] = l[it] * ul - r[it] * ug;
-    df[3] = ul * (l[3] + pl) - ug * (r[3] + pg);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        L.q[k] = __fma_rn(hl, df[k], l[k]);
-        R.q[k] = __fma_rn(hl, df[k], r[k]);
-    }
-    rr = rcp64(L.q[0] * R.q[0]);
-    L.ir = R.q[0] * rr;
-    R.ir = L.q[0] * rr;
-    L.p = press64(g1, L.q, L.ir);
-    R.p = press64(g1, R.q, R.ir);
-    if (!(pos64(L.q[0]) && pos64(R.q[0]) && pos64(L.p) && pos64(R.p))) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) L.q[k] = R.q[k] = q0[k];
-        L.ir = R.ir = rcp64(q0[0]);
-        L.p = R.p = press64(g1, q0, L.ir);
-    }
-}
-// HLLC flux (the function hllc above), the star flux in the form
-// [S* (S Q - F) + S p* (0, n, S*)] / (S - S*) with p* = p + rho (S - u)(S* - u)
-// of the side that holds the face (Toro, ch. 10)
-template <int D>
-__device__ __forceinline__ void hllc64(double g, const S64 &L, const S64 &R, double *F) {
-    constexpr int in = 1 + D, it = 2 - D;
-    const double uL = L.q[in] * L.ir, uR = R.q[in] * R.ir;
-    const double cL = sqrt64(g * (L.p * L.ir)), cR = sqrt64(g * (R.p * R.ir));
-    const double SL = min64(uL - cL, uR - cR), SR = max64(uL + cL, uR + cR);
-    const bool supL = nonneg64(SL), supR = !pos64(SR);
-    if (supL || supR) {
-        const S64 &s = supL ? L : R;
-        const double u = supL ? uL : uR;
-        F[0] = s.q[in];
-        F[in] = __fma_rn(s.q[in], u, s.p);
-        F[it] = s.q[it] * u;
-        F[3] = u * (s.q[3] + s.p);
-        return;
-    }
-    const double vL = SL - uL, vR = SR - uR;
-    const double aL = L.q[0] * vL, aR = R.q[0] * vR;
-    const double num = __fma_rn(uL, aL, __fma_rn(-uR, aR, R.p - L.p));
-    const double Ss = num * rcp64(aL - aR);
-    const bool left = nonneg64(Ss);
-    const double S = left ? SL : SR, u = left ? uL : uR, v = left ? vL : vR, a = left ? aL : aR;
-    const double p = left ? L.p : R.p;
-    const double mn = left ? L.q[in] : R.q[in], mt = left ? L.q[it] : R.q[it], E = left ? L.q[3] : R.q[3];
-    const double k = rcp64(S - Ss), kS = k * Ss;
-    const double Sp = S * __fma_rn(a, Ss - u, p);
-    F[0] = a * kS;
-    F[in] = __fma_rn(kS, __fma_rn(mn, v, -p), k * Sp);
-    F[it] = mt * v * kS;
-    F[3] = kS * (__fma_rn(E, v, -(u * p)) + Sp);
-}
-
-// ---------------------------------------------------------------------------
 // stabilised flux of one face: aperture times F2D (eqs. Klein2shieldedFluxMethod2
 // and Klein2DtotalfluxaMethod2 with the one- or two-sided shielded parts).
 // Not inlined, so that a face shared by two band cells gets identical bits.
@@ -508,11 +422,11 @@ __device__ __noinline__ void face_stab(int eq, T g, int dir, T lamT, T av0, T av
     if (sizeof(T) == 8 && eq == 0) {
         auto fluxes = [&](auto dc) {
             constexpr int DC = decltype(dc)::value;
-            S64 x, a, b;
+            Side<4> x, a, b;
             const double g1 = (double)g - 1.0, hl = 0.5 * (double)lamT;
-            evolve64<DC>(g1, hl, (const double *)w[0].q, (const double *)w[1].q, (const double *)w[2].q, limA, x, a);
-            evolve64<DC>(g1, hl, (const double *)w[1].q, (const double *)w[2].q, (const double *)w[3].q, limB, b, x);
-            hllc64<DC>((double)g, a, b, (double *)F);
+            evolve64<4, DC>(g1, hl, (const double *)w[0].q, (const double *)w[1].q, (const double *)w[2].q, limA, x, a);
+            evolve64<4, DC>(g1, hl, (const double *)w[1].q, (const double *)w[2].q, (const double *)w[3].q, limB, b, x);
+            hllc64<4, DC>((double)g, a, b, (double *)F);
         };
         if (dir == 0) fluxes(std::integral_constant<int, 0>());
         else fluxes(std::integral_constant<int, 1>());
@@ -710,19 +624,19 @@ struct Flow {                     // advection
 template <>
 struct Flow<double, 0> {          // Euler, FP64
     static constexpr int NC = 4;
-    using S = S64;
+    using S = Side<4>;
     double g, g1, lam, hl;
     __device__ __forceinline__ Flow(const InstDesc &I, double l, int)
         : g(I.gamma), g1(I.gamma - 1.0), lam(l), hl(0.5 * l) {}
     template <int D>
     __device__ __forceinline__ void states(const double *qm, const double *q0, const double *qp, bool lim, S &L,
                                            S &R) const {
-        evolve64<D>(g1, hl, qm, q0, qp, lim, L, R);
+        evolve64<4, D>(g1, hl, qm, q0, qp, lim, L, R);
     }
     template <int D>
-    __device__ __forceinline__ void flux(const S &L, const S &R, double *F) const { hllc64<D>(g, L, R, F); }
+    __device__ __forceinline__ void flux(const S &L, const S &R, double *F) const { hllc64<4, D>(g, L, R, F); }
 };
-__device__ __forceinline__ void up_state(S64 &s) {
+__device__ __forceinline__ void up_state(Side<4> &s) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) s.q[k] = __shfl_up_sync(0xffffffffu, s.q[k], 1);
     s.ir = __shfl_up_sync(0xffffffffu, s.ir, 1);
@@ -738,19 +652,15 @@ __device__ __forceinline__ void new_state(const Flow<double, 0> &f, const double
                                           double &s1) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) qn[k] = __fma_rn(f.lam, Flo[k] - Fhi[k], q[k]);
-    // p > 0 as 2 rho E > |m|^2; on the step's last sweep from the pressure
-    const double m2 = __fma_rn(qn[1], qn[1], qn[2] * qn[2]);
-    bool ok = pos64(qn[0]);
     if (last) {
-        const double ir = rcp64(qn[0]), p = f.g1 * __fma_rn(-0.5 * m2, ir, qn[3]);
-        ok = ok && pos64(p);
+        const double ir = rcp64(qn[0]), p = press64<4>(f.g1, qn, ir);
+        if (!pos64(qn[0]) || !pos64(p)) list_bulk_bad(y, ci);
         const double c = sqrt64(f.g * (p * ir));
         s0 = __fma_rn(abs64(qn[1]), ir, c);
         s1 = __fma_rn(abs64(qn[2]), ir, c);
-    } else {
-        ok = ok && pos64(__fma_rn(twice64(qn[0]), qn[3], neg64(m2)));
+    } else if (!physical64<4>(qn)) {
+        list_bulk_bad(y, ci);
     }
-    if (!ok) list_bulk_bad(y, ci);
 }
 template <class T>
 __device__ __forceinline__ void new_state(const Flow<T, 1> &f, const T *q, const T *Flo, const T *Fhi, bool, int,
