@@ -963,8 +963,15 @@ __device__ __forceinline__ void evolve2(float g1, float lam, const float2 *qm, c
             QL.q[k] = sel2(okx, oky, QL.q[k], q0[k]);
             QR.q[k] = sel2(okx, oky, QR.q[k], q0[k]);
         }
-        prim2(g1, QL.q, QL.ir, QL.p);
-        prim2(g1, QR.q, QR.ir, QR.p);
+        // (a half that is fine keeps its bits, whatever the other half holds:
+        // past the grid's last column that is padding)
+        float2 ir, p;
+        prim2(g1, QL.q, ir, p);
+        QL.ir = sel2(okx, oky, QL.ir, ir);
+        QL.p = sel2(okx, oky, QL.p, p);
+        prim2(g1, QR.q, ir, p);
+        QR.ir = sel2(okx, oky, QR.ir, ir);
+        QR.p = sel2(okx, oky, QR.p, p);
     }
 }
 

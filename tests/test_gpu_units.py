@@ -55,7 +55,8 @@ def test_unit_edges(mb, nx, ny, bc, equation):
         assert r["cls"] == 0 and r["contents"] <= 1e-12, (d, r["contents"])
 
 
-@pytest.mark.parametrize("equation,precision", [(inputs.EULER, 0), (inputs.ADVECTION, 0), (inputs.ADVECTION, 1)])
+@pytest.mark.parametrize("equation,precision", [(inputs.EULER, 0), (inputs.EULER, 1), (inputs.ADVECTION, 0),
+                                                (inputs.ADVECTION, 1)])
 def test_far_units_beside_the_geometry(mb, equation, precision):
     probs = [_problem(nx, ny, bc, equation) for nx, ny in SIZES[1:] for bc in SIDES]
     out = []
