@@ -106,7 +106,7 @@ struct mb_sim {
     // budget and ring depth per direction of the FP32x2 kernels, rows per
     // thread of the y sweep
     int tune_cta[2] = {64 | SHAPE_MINB4 | SHAPE_RING8, 64 | SHAPE_MINB4};
-    int tune_yseg = 64;
+    int tune_yseg = 0;            // 0: chosen by relayout
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     int cur = 0;          // buffer holding the latest state (between steps)
@@ -314,7 +314,7 @@ static void describe_instance(int prec, int yseg, const mb_grid &g, double gamma
 // descriptor and device buffers of one instance
 static cudaError_t make_instance(mb_sim *s, const mb_grid &g, double gamma, const mb_body &b, const mb_motion &m,
                                  InstDesc &I, InstHost &h) {
-    describe_instance(s->prec, s->tune_yseg, g, gamma, b, m, I, h);
+    describe_instance(s->prec, 64, g, gamma, b, m, I, h);
     I.serial_bulk = s->overlap ? 0 : 1;
     const size_t esz = s->prec == MB_FP32 ? 4 : 8;
     const size_t cells = (size_t)I.pitch * g.ny;
@@ -343,6 +343,22 @@ static size_t instance_bytes(const InstDesc &I, int prec) {
            (size_t)I.nx * I.ny * I.nc * 8;
 }
 
+// rows per thread of the FP32 Euler y sweep: 64, halved down to 8 while the
+// batch's units leave fewer than 16 warps per SM.  A unit's first rows (ring
+// fill, two rows of stencil) cost about as much as six of its own, so large
+// batches keep 64 (28.7 M cells: 32 measured slower).  400 x 400 cells: 91 us
+// per sweep with 64 rows (25 CTAs), 21 with 8; 1024 x 1024: 83 -> 19
+static int auto_yseg(const mb_sim *s) {
+    int seg = 64;
+    auto units = [&](int g) {
+        long long u = 0;
+        for (const auto &I : s->hd) u += (long long)I.tiles_x[1] * ((I.ny + g - 1) / g);
+        return u;
+    };
+    while (seg > 8 && units(seg) < 16LL * s->nsm) seg /= 2;
+    return seg;
+}
+
 // offsets of every instance in the shared arrays, those arrays, the
 // descriptors and the instance of every geometry group; the dynamic state of
 // new instance k is the old instance from[k]'s (zero when from[k] < 0).  The
@@ -362,6 +378,8 @@ static cudaError_t relayout(mb_sim *s, int old_n, const std::vector<int> &from) 
     std::vector<int> hnext;
     int rec_total = 0, tiles0 = 0, tiles1 = 0;
     size_t max_cells = 1;
+    const int yseg = s->tune_yseg ? s->tune_yseg : auto_yseg(s);
+    for (auto &I : s->hd) bulk_items(s->prec, yseg, I);
     for (int k = 0; k < n; ++k) {
         InstDesc &I = s->hd[k];
         const InstHost &h = s->ih[k];
@@ -1099,7 +1117,6 @@ mb_status mb_merge_count(mb_sim *sim, int inst, long long *cells) {
 static cudaError_t set_yseg(mb_sim *s, int yseg) {
     if (yseg == s->tune_yseg) return cudaSuccess;
     s->tune_yseg = yseg;
-    for (auto &I : s->hd) bulk_items(s->prec, yseg, I);
     std::vector<int> from(s->n);
     for (int k = 0; k < s->n; ++k) from[k] = k;
     return relayout(s, s->n, from);
@@ -1156,7 +1173,7 @@ mb_status mb_autotune(mb_sim *sim, double *report) {
     }
     const int ysegs[3] = {32, 64, 128};
     double best_x = 1e30, best_y = 1e30;
-    int bx = sim->tune_cta[0], by = sim->tune_cta[1], bs = sim->tune_yseg;
+    int bx = sim->tune_cta[0], by = sim->tune_cta[1], bs = sim->tune_yseg ? sim->tune_yseg : 64;
     for (int shape : xs) {
         double t = time_bulk(0, shape);
         if (t < best_x) { best_x = t; bx = shape; }

@@ -1345,8 +1345,11 @@ __global__ void __launch_bounds__(128, MINB) k_bulk_x_p(const InstDesc *__restri
     const int inst = find_inst_warp(D, n_inst, gw, 0);
     const InstDesc &I = D[inst];
     InstDyn &y = Y[inst];
-    if ((MODE == 0) == (y.defer_all != 0)) return;
     const int j = gw - I.tile_off[0];
+    // a row outside the body's extent over the sweep's poses needs no band
+    // data, also around a rotating body
+    const bool far = !I.serial_bulk && I.bc[0] != 2 && (j < y.row0 || j > y.row1);
+    if (MODE == 0 ? y.defer_all && !far : !y.defer_all || far) return;
     const int n = I.nx;
     const int c_last = (n + 1) >> 6;   // chunk holding face n
     const float lam = y.lamf;
@@ -1356,8 +1359,7 @@ __global__ void __launch_bounds__(128, MINB) k_bulk_x_p(const InstDesc *__restri
     const float *__restrict__ Q = (const float *)I.Q[src] + rowb;
     float *__restrict__ Qb = (float *)I.Q[dst];
     float *__restrict__ Qo = Qb + rowb;
-    if (MODE == 0 && I.bc[0] != 2 && (j < y.row0 || j > y.row1)) {
-        // a row outside the body's extent: plain throughout
+    if (MODE == 0 && far) {   // plain throughout
         float s0 = 0.0f, s1 = 0.0f;
         bulk_x_far<XC>(I, y, rg, Q, Qo, rowb, plane, lam, g, g1, last != 0, s0, s1);
         finish_warp<float>(y, last != 0, s0, s1);
@@ -1757,7 +1759,6 @@ __global__ void __launch_bounds__(128, MINB) k_bulk_y_p(const InstDesc *__restri
     const int inst = find_inst_warp(D, n_inst, gw, 1);
     const InstDesc &I = D[inst];
     InstDyn &y = Y[inst];
-    if ((MODE == 0) == (y.defer_all != 0)) return;
     const int local = gw - I.tile_off[1];
     const int ncg = I.tiles_x[1];
     const int cg = local % ncg, sg = local / ncg;
@@ -1773,9 +1774,11 @@ __global__ void __launch_bounds__(128, MINB) k_bulk_y_p(const InstDesc *__restri
     const float *__restrict__ Q = (const float *)I.Q[src];
     float *__restrict__ Qo = (float *)I.Q[dst];
     const int bclo = I.bc[2], bchi = I.bc[3];
-    if (MODE == 0 && bclo != 2 && !(col0 <= y.col1 && col0 + YCOLS_P - 1 >= y.col0 && j1 + 3 >= y.row0 &&
-                                    j0 - 3 <= y.row1)) {
-        // a tile the body cannot reach: plain throughout
+    // a tile the body cannot reach
+    const bool far = !I.serial_bulk && bclo != 2 && !(col0 <= y.col1 && col0 + YCOLS_P - 1 >= y.col0 &&
+                                                      j1 + 3 >= y.row0 && j0 - 3 <= y.row1);
+    if (MODE == 0 ? y.defer_all && !far : !y.defer_all || far) return;
+    if (MODE == 0 && far) {   // plain throughout
         float s0 = 0.0f, s1 = 0.0f;
         bulk_y_far(I, y, rg, Q, Qo, i, st0, j0, j1, plane, lam, g, g1, last != 0, s0, s1);
         finish_warp<float>(y, last != 0, s0, s1);
