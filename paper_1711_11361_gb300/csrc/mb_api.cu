@@ -27,7 +27,7 @@ void launch_nodes(const InstDesc *, int, cudaStream_t);
 void launch_pose(const InstDesc *, InstDyn *, const double *, const double *, const unsigned char *, const int *,
                  double *, double *, float *, int, int, int, int, double, int *, cudaStream_t);
 void launch_geom(const InstDesc *, InstDyn *, const int *, const double *, const double *, const float *, const int *,
-                 const unsigned char *, int, int, int, int, BandRec *, double *, cudaStream_t);
+                 const unsigned char *, int, int, int, int, int, BandRec *, double *, cudaStream_t);
 void launch_classify(const InstDesc *, InstDyn *, const double *, const double *, const unsigned char *, double *,
                      double *, float *, const int *, int, int, int, int, double *, cudaStream_t);
 template <class T>
@@ -88,6 +88,7 @@ struct mb_sim {
     const double **iop = nullptr; // batched state I/O: per-instance pointers into bstage
     size_t cap_iop = 0;
     int total_cols = 0;           // geometry groups
+    int gcw = GEO_GC;             // grid columns per geometry group
     int *ginst = nullptr;         // instance of each geometry group
     int total_tiles[2] = {0, 0};
     int bulk_grid[2] = {0, 0};
@@ -396,7 +397,22 @@ static cudaError_t relayout(mb_sim *s, int old_n, const std::vector<int> &from) 
         tiles1 += I.ntiles[1];
         max_cells = std::max(max_cells, (size_t)I.nx * I.ny);
     }
-    // geometry groups (GEO_GC columns, one CTA each): instances with more
+    // columns per geometry group: 2 where the groups run in one wave of three
+    // CTAs per SM, else 4, 8 or GEO_GC, the fewest that run in two.  A group's
+    // queries share its warps, so a narrow group is done sooner (400 x 400
+    // cylinder, per sweep of the whole step: 176 us with 16 columns, 142 with
+    // 8, 121 with 4, 117 with 2), while more groups repeat its gathering
+    // (940 x 376 tube: 243 us with 235 groups of 4, 247 with 470 of 2; 12 mixed
+    // grids: 16 requests in 94 ms with 16 columns, 88, 86, 93 with 8, 4, 2)
+    auto groups = [&](int w) {
+        long long g = 0;
+        for (const auto &I : s->hd) g += (I.gcol_max + w - 1) / w;
+        return g;
+    };
+    s->gcw = 2;
+    if (groups(2) > 3LL * s->nsm)
+        for (s->gcw = 4; s->gcw < GEO_GC && groups(s->gcw) > 6LL * s->nsm;) s->gcw *= 2;
+    // geometry groups (gcw columns, one CTA each): instances with more
     // polygon vertices first, so that the groups with the most cut cells start
     // in the first wave of CTAs
     std::vector<int> order(n), ginst;
@@ -406,7 +422,7 @@ static cudaError_t relayout(mb_sim *s, int old_n, const std::vector<int> &from) 
     for (int k : order) {
         InstDesc &I = s->hd[k];
         I.gcol_off = col_total;
-        const int ng = (I.gcol_max + GEO_GC - 1) / GEO_GC;
+        const int ng = (I.gcol_max + s->gcw - 1) / s->gcw;
         for (int q = 0; q < ng; ++q) ginst.push_back(k);
         col_total += ng;
     }
@@ -651,7 +667,7 @@ static mb_status do_sweep(mb_sim *s, int dir, double dt) {
     };
     auto geom_band = [&](cudaStream_t sx) {
         launch_geom(s->dd, s->dy, s->ginst, s->px, s->py, s->ebox, s->vnext, s->vmov, s->total_v, s->n, s->total_cols,
-                    dir, s->rec, s->bnd, sx);
+                    s->gcw, dir, s->rec, s->bnd, sx);
         band(0, sx);
         band(1, sx);
     };

@@ -13,6 +13,7 @@
 // line).  Only edges meeting R enter, so no far-away edge is ever integrated.
 #include "mb_internal.cuh"
 
+#include <cstddef>
 #include <cstring>
 #include <mutex>
 #include <string>
@@ -97,7 +98,8 @@ __global__ void k_pose(const InstDesc *__restrict__ D, InstDyn *__restrict__ Y, 
     InstDyn &y = Y[inst];
     __shared__ double sh[16];
     __shared__ int last_cta;
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 3) {   // a lane per pose (0: A, 1: M, 2: B)
+        const int P = threadIdx.x;
         double dt;
         if (sidx == 0) {
             if (dt_host > 0.0) {
@@ -114,56 +116,54 @@ __global__ void k_pose(const InstDesc *__restrict__ D, InstDyn *__restrict__ Y, 
         } else {
             dt = y.dt;
         }
-        const double tA = y.t + (sidx == 0 ? 0.0 : 0.5 * dt);
-        const double tB = y.t + (sidx == 0 ? 0.5 * dt : dt);
-        const double tM = y.t + (sidx == 0 ? 0.25 * dt : 0.75 * dt);
-        double thA = 0.0, thB = 0.0, thM = 0.0, Om = 0.0;
+        // times at 0, 1/4, 1/2 of the step in its first sweep, 1/2, 3/4, 1 in
+        // its second
+        const double t = y.t + (0.5 * sidx + 0.25 * P) * dt;
+        double th = 0.0, Om = 0.0, c = 1.0, s = 0.0;   // identity for a translating body
         if (I.rotating) {
-            thA = I.a0 + I.a1 * sin(I.omega * tA);
-            thB = I.a0 + I.a1 * sin(I.omega * tB);
-            thM = I.a0 + I.a1 * sin(I.omega * tM);
-            Om = I.a1 * I.omega * cos(I.omega * tM);
+            th = I.a0 + I.a1 * sin(I.omega * t);
+            if (P == 1) Om = I.a1 * I.omega * cos(I.omega * t);
+            sincos(th, &s, &c);
         }
         const double delta = I.U[dir] * dt;
-        double cA = 1.0, sA = 0.0, cB = 1.0, sB = 0.0, cM = 1.0, sM = 0.0;   // identity for a translating body
-        if (I.rotating) {
-            sincos(thA, &sA, &cA);
-            sincos(thB, &sB, &cB);
-            sincos(thM, &sM, &cM);
-        }
-        const double XA = y.X, YA = y.Y;
-        const double XB = dir == 0 ? y.X + delta : y.X, YB = dir == 1 ? y.Y + delta : y.Y;
-        const double XM = dir == 0 ? y.X + 0.5 * delta : y.X, YM = dir == 1 ? y.Y + 0.5 * delta : y.Y;
+        const double f = P == 0 ? 0.0 : P == 1 ? 0.5 * delta : delta;
+        const double X = dir == 0 && P ? y.X + f : y.X, Yp = dir == 1 && P ? y.Y + f : y.Y;
+        sh[2 * P] = X;
+        sh[2 * P + 1] = Yp;
+        sh[6 + 2 * P] = c;
+        sh[7 + 2 * P] = s;
         if (part == 0) {
-            if (sidx == 0) {
-                y.dt = dt;
+            if (P == 0) {
+                if (sidx == 0) {
+                    y.dt = dt;
+                } else {
+                    if (dt_host > 0.0 && dt_host != dt) y.err |= ERR_STATE;
+                    // the last sweep of the step gathers the wave speeds of the next step's dt
+                    y.S[0] = 0ull;
+                    y.S[1] = 0ull;
+                }
+                y.lam = dt / (dir == 0 ? I.dx : I.dy);
+                y.lamf = (float)y.lam;
+                y.delta = delta;
+                // the concurrent bulk pass may update a cell before this sweep's
+                // geometry is known only when the body moves by less than a cell
+                // along the sweep and does not rotate (its band then lies within one
+                // cell, along the sweep, of the cells touched at the start pose)
+                y.defer_all = (I.serial_bulk || I.rotating || fabs(delta) >= 0.9 * (dir == 0 ? I.dx : I.dy)) ? 1 : 0;
+                y.XA = X; y.YA = Yp; y.thA = th; y.cA = c; y.sA = s;
+                y.band_count = 0;
+                y.nbad = 0;
+                y.nbadlist = 0;
+                y.nbulk = 0;
+                y.mixed = 0;
+                for (int q = 0; q < MAXC; ++q) y.wall_sum[q] = 0.0;
+            } else if (P == 1) {
+                y.XM = X; y.YM = Yp; y.thM = th; y.cM = c; y.sM = s;
+                y.Om = Om;
             } else {
-                if (dt_host > 0.0 && dt_host != dt) y.err |= ERR_STATE;
-                // the last sweep of the step gathers the wave speeds of the next step's dt
-                y.S[0] = 0ull;
-                y.S[1] = 0ull;
+                y.XB = X; y.YB = Yp; y.thB = th; y.cB = c; y.sB = s;
             }
-            y.lam = dt / (dir == 0 ? I.dx : I.dy);
-            y.lamf = (float)y.lam;
-            y.delta = delta;
-            // the concurrent bulk pass may update a cell before this sweep's
-            // geometry is known only when the body moves by less than a cell
-            // along the sweep and does not rotate (its band then lies within one
-            // cell, along the sweep, of the cells touched at the start pose)
-            y.defer_all = (I.serial_bulk || I.rotating || fabs(delta) >= 0.9 * (dir == 0 ? I.dx : I.dy)) ? 1 : 0;
-            y.XA = XA; y.YA = YA; y.XB = XB; y.YB = YB; y.XM = XM; y.YM = YM;
-            y.thA = thA; y.thB = thB; y.thM = thM;
-            y.cA = cA; y.sA = sA; y.cB = cB; y.sB = sB; y.cM = cM; y.sM = sM;
-            y.Om = Om;
-            y.band_count = 0;
-            y.nbad = 0;
-            y.nbadlist = 0;
-            y.nbulk = 0;
-            y.mixed = 0;
-            for (int q = 0; q < MAXC; ++q) y.wall_sum[q] = 0.0;
         }
-        sh[0] = XA; sh[1] = YA; sh[2] = XM; sh[3] = YM; sh[4] = XB; sh[5] = YB;
-        sh[6] = cA; sh[7] = sA; sh[8] = cM; sh[9] = sM; sh[10] = cB; sh[11] = sB;
     }
     __syncthreads();
     // posed position of vertex a at pose P (0: A, 1: M, 2: B)
@@ -503,7 +503,7 @@ __device__ double swept_face_B(const GeoBuf &G, const InstDesc &I, int dir, doub
 // cell of the group gets a thread, and each column keeps a bit list of the
 // edges that can meet its cells.
 // ---------------------------------------------------------------------------
-constexpr int GC = GEO_GC;          // columns per group
+constexpr int GC = GEO_GC;          // columns per group, at most (gcw of them in a launch)
 constexpr int EMAXG = 384;          // edges per group and pose
 constexpr int LMAXG = 32;           // crossings per grid line
 constexpr int NWB = 64;             // bitmap words per column (2048 rows of the body's extent)
@@ -533,10 +533,19 @@ struct GeoBufG {
     int cnt;
 };
 
+// a warp's (query, edge) pairs of rect_edges_w: the edge and the query's lane,
+// then the pair's contribution
+constexpr int NPAIRW = 88;           // (three CTAs' shared memory fits an SM)
+struct GeoPairs {
+    double a[NPAIRW], x[NPAIRW], y[NPAIRW];
+    unsigned short pr[NPAIRW];
+};
+static_assert(EMAXG <= 512, "9 bits of a pair hold its edge");
 struct GeoWarpG {
     GeoBufG G;
     unsigned bA[GC][NWB], bB[GC][NWB], bM[GC][NWB];
     int wpre[GC * NWB + 1];
+    GeoPairs P[GEOMG_THREADS / 32];   // (k_geom<true> only)
 };
 
 __device__ __forceinline__ bool edge_yrange_s(double xa, double ya, double xb, double yb, double slope, double xl,
@@ -704,33 +713,27 @@ __device__ void gather_g(GeoBufG &G, const InstDesc &I, const double *__restrict
 // closed cell an edge meets (exact predicate)
 __device__ void index_g(GeoBufG &G, const InstDesc &I, int i0, int ncol, int row0, int nwb, unsigned (*bits)[NWB],
                         int tid) {
-    const int n = G.cnt, nwd = (n + 31) >> 5;
-    for (int p = tid; p < (2 * ncol + 1) * nwd; p += GEOMG_THREADS) {
-        const int r = p / nwd, w = p - r * nwd;
-        unsigned msk = 0u;
+    const int n = G.cnt, nwd = (n + 31) >> 5, lane = tid & 31;
+    // a warp per list and word, a lane per edge
+    for (int p = tid >> 5; p < (2 * ncol + 1) * nwd; p += GEOMG_THREADS / 32) {
+        const int r = p / nwd, w = p - r * nwd, e = w * 32 + lane;
+        bool in = e < n;
         if (r < ncol) {
             const int i = i0 + r;
-            for (int b = 0; b < 32; ++b) {
-                const int e = w * 32 + b;
-                if (e < n && G.ilo[e] <= i && i <= G.ihi[e]) msk |= 1u << b;
-            }
-            G.cm[r][w] = msk;
+            in = in && G.ilo[e] <= i && i <= G.ihi[e];
         } else {
-            const int L = r - ncol;
-            const double xs = G.xln[L];
+            const double xs = G.xln[r - ncol];
             const float fxs = (float)xs;
-            unsigned cand = 0u;
-            for (int b = 0; b < 32; ++b) {
-                const int e = w * 32 + b;
-                if (e < n && G.fx1[e] >= fxs && G.fx0[e] <= fxs) cand |= 1u << b;
+            in = in && G.fx1[e] >= fxs && G.fx0[e] <= fxs;
+            if (in) {
+                const long long ka = dk(G.xa[e]), kb = dk(G.xb[e]), ks = dk(xs);
+                in = ka != kb && (ka < kb ? (ka <= ks && ks <= kb) : (kb <= ks && ks <= ka));
             }
-            for (; cand; cand &= cand - 1u) {
-                const int b = __ffs(cand) - 1, e = w * 32 + b;
-                const double xa = G.xa[e], xb = G.xb[e];
-                const long long ka = dk(xa), kb = dk(xb), ks = dk(xs);
-                if (ka != kb && (ka < kb ? (ka <= ks && ks <= kb) : (kb <= ks && ks <= ka))) msk |= 1u << b;
-            }
-            G.lm[L][w] = msk;
+        }
+        const unsigned msk = __ballot_sync(0xffffffffu, in);
+        if (lane == 0) {
+            if (r < ncol) G.cm[r][w] = msk;
+            else G.lm[r - ncol][w] = msk;
         }
     }
     if (!bits) return;
@@ -747,17 +750,24 @@ __device__ void index_g(GeoBufG &G, const InstDesc &I, int i0, int ncol, int row
         double elo, ehi;
         if (!edge_yrange_s(G.xa[e], G.ya[e], G.xb[e], G.yb[e], G.slope[e], xl, xr, &elo, &ehi)) continue;
         const int jf0 = row_floor_f(I, elo), jf1 = row_floor_f(I, ehi);
-        int jl = jf0 - 1, jh = jf1 + 1;
-        if (jl < row0) jl = row0;
-        if (jh > I.ny - 1) jh = I.ny - 1;
-        if (jh > row0 + 32 * nwb - 1) jh = row0 + 32 * nwb - 1;
-        for (int j = jl; j <= jh; ++j) {
-            // rows jf0+1 .. jf1-1 lie strictly inside [elo, ehi] whatever the
-            // rounding of the floors; the exact predicate decides the rest
-            bool hit = j > jf0 && j < jf1;
-            if (!hit) hit = dle(I.yn[j], ehi) && dle(elo, I.yn[j + 1]);
-            if (hit) atomicOr(&bits[c][(j - row0) >> 5], 1u << ((j - row0) & 31));
-        }
+        const int jmax = min(I.ny - 1, row0 + 32 * nwb - 1);
+        // rows jf0+1 .. jf1-1 lie strictly inside [elo, ehi] whatever the
+        // rounding of the floors; the exact predicate decides the two rows
+        // at each end (their grid lines loaded together)
+        double yl[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) yl[k] = I.yn[min(max((k < 3 ? jf0 - 1 : jf1 - 3) + k, 0), I.ny)];
+        auto mark = [&](int j) {
+            if (j >= row0 && j <= jmax) atomicOr(&bits[c][(j - row0) >> 5], 1u << ((j - row0) & 31));
+        };
+        auto test = [&](int j, double y0, double y1) {
+            if (dle(y0, ehi) && dle(elo, y1)) mark(j);
+        };
+        test(jf0 - 1, yl[0], yl[1]);
+        test(jf0, yl[1], yl[2]);
+        for (int j = jf0 + 1; j < jf1; ++j) mark(j);
+        if (jf1 > jf0) test(jf1, yl[3], yl[4]);
+        test(jf1 + 1, yl[4], yl[5]);
     }
 }
 
@@ -974,12 +984,132 @@ __device__ double rect_edges_g(const GeoBufG &G, int c, int ja, int jb, double r
     return A;
 }
 
-__device__ __forceinline__ double cell_alpha_g(const GeoBufG &G, const InstDesc &I, int c, int i, int j, double xl,
-                                               double xr, double yb, double yt, double *nlx, double *nly, bool *mov) {
-    double A = rect_edges_g(G, c, j, j, xl, xr, yb, yt, xl, xr, nlx, nly, mov) +
-               (xr - xl) * line_solid_vg(G, c + 1, yb, yt, true);
-    double a = clamp01(1.0 - A / (I.dx * I.dy));
-    return a < ALPHA_MIN ? 0.0 : a;
+// rect_edges_g for a warp of queries (act: this lane has one), the work
+// spread over the lanes: for one query after the other the lanes test 32
+// edges of its column at a time and list the candidates, then the warp clips
+// 32 (query, edge) pairs at a time, and each lane adds its pairs'
+// contributions in edge order, so that the sums are rect_edges_g's bit for
+// bit.  A thread per query walked its column's edges one by one (about 400
+// cycles per edge, the lanes diverging) and clipped its candidates one by
+// one, while the FP64 pipe takes 64 cycles per warp instruction whatever the
+// active lanes.  For groups narrower than GEO_GC (few cells per group); with
+// full groups the tests of all edges for every query cost more than they save
+// (64 grids: 178 us per launch with a thread per query, 238 so).
+struct RectSum {
+    double A, nlx, nly;
+    bool mov;
+};
+template <bool NRM>
+__device__ __forceinline__ RectSum rect_edges_w(const GeoBufG &G, GeoPairs &S, bool act, int c, int ja, int jb,
+                                                double rx0, double rx1, double ry0, double ry1, double xo, double xs) {
+    const int lane = threadIdx.x & 31;
+    const float frx0 = __double2float_rd(rx0), frx1 = __double2float_ru(rx1);
+    const float fry0 = __double2float_rd(ry0), fry1 = __double2float_ru(ry1);
+    const int jab = (ja & 0xffff) | jb << 16;   // (rows lie within +-16384)
+    RectSum r = {0.0, 0.0, 0.0, false};
+    const int nwd = (G.cnt + 31) >> 5;
+    unsigned todo = __ballot_sync(0xffffffffu, act);
+    int w = 0;
+    while (todo) {
+        // the candidate pairs of as many queries as the list holds
+        int off = 0, ns = 0, tot = 0;   // this lane's pairs in the list, the list's length
+        while (todo && tot <= NPAIRW - 32) {
+            const int q = __ffs(todo) - 1;
+            const int qc = __shfl_sync(0xffffffffu, c, q), qj = __shfl_sync(0xffffffffu, jab, q);
+            const float x0 = __shfl_sync(0xffffffffu, frx0, q), x1 = __shfl_sync(0xffffffffu, frx1, q);
+            const float y0 = __shfl_sync(0xffffffffu, fry0, q), y1 = __shfl_sync(0xffffffffu, fry1, q);
+            const int qja = (short)qj, qjb = qj >> 16;
+            if (lane == q) off = tot;
+            for (; w < nwd && tot <= NPAIRW - 32; ++w) {
+                const unsigned col = G.cm[qc][w];
+                if (!col) continue;
+                const int e = w * 32 + lane;
+                bool cand = (col >> lane) & 1u;
+                if (cand)
+                    cand = (int)G.jhi[e] >= qja && (int)G.jlo[e] <= qjb && G.fy1[e] >= y0 && G.fy0[e] <= y1 &&
+                           G.fx1[e] >= x0 && G.fx0[e] <= x1;
+                const unsigned m = __ballot_sync(0xffffffffu, cand);
+                if (cand) S.pr[tot + __popc(m & ((1u << lane) - 1u))] = (unsigned short)(e | q << 9);
+                tot += __popc(m);
+                if (lane == q) ns += __popc(m);
+            }
+            if (w == nwd) {
+                w = 0;
+                todo &= todo - 1u;
+            }
+        }
+        __syncwarp();
+        for (int p0 = 0; p0 < tot; p0 += 32) {
+            const int p = p0 + lane;
+            const bool in = p < tot;
+            const int pr = in ? S.pr[p] : 0, q = pr >> 9, e = pr & 511;
+            const double bx0 = __shfl_sync(0xffffffffu, rx0, q), bx1 = __shfl_sync(0xffffffffu, rx1, q);
+            const double by0 = __shfl_sync(0xffffffffu, ry0, q), by1 = __shfl_sync(0xffffffffu, ry1, q);
+            const double bxo = __shfl_sync(0xffffffffu, xo, q), bxs = __shfl_sync(0xffffffffu, xs, q);
+            if (!in) continue;
+            double da = 0.0, dx = 0.0, dy = 0.0;
+            bool hit = false;
+            const double xa = G.xa[e], xb = G.xb[e], ya = G.ya[e], yb = G.yb[e];
+            const long long kxa = dk(xa), kxb = dk(xb), kya = dk(ya), kyb = dk(yb);
+            const long long krx0 = dk(bx0), krx1 = dk(bx1), kry0 = dk(by0), kry1 = dk(by1);
+            if (!((kya < kry0 && kyb < kry0) || (kya > kry1 && kyb > kry1) || (kxa < krx0 && kxb < krx0) ||
+                  (kxa > krx1 && kxb > krx1))) {
+                const double lx0 = bx0 - bxo, lx1 = bx1 - bxo, ly1 = by1 - by0;
+                const double ax = xa - bxo, ay = ya - by0, bx = xb - bxo, by = yb - by0;
+                const double ddx = bx - ax, ddy = by - ay;
+                double t0 = 0.0, t1 = 1.0;
+                bool ok = true;
+                if (dzero(ddx)) {
+                    const long long kax = dk(ax);
+                    if (kax < dk(lx0) || kax > dk(lx1)) ok = false;
+                } else {
+                    const double inv = G.idx[e];
+                    const double ra = (lx0 - ax) * inv, rb = (lx1 - ax) * inv;
+                    t0 = dmax(t0, dmin(ra, rb));
+                    t1 = dmin(t1, dmax(ra, rb));
+                }
+                if (dzero(ddy)) {
+                    const long long kay = dk(ay);
+                    if (kay < 0 || kay > dk(ly1)) ok = false;
+                } else {
+                    const double inv = G.idy[e];
+                    const double ra = (0.0 - ay) * inv, rb = (ly1 - ay) * inv;
+                    t0 = dmax(t0, dmin(ra, rb));
+                    t1 = dmin(t1, dmax(ra, rb));
+                }
+                if (ok && !dlt(t1, t0)) {
+                    hit = true;
+                    // (not a vertical edge on the grid side)
+                    if (!(kxa == kxb && kxa == dk(bxs)) && dlt(t0, t1)) {
+                        const double xc0 = ax + t0 * ddx, xc1 = ax + t1 * ddx;
+                        const double ly = ddy * (t1 - t0);
+                        da = ly * (0.5 * (xc0 + xc1));
+                        if (NRM) {
+                            dx = ly;
+                            dy = ddx * (t1 - t0);
+                        }
+                    }
+                }
+            }
+            S.a[p] = da;
+            if (NRM) {
+                S.x[p] = dx;
+                S.y[p] = dy;
+            }
+            S.pr[p] = hit && G.mov[e];
+        }
+        __syncwarp();
+        for (int k = 0; k < ns; ++k) {
+            r.A += S.a[off + k];
+            if (NRM) {
+                r.nlx -= S.x[off + k];
+                r.nly += S.y[off + k];
+            }
+            r.mov = r.mov || S.pr[off + k];
+        }
+        __syncwarp();
+    }
+    return r;
 }
 
 __device__ double face_ap_g(const GeoBufG &G, const InstDesc &I, int dir, bool hi, int c, int i, int j, double xl,
@@ -1013,12 +1143,29 @@ __device__ double swept_face_Bg(const GeoBufG &G, const InstDesc &I, int dir, do
     return clamp01(1.0 - A / ((y1 - y0) * I.dx));
 }
 
-// the band cells of geometry group gw (one CTA)
+// position of the n-th (from 0) set bit of m
+__device__ __forceinline__ int nth_bit(unsigned m, int n) {
+    int p = 0;
+#pragma unroll
+    for (int h = 16; h > 0; h >>= 1) {
+        const int low = __popc(m & ((1u << h) - 1u));
+        if (n >= low) {
+            n -= low;
+            m >>= h;
+            p += h;
+        }
+    }
+    return p;
+}
+
+// the band cells of geometry group gw (one CTA).  WIDE: a warp shares its
+// queries' edges among its lanes (rect_edges_w); else a thread per query.
+template <bool WIDE>
 __device__ __forceinline__ void geom_group(int gw, const InstDesc *__restrict__ D, InstDyn *__restrict__ Y,
                                            const int *__restrict__ ginst, const double *__restrict__ px,
                                            const double *__restrict__ py, const float *__restrict__ ebox,
                                            const int *__restrict__ vnext, const unsigned char *__restrict__ vmov,
-                                           int total_v, int n_inst, int total_groups, int dir,
+                                           int total_v, int n_inst, int total_groups, int gcw, int dir,
                                            BandRec *__restrict__ R, double *__restrict__ bnd, int &sh_base) {
     extern __shared__ __align__(16) unsigned char gsm[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tid = threadIdx.x;
@@ -1028,9 +1175,9 @@ __device__ __forceinline__ void geom_group(int gw, const InstDesc *__restrict__ 
     const int lo = ginst[gw];
     const InstDesc &I = D[lo];
     InstDyn &y = Y[lo];
-    const int i0 = y.col0 + GC * (gw - I.gcol_off);
+    const int i0 = y.col0 + gcw * (gw - I.gcol_off);
     if (i0 > y.col1 || i0 >= I.nx || I.nv == 0) return;
-    const int ncol = min(GC, min(y.col1, I.nx - 1) - i0 + 1);
+    const int ncol = min(gcw, min(y.col1, I.nx - 1) - i0 + 1);
     const double delta = y.delta;
     const bool own_hi = I.rotating || delta >= 0.0;
     const double ad = fabs(delta);
@@ -1102,7 +1249,7 @@ __device__ __forceinline__ void geom_group(int gw, const InstDesc *__restrict__ 
         *c = a / nwb;
         *k = a % nwb;
         const unsigned mask = W.bA[*c][*k] | W.bB[*c][*k] | W.bM[*c][*k];
-        *bit = __fns(mask, 0, t - W.wpre[a] + 1);
+        *bit = nth_bit(mask, t - W.wpre[a]);
         *j = row0 + (*k) * 32 + *bit;
     };
     const double wsimp_B = 1.0 / 6.0, wsimp_M = 4.0 / 6.0, wsimp_A = 1.0 / 6.0;
@@ -1111,9 +1258,15 @@ __device__ __forceinline__ void geom_group(int gw, const InstDesc *__restrict__ 
     // clipping work evenly; the pass-M partial results wait in the record
     // (aM, nx, ny, d, wx, pad) for the per-cell step that combines them.
     // pass B (edges of the end pose are in G): 0: alpha_B and flags, 1: the
-    // owned face's time-averaged aperture
-    for (int u = tid; u < 2 * T; u += GEOMG_THREADS) {
-        const int part = u >= T ? 1 : 0, t = u - part * T;   // parts in contiguous blocks: warps stay uniform
+    // owned face's time-averaged aperture.  The queries go to the warps in
+    // equal shares (parts in contiguous blocks: warps stay nearly uniform).
+    constexpr int NWARP = GEOMG_THREADS / 32;
+    const bool strip = !I.rotating && delta != 0.0;   // the owned face sweeps a strip
+    const int perB = WIDE ? min(32, (2 * T + NWARP - 1) / NWARP) : 32;
+    for (int u0 = warp * perB; u0 < 2 * T; u0 += NWARP * perB) {
+        const bool act = lane < perB && u0 + lane < 2 * T;
+        const int u = act ? u0 + lane : 0;
+        const int part = u >= T ? 1 : 0, t = u - part * T;
         int c, j, k, bit;
         locate(t, &c, &j, &k, &bit);
         const int i = i0 + c;
@@ -1121,13 +1274,44 @@ __device__ __forceinline__ void geom_group(int gw, const InstDesc *__restrict__ 
         const double xl = G.xln[c], xr = G.xln[c + 1];
         const double yb = I.yn[j], yt = I.yn[j + 1];
         const int cell = j * I.pitch + i;
+        // the query's rectangle: the cell, or the strip its owned face sweeps
+        // (swept_face_Bg), and the grid line whose solid length closes it
+        double rx0 = xl, rx1 = xr, ry0 = yb, ry1 = yt, xo = xl, xs = xr;
+        int ja = j, jb = j, line = c + 1;
+        bool left = true;
+        if (part == 1) {
+            if (dir == 0) {
+                xs = own_hi ? xr : xl;
+                line = own_hi ? c + 1 : c;
+                rx0 = delta > 0.0 ? xs : xs + delta;
+                rx1 = delta > 0.0 ? xs + delta : xs;
+                xo = delta > 0.0 ? rx1 : rx0;
+                left = !(delta > 0.0);
+            } else {
+                const double ys = own_hi ? yt : yb;
+                ry0 = delta > 0.0 ? ys : ys + delta;
+                ry1 = delta > 0.0 ? ys + delta : ys;
+                ja = delta > 0.0 ? j : j - 1;
+                jb = delta > 0.0 ? j + 1 : j;
+            }
+        }
+        RectSum sum = {0.0, 0.0, 0.0, false};
+        const bool rect = act && (part == 0 || strip);
+        if constexpr (WIDE)
+            sum = rect_edges_w<false>(G, W.P[warp], rect, c, ja, jb, rx0, rx1, ry0, ry1, xo, xs);
+        else if (rect)
+            sum.A = rect_edges_g(G, c, ja, jb, rx0, rx1, ry0, ry1, xo, xs, nullptr, nullptr, &sum.mov);
+        const double Ae = sum.A;
+        const bool mov = sum.mov;
+        if (!act) continue;
         if (part == 0) {
             const bool tA = (W.bA[c][k] >> bit) & 1u, tB = (W.bB[c][k] >> bit) & 1u, tM = (W.bM[c][k] >> bit) & 1u;
             r.cell = cell;
             r.i = i;
             r.j = j;
-            bool mov = false;
-            r.aB = cell_alpha_g(G, I, c, i, j, xl, xr, yb, yt, nullptr, nullptr, &mov);
+            const double A = Ae + (xr - xl) * line_solid_vg(G, c + 1, yb, yt, true);
+            const double al = clamp01(1.0 - A / (I.dx * I.dy));
+            r.aB = al < ALPHA_MIN ? 0.0 : al;
             r.aA = I.alpha[cell];
             const bool movA = (I.cls[cell] & CLS_MOVT) != 0;
             r.flags = (tA ? RF_TOUCH_A : 0) | (tB ? RF_TOUCH_B : 0) | (tM ? RF_TOUCH_M : 0) |
@@ -1137,12 +1321,17 @@ __device__ __forceinline__ void geom_group(int gw, const InstDesc *__restrict__ 
                 dir == 0 ? ((own_hi && i == 0 && I.bc[0] != 2) || (!own_hi && i == I.nx - 1 && I.bc[1] != 2))
                          : ((own_hi && j == 0 && I.bc[2] != 2) || (!own_hi && j == I.ny - 1 && I.bc[3] != 2));
             double bo, bb = 0.0;
-            if (I.rotating) {
+            if (strip) {
+                const double w = dir == 0 ? rx1 - rx0 : xr - xl;
+                const double A = Ae + w * line_solid_vg(G, line, ry0, ry1, left);
+                bo = clamp01(1.0 - A / (dir == 0 ? (rx1 - rx0) * I.dy : (ry1 - ry0) * I.dx));
+                if (need_bnd) bb = swept_face_Bg(G, I, dir, delta, !own_hi, c, i, j, xl, xr, yb, yt);
+            } else if (I.rotating) {
                 bo = wsimp_B * face_ap_g(G, I, dir, true, c, i, j, xl, xr, yb, yt);
                 if (need_bnd) bb = wsimp_B * face_ap_g(G, I, dir, false, c, i, j, xl, xr, yb, yt);
-            } else {
-                bo = swept_face_Bg(G, I, dir, delta, own_hi, c, i, j, xl, xr, yb, yt);
-                if (need_bnd) bb = swept_face_Bg(G, I, dir, delta, !own_hi, c, i, j, xl, xr, yb, yt);
+            } else {   // the body does not move along the sweep
+                bo = face_ap_g(G, I, dir, own_hi, c, i, j, xl, xr, yb, yt);
+                if (need_bnd) bb = face_ap_g(G, I, dir, !own_hi, c, i, j, xl, xr, yb, yt);
             }
             r.bown = bo;
             bnd[I.rec_base + base + t] = bb;
@@ -1157,7 +1346,10 @@ __device__ __forceinline__ void geom_group(int gw, const InstDesc *__restrict__ 
     __syncthreads();
     if (warp == 1) compact_lines_g(G, ncol, lane, &err);
     __syncthreads();
-    for (int u = tid; u < 3 * T; u += GEOMG_THREADS) {
+    const int perM = WIDE ? min(32, (3 * T + NWARP - 1) / NWARP) : 32;
+    for (int u0 = warp * perM; u0 < 3 * T; u0 += NWARP * perM) {
+        const bool act = lane < perM && u0 + lane < 3 * T;
+        const int u = act ? u0 + lane : 0;
         const int part = u / T, t = u - part * T;
         int c, j, k, bit;
         locate(t, &c, &j, &k, &bit);
@@ -1166,13 +1358,19 @@ __device__ __forceinline__ void geom_group(int gw, const InstDesc *__restrict__ 
         BandRec &r = R[ri];
         const double xl = G.xln[c], xr = G.xln[c + 1];
         const double yb = I.yn[j], yt = I.yn[j + 1];
+        RectSum sum = {0.0, 0.0, 0.0, false};
+        if constexpr (WIDE)
+            sum = rect_edges_w<true>(G, W.P[warp], act && part == 0, c, j, j, xl, xr, yb, yt, xl, xr);
+        else if (act && part == 0)
+            sum.A = rect_edges_g(G, c, j, j, xl, xr, yb, yt, xl, xr, &sum.nlx, &sum.nly, &sum.mov);
+        if (!act) continue;
         if (part == 0) {
-            bool mov = false;
-            double nlx = 0.0, nly = 0.0;
-            r.aM = cell_alpha_g(G, I, c, i, j, xl, xr, yb, yt, &nlx, &nly, &mov);
-            r.nx = nlx;
-            r.ny = nly;
-            r.aux = mov ? 1 : 0;
+            const double A = sum.A + (xr - xl) * line_solid_vg(G, c + 1, yb, yt, true);
+            const double al = clamp01(1.0 - A / (I.dx * I.dy));
+            r.aM = al < ALPHA_MIN ? 0.0 : al;
+            r.nx = sum.nlx;
+            r.ny = sum.nly;
+            r.aux = sum.mov ? 1 : 0;
         } else if (part == 1) {
             if (I.rotating) {
                 r.bown += wsimp_M * face_ap_g(G, I, dir, true, c, i, j, xl, xr, yb, yt);
@@ -1252,16 +1450,21 @@ __device__ __forceinline__ void geom_group(int gw, const InstDesc *__restrict__ 
 
 // One CTA per geometry group (a grid capped below the group count, looping
 // over the groups so that bulk CTAs find room beside it, measured slower).
+// Bound by latency: FP64 chains and barriers of few warps.  400 x 400 grid
+// around a cylinder: 95 us with 6 groups of 16 columns and a thread per query,
+// 56 with 44 groups of 2 and the queries' edges shared by the lanes; 1024 x
+// 1024 around the aerofoil 120 -> 66.
+template <bool WIDE>
 __global__ void __launch_bounds__(GEOMG_THREADS, 3) k_geom(const InstDesc *__restrict__ D, InstDyn *__restrict__ Y,
                                                             const int *__restrict__ ginst,
                                                             const double *__restrict__ px, const double *__restrict__ py,
                                                             const float *__restrict__ ebox,
                                                             const int *__restrict__ vnext,
                                                             const unsigned char *__restrict__ vmov, int total_v,
-                                                            int n_inst, int total_groups, int dir,
+                                                            int n_inst, int total_groups, int gcw, int dir,
                                                             BandRec *__restrict__ R, double *__restrict__ bnd) {
     __shared__ int sh_base;
-    geom_group(blockIdx.x, D, Y, ginst, px, py, ebox, vnext, vmov, total_v, n_inst, total_groups, dir, R, bnd,
+    geom_group<WIDE>(blockIdx.x, D, Y, ginst, px, py, ebox, vnext, vmov, total_v, n_inst, total_groups, gcw, dir, R, bnd,
                sh_base);
 }
 
@@ -1394,10 +1597,11 @@ __global__ void k_nodes(const InstDesc *__restrict__ D) {
 // launchers
 // ---------------------------------------------------------------------------
 static size_t geom_smem() { return sizeof(GeoWarp) * GEOM_WARPS; }
-static size_t geomg_smem() { return sizeof(GeoWarpG); }
+static size_t geomg_smem(bool wide) { return wide ? sizeof(GeoWarpG) : offsetof(GeoWarpG, P); }
 
 void geom_init() {
-    cudaFuncSetAttribute(k_geom, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)geomg_smem());
+    cudaFuncSetAttribute(k_geom<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)geomg_smem(true));
+    cudaFuncSetAttribute(k_geom<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)geomg_smem(false));
     cudaFuncSetAttribute(k_classify, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)geom_smem());
 }
 
@@ -1413,12 +1617,16 @@ void launch_pose(const InstDesc *D, InstDyn *Y, const double *vx, const double *
 }
 
 void launch_geom(const InstDesc *D, InstDyn *Y, const int *ginst, const double *px, const double *py, const float *ebox,
-                 const int *vnext, const unsigned char *vmov, int total_v, int n_inst, int total_groups, int dir,
+                 const int *vnext, const unsigned char *vmov, int total_v, int n_inst, int total_groups, int gcw, int dir,
                  BandRec *R, double *bnd, cudaStream_t st) {
-    const int blocks = total_groups;
-    if (blocks > 0)
-        k_geom<<<blocks, GEOMG_THREADS, geomg_smem(), st>>>(D, Y, ginst, px, py, ebox, vnext, vmov, total_v, n_inst,
-                                                             total_groups, dir, R, bnd);
+    if (total_groups <= 0) return;
+    if (gcw < GC)
+        k_geom<true><<<total_groups, GEOMG_THREADS, geomg_smem(true), st>>>(D, Y, ginst, px, py, ebox, vnext, vmov, total_v,
+                                                                            n_inst, total_groups, gcw, dir, R, bnd);
+    else
+        k_geom<false><<<total_groups, GEOMG_THREADS, geomg_smem(false), st>>>(D, Y, ginst, px, py, ebox, vnext, vmov,
+                                                                              total_v, n_inst, total_groups, gcw, dir, R,
+                                                                              bnd);
 }
 
 void launch_classify(const InstDesc *D, InstDyn *Y, const double *vx, const double *vy, const unsigned char *vmov,

@@ -8,7 +8,7 @@ namespace mb {
 
 constexpr int MAXC = 4;
 constexpr int NBULK = 32;              // non-physical bulk cells listed per sweep
-constexpr int GEO_GC = 16;            // grid columns per geometry group (one CTA each)
+constexpr int GEO_GC = 16;            // grid columns per geometry group (one CTA each), at most
 constexpr double ALPHA_MIN = 1e-10;   // smaller volume fractions count as solid
 // launch shape of the FP32x2 bulk kernels: bits 0-9 CTA threads (64 or 128),
 // bit 10 registers budgeted for 4 resident CTAs per SM (else 5), bit 11 an
