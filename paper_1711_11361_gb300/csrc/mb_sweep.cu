@@ -108,31 +108,6 @@ struct CellW {
     int rec;       // band record (real cells only) or -1
 };
 
-template <class T>
-__device__ __forceinline__ void fetch(const InstDesc &I, const BandRec *R, int dir, int src, int l, int k,
-                                      CellW<T> &c) {
-    bool real, flip;
-    int ci = line_cell(I, dir, l, k, &real, &flip);
-    uint8_t cl = I.cls[ci];
-    int ri = (cl & CLS_BAND) ? I.rec[ci] : -1;
-    c.rec = real ? ri : -1;
-    const T *Q = buf<T>(I, src);
-    size_t plane = (size_t)I.pitch * I.ny;
-    if (ri >= 0) {
-        const BandRec &r = R[ri];
-        c.fluid = (r.flags & RF_FLUID_A) != 0;
-        if (c.fluid && (r.flags & RF_UNCOV)) {
-            for (int q = 0; q < I.nc; ++q) c.q[q] = (T)r.Qp[q];
-        } else {
-            for (int q = 0; q < I.nc; ++q) c.q[q] = Q[q * plane + ci];
-        }
-    } else {
-        c.fluid = !(cl & CLS_SOLID);
-        for (int q = 0; q < I.nc; ++q) c.q[q] = Q[q * plane + ci];
-    }
-    if (flip && I.nc == 4) c.q[1 + dir] = -c.q[1 + dir];
-}
-
 // time-averaged aperture of the face between along positions a and a+1
 __device__ double face_beta(const InstDesc &I, const BandRec *R, const double *bnd, int dir, int l, int a,
                             bool own_hi) {
@@ -470,31 +445,81 @@ __device__ __forceinline__ bool band_sweep_rec(const InstDesc *__restrict__ D, I
     const double lam = y.lam;
     const T g = (T)I.gamma, lamT = (T)lam, av0 = (T)I.adv[0], av1 = (T)I.adv[1];
     const bool own_hi = I.rotating || y.delta >= 0.0;
+    // the five cells of the two faces' stencils: their class, record index and
+    // state together, then what the records hold together (a cell without a
+    // record reads this one's), so that a record waits for two rounds of
+    // loads instead of three for each cell and face in turn
     CellW<T> w[5];
-    for (int m = 0; m < 5; ++m) fetch<T>(I, R, dir, src, l, k - 2 + m, w[m]);
+    uint8_t cl[5];
+    int ri[5];
+    bool flip[5];
+    const T *Q = buf<T>(I, src);
+    const size_t plane = (size_t)I.pitch * I.ny;
+#pragma unroll
+    for (int m = 0; m < 5; ++m) {
+        bool real;
+        const int ci = line_cell(I, dir, l, k - 2 + m, &real, &flip[m]);
+        cl[m] = I.cls[ci];
+        ri[m] = I.rec[ci];
+#pragma unroll
+        for (int q = 0; q < MAXC; ++q) w[m].q[q] = q < I.nc ? Q[q * plane + ci] : T(0);
+        w[m].rec = real ? 0 : -1;
+    }
+    int fl[5];
+    double bo[5];
+#pragma unroll
+    for (int m = 0; m < 5; ++m) {
+        ri[m] = (cl[m] & CLS_BAND) ? ri[m] : -1;
+        const BandRec &o = R[ri[m] >= 0 ? ri[m] : r];
+        fl[m] = ri[m] >= 0 ? o.flags : 0;
+        bo[m] = o.bown;
+    }
+    bool has[3];
+    double dd[3], FBw[3][MAXC];
+#pragma unroll
+    for (int m = 1; m < 4; ++m) {
+        const BandRec &o = R[ri[m] >= 0 ? ri[m] : r];
+        has[m - 1] = w[m].rec == 0 && (fl[m] & RF_WALL);
+        dd[m - 1] = o.d;
+#pragma unroll
+        for (int q = 0; q < MAXC; ++q) FBw[m - 1][q] = o.FB[q];
+    }
+#pragma unroll
+    for (int m = 0; m < 5; ++m) {
+        w[m].rec = w[m].rec == 0 ? ri[m] : -1;
+        w[m].fluid = ri[m] >= 0 ? (fl[m] & RF_FLUID_A) != 0 : !(cl[m] & CLS_SOLID);
+        if (w[m].fluid && (fl[m] & RF_UNCOV))
+            for (int q = 0; q < I.nc; ++q) w[m].q[q] = (T)R[ri[m]].Qp[q];
+        if (flip[m] && I.nc == 4) w[m].q[1 + dir] = -w[m].q[1 + dir];
+    }
+    // apertures of the faces between cells m and m+1, each its owner's value
     double bt[4];
-    for (int m = 0; m < 4; ++m) bt[m] = face_beta(I, R, bnd, dir, l, k - 2 + m, own_hi);
-    auto wall_of = [&](const CellW<T> &c, bool *has, double *d, double *FB) {
-        *has = false;
-        if (c.rec >= 0 && (R[c.rec].flags & RF_WALL)) {
-            const BandRec &o = R[c.rec];
-            *has = true;
-            *d = o.d;
-            for (int q = 0; q < MAXC; ++q) FB[q] = o.FB[q];
-        }
+    const int n = dir == 0 ? I.nx : I.ny;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        const int om = own_hi ? m : m + 1, o = k - 2 + om;
+        const uint8_t oc = own_hi ? cl[m] : cl[m + 1];
+        if ((o >= 0 && o < n) || I.bc[2 * dir] == 2)
+            bt[m] = (oc & CLS_BAND) ? (own_hi ? bo[m] : bo[m + 1]) : (oc & CLS_SOLID) ? 0.0 : 1.0;
+        else bt[m] = face_beta(I, R, bnd, dir, l, k - 2 + m, own_hi);
+    }
+    auto wall_of = [&](int m, bool *h, double *d, double *FB) {
+        *h = has[m - 1];
+        *d = dd[m - 1];
+        for (int q = 0; q < MAXC; ++q) FB[q] = FBw[m - 1][q];
     };
     FaceIn fi;
     fi.dL = fi.dR = 0.0;
     // low face: cells k-1 | k
     fi.btL = bt[0]; fi.btF = bt[1]; fi.btR = bt[2];
-    wall_of(w[1], &fi.hasL, &fi.dL, fi.FBL);
-    wall_of(w[2], &fi.hasR, &fi.dR, fi.FBR);
+    wall_of(1, &fi.hasL, &fi.dL, fi.FBL);
+    wall_of(2, &fi.hasR, &fi.dR, fi.FBR);
     double Flo[MAXC], Fhi[MAXC];
     face_stab<T>(I.eq, g, dir, lamT, av0, av1, I.nc, &w[0], &fi, Flo);
     // high face: cells k | k+1
     fi.btL = bt[1]; fi.btF = bt[2]; fi.btR = bt[3];
-    wall_of(w[2], &fi.hasL, &fi.dL, fi.FBL);
-    wall_of(w[3], &fi.hasR, &fi.dR, fi.FBR);
+    wall_of(2, &fi.hasL, &fi.dL, fi.FBL);
+    wall_of(3, &fi.hasR, &fi.dR, fi.FBR);
     face_stab<T>(I.eq, g, dir, lamT, av0, av1, I.nc, &w[1], &fi, Fhi);
     for (int q = 0; q < MAXC; ++q) {
         b.Flo[q] = Flo[q];
