@@ -54,7 +54,29 @@ struct Body3 {
     int np;
     double n[3 * MAXP];
     double c[MAXP];     // offsets of the posed planes
+    float nf[3 * MAXP], cf[MAXP];   // the same in FP32 (side_of only)
 };
+
+// The box [lo, lo + h] (FP32, h >= 0, |lo| + h formed from terms of magnitude
+// up to big) against plane f: 1 it lies outside, -1 it lies inside, 0 not
+// decided.  Every FP64 corner's distance differs from its FP32 value by less
+// than the margin (the rounding of the inputs and of the sums is below 12 x
+// 2^-24 of the terms' magnitudes, the margin 4e-6 of them), so a decision is
+// the FP64 tests' too.  Most of R is decided so, off the FP64 pipe (44 x 44 x
+// 24 cells, two poses: 672 us per launch with FP64 tests, 418 so; 9.9 M FP64
+// warp instructions against 4.9 M).
+__device__ __forceinline__ int side_of(const Body3 &B, int f, const float *lo, const float *h, const float *big) {
+    float c = B.cf[f], least = 0.0f, most = 0.0f, mag = fabsf(c);
+    for (int a = 0; a < 3; ++a) {
+        const float n = B.nf[3 * f + a], e = n * h[a];
+        c -= n * lo[a];
+        least += fminf(e, 0.0f);
+        most += fmaxf(e, 0.0f);
+        mag += fabsf(n) * big[a];
+    }
+    const float m = 4e-6f * mag;
+    return least - c > m ? 1 : most - c < -m ? -1 : 0;
+}
 
 __host__ __device__ inline double dot3(const double *a, const double *b) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; }
 
@@ -175,6 +197,15 @@ __device__ double box_solid_volume(const Body3 &B, const double *lo, const doubl
     return fmin(vol, fmax(0.0, V / 3.0));
 }
 
+// all 32 lanes of a warp: 1 the box lies outside the body, -1 inside, 0 not
+// decided by FP32
+__device__ __forceinline__ int box_side(const Body3 &B, const float *lo, const float *h, const float *big) {
+    const int lane = threadIdx.x & 31;
+    const int s = lane < B.np ? side_of(B, lane, lo, h, big) : -1;
+    if (__any_sync(0xffffffffu, s > 0)) return 1;
+    return __all_sync(0xffffffffu, s < 0) ? -1 : 0;
+}
+
 // solid area of the rectangle {x_a = v} x [lb, lb + wb] x [lc, lc + wc]
 // (b, c the axes after a, cyclically): the rectangle clipped by the body's
 // planes, in coordinates relative to (lb, lc)
@@ -182,8 +213,19 @@ __device__ double rect_solid_area(const Body3 &B, int a, double v, double lb, do
     const int b = (a + 1) % 3, c = (a + 2) % 3;
     // the planes against the rectangle's corners first: none inside one
     // plane leaves no solid, all inside one leaves that plane out
-    unsigned cut = 0;
+    // (first in FP32, as side_of, which decides most planes)
+    unsigned cut = 0, test = 0;
+    const float fv = (float)v, fb = (float)lb, fc = (float)lc, hb = (float)wb, hc = (float)wc;
+    const float sv = fabsf(fv), sb = fabsf(fb) + hb, sc = fabsf(fc) + hc;
     for (int f = 0; f < B.np; ++f) {
+        const float na = B.nf[3 * f + a], nb = B.nf[3 * f + b], nc = B.nf[3 * f + c];
+        const float d = B.cf[f] - na * fv - nb * fb - nc * fc, eb = nb * hb, ec = nc * hc;
+        const float m = 4e-6f * (fabsf(B.cf[f]) + fabsf(na) * sv + fabsf(nb) * sb + fabsf(nc) * sc);
+        if (fminf(eb, 0.0f) + fminf(ec, 0.0f) - d > m) return 0.0;
+        if (!(fmaxf(eb, 0.0f) + fmaxf(ec, 0.0f) - d < -m)) test |= 1u << f;
+    }
+    for (; test; test &= test - 1) {
+        const int f = __ffs(test) - 1;
         const double *nn = &B.n[3 * f];
         const double cc = B.c[f] - nn[a] * v - nn[b] * lb - nn[c] * lc;
         const double lo_ = (nn[b] < 0.0 ? nn[b] * wb : 0.0) + (nn[c] < 0.0 ? nn[c] * wc : 0.0) - cc;
@@ -235,6 +277,8 @@ __device__ double rect_solid_area(const Body3 &B, int a, double v, double lb, do
 struct Desc {
     int nx, ny, nz, n;
     double lo[3], h[3];
+    float lof[3], hf[3];    // the same in FP32 (side_of only)
+    float bigf[3];          // |lo| + the extent + a cell: bounds every coordinate formed
     int bc[6];
     double gamma, U[3];
     int gcl;
@@ -400,12 +444,17 @@ __global__ void k3_cells(Desc D, Body3 BA, Body3 BM, Body3 BB, int mode) {
     const int t = w % rc, pose = w / rc;   // 0: B, 1: M, 2: A
     int i, j, k;
     r_cell(D, t, &i, &j, &k);
-    const double lo[3] = {node(D, 0, i), node(D, 1, j), node(D, 2, k)};
-    const double hi[3] = {node(D, 0, i + 1), node(D, 1, j + 1), node(D, 2, k + 1)};
-    const double h[3] = {hi[0] - lo[0], hi[1] - lo[1], hi[2] - lo[2]};
-    const double vol = h[0] * h[1] * h[2];
-    bool touch;
-    const double a = fraction(box_solid_volume(pose == 0 ? BB : pose == 1 ? BM : BA, lo, h, &touch), vol);
+    const Body3 &B = pose == 0 ? BB : pose == 1 ? BM : BA;
+    const float fl[3] = {D.lof[0] + i * D.hf[0], D.lof[1] + j * D.hf[1], D.lof[2] + k * D.hf[2]};
+    const int side = box_side(B, fl, D.hf, D.bigf);
+    bool touch = false;
+    double a = side > 0 ? 1.0 : 0.0;   // no solid, or solid throughout
+    if (side == 0) {
+        const double lo[3] = {node(D, 0, i), node(D, 1, j), node(D, 2, k)};
+        const double hi[3] = {node(D, 0, i + 1), node(D, 1, j + 1), node(D, 2, k + 1)};
+        const double h[3] = {hi[0] - lo[0], hi[1] - lo[1], hi[2] - lo[2]};
+        a = fraction(box_solid_volume(B, lo, h, &touch), h[0] * h[1] * h[2]);
+    }
     if ((threadIdx.x & 31) != 0) return;
     if (pose == 0) {
         D.aB[t] = a;
@@ -464,6 +513,21 @@ __global__ void k3_swept(Desc D, Body3 BA, double delta) {
     const int m0 = D.rn[0] + (ax == 0), m1 = D.rn[1] + (ax == 1), m2 = D.rn[2] + (ax == 2);
     if (t >= m0 * m1 * m2) return;
     const int ijk[3] = {D.r0[0] + t % m0, D.r0[1] + (t / m0) % m1, D.r0[2] + t / (m0 * m1)};
+    {
+        float fl[3], fh[3], big[3];
+        const float dl = (float)delta;
+        for (int q = 0; q < 3; ++q) {
+            const bool m = q == ax;
+            fl[q] = D.lof[q] + ijk[q] * D.hf[q] - (m && dl > 0.0f ? dl : 0.0f);
+            fh[q] = m ? fabsf(dl) : D.hf[q];
+            big[q] = D.bigf[q] + (m ? fabsf(dl) : 0.0f);
+        }
+        const int side = box_side(BA, fl, fh, big);
+        if (side != 0) {
+            if ((threadIdx.x & 31) == 0) D.bt[t] = side > 0 ? 1.0 : 0.0;
+            return;
+        }
+    }
     double lo[3], h[3];
     for (int q = 0; q < 3; ++q) { lo[q] = node(D, q, ijk[q]); h[q] = node(D, q, ijk[q] + 1) - lo[q]; }
     const double xf = node(D, ax, ijk[ax]);
@@ -1655,8 +1719,12 @@ static mb3::Body3 posed(const mb3_sim *s, const double *T) {
     memset(&B, 0, sizeof(B));
     B.np = s->nplane;
     for (int f = 0; f < s->nplane; ++f) {
-        for (int a = 0; a < 3; ++a) B.n[3 * f + a] = s->pn[3 * f + a];
+        for (int a = 0; a < 3; ++a) {
+            B.n[3 * f + a] = s->pn[3 * f + a];
+            B.nf[3 * f + a] = (float)s->pn[3 * f + a];
+        }
         B.c[f] = s->pc[f] + (s->pn[3 * f] * T[0] + s->pn[3 * f + 1] * T[1] + s->pn[3 * f + 2] * T[2]);
+        B.cf[f] = (float)B.c[f];
     }
     return B;
 }
@@ -1768,6 +1836,9 @@ mb_status mb3_create(const mb3_grid *g, double gamma, double cfl, const mb3_body
     for (int a = 0; a < 3; ++a) {
         D.lo[a] = g->lo[a];
         D.h[a] = (g->hi[a] - g->lo[a]) / nn[a];
+        D.lof[a] = (float)D.lo[a];
+        D.hf[a] = (float)D.h[a];
+        D.bigf[a] = (float)(std::fabs(g->lo[a]) + (g->hi[a] - g->lo[a]) + 2.0 * D.h[a]);
         D.U[a] = b->U[a];
     }
     for (int q = 0; q < 6; ++q) D.bc[q] = g->bc[q];
