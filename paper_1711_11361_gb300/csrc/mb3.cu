@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -1683,10 +1684,18 @@ struct mb3_sim {
     size_t rcap = 0, rfcap = 0;
     bool prev_ok = false;        // aB / tB hold the current pose over the region q0, qn
     int q0[3] = {0, 0, 0}, qn[3] = {0, 0, 0};
-    double wall_host[NC] = {0, 0, 0, 0, 0};
-    int merged = 0;
+    // what a sweep reports (device: D.wall .. D.err in one block; host: one
+    // page-locked slot per sweep of a step, filled without waiting)
+    struct Report {
+        double wall[NC];
+        int mixed, nseed, err, pad;
+    };
+    Report *dev_report = nullptr, *report = nullptr;
+    int last_report = 0;
+    double *smax_host = nullptr;
     cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};   // around the last sweep's two line launches
     float flux_ms = 0.0f;
+    bool near_timed = false;
     std::vector<void *> owned;
 };
 
@@ -1866,15 +1875,23 @@ mb_status mb3_create(const mb3_grid *g, double gamma, double cfl, const mb3_body
     if (e == cudaSuccess) e = dalloc(s, &D.Qn, NC * n);
     if (e == cudaSuccess) e = dalloc(s, &D.C, NC * n);
     if (e == cudaSuccess) e = dalloc(s, &D.Cn, NC * n);
-    if (e == cudaSuccess) e = dalloc(s, &D.err, 1);
-    if (e == cudaSuccess) e = dalloc(s, &D.wall, NC);
+    if (e == cudaSuccess) e = dalloc(s, &s->dev_report, 1);
+    if (e == cudaSuccess) {
+        D.wall = s->dev_report->wall;
+        D.mixed = &s->dev_report->mixed;
+        D.nseed = &s->dev_report->nseed;
+        D.err = &s->dev_report->err;
+        e = cudaHostAlloc((void **)&s->report, 3 * sizeof(mb3_sim::Report) + 3 * sizeof(double), cudaHostAllocDefault);
+    }
+    if (e == cudaSuccess) {
+        memset(s->report, 0, 3 * sizeof(mb3_sim::Report));
+        s->smax_host = (double *)(s->report + 3);
+    }
     if (e == cudaSuccess) e = dalloc(s, &D.seeds, mb3::SEEDCAP + mb3::NODECAP);
-    if (e == cudaSuccess) e = dalloc(s, &D.nseed, 1);
     if (e == cudaSuccess) e = dalloc(s, &D.lab, n);
     if (e == cudaSuccess) e = dalloc(s, &D.par_, mb3::NODECAP);
     if (e == cudaSuccess) e = dalloc(s, &D.nodes, mb3::NODECAP);
     if (e == cudaSuccess) e = dalloc(s, &D.ntot, (NC + 1) * (size_t)mb3::NODECAP);
-    if (e == cudaSuccess) e = dalloc(s, &D.mixed, 1);
     if (e == cudaSuccess) e = dalloc(s, &D.smax, 3);
     if (e == cudaSuccess) e = cudaMemsetAsync(D.lab, 0xff, n * sizeof(int), s->st);
     if (e == cudaSuccess) e = cudaMemsetAsync(D.err, 0, sizeof(int), s->st);
@@ -1894,6 +1911,7 @@ void mb3_destroy(mb3_sim *s) {
     if (s->st) cudaStreamSynchronize(s->st);
     for (int q = 0; q < 3; ++q) if (s->gs[q]) cudaStreamSynchronize(s->gs[q]);
     for (void *p : s->owned) cudaFree(p);
+    if (s->report) cudaFreeHost(s->report);
     for (int q = 0; q < 4; ++q) if (s->ev[q]) cudaEventDestroy(s->ev[q]);
     if (s->fork) cudaEventDestroy(s->fork);
     for (int q = 0; q < 3; ++q) {
@@ -1995,9 +2013,9 @@ static void line_sweep(const Desc &D, bool near, cudaStream_t st) {
 }
 }
 
-mb_status mb3_sweep(mb3_sim *s, int d, double dt) {
-    if (!s || d < 0 || d > 2 || !(dt > 0.0)) return MB_E_INVAL;
-    if (s->sidx > 0 && dt != s->dt_step) return fail3(s, MB_E_STATE, "the sweeps of a step must share dt");
+// one sweep's work on the streams, its report into slot `slot`, nothing
+// waited for (nothing of the queue depends on a result on the host)
+static mb_status queue_sweep(mb3_sim *s, int d, double dt, int slot) {
     cudaError_t e = cudaSuccess;
     const double delta = s->D.U[d] * dt;
     double TA[3] = {s->T[0], s->T[1], s->T[2]}, TM[3] = {TA[0], TA[1], TA[2]}, TB[3] = {TA[0], TA[1], TA[2]};
@@ -2027,9 +2045,7 @@ mb_status mb3_sweep(mb3_sim *s, int d, double dt) {
     D.d = d;
     D.lam = dt / D.h[d];
     D.hlamf = 0.5f * (float)D.lam;
-    if (e == cudaSuccess) e = cudaMemsetAsync(D.wall, 0, NC * sizeof(double), s->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(D.nseed, 0, sizeof(int), s->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(D.mixed, 0, sizeof(int), s->st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s->dev_report, 0, offsetof(mb3_sim::Report, err), s->st);
     if (e != cudaSuccess) return cuda3(s, e, "mb3_sweep");
     const mb3::Body3 BA = posed(s, TA), BM = posed(s, TM), BB = posed(s, TB);
     if (rc > 0) {
@@ -2078,31 +2094,52 @@ mb_status mb3_sweep(mb3_sim *s, int d, double dt) {
     s->D.Qn = D.Qn;
     s->D.Q = D.Cn;
     std::swap(s->D.Qf, s->D.Qfn);
-    int w = 0;
     e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(s->wall_host, D.wall, NC * sizeof(double), cudaMemcpyDeviceToHost, s->st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&s->merged, D.mixed, sizeof(int), cudaMemcpyDeviceToHost, s->st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&w, D.err, sizeof(int), cudaMemcpyDeviceToHost, s->st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(s->report + slot, s->dev_report, sizeof(mb3_sim::Report), cudaMemcpyDeviceToHost, s->st);
     if (e != cudaSuccess) return cuda3(s, e, "mb3_sweep");
     s->prev_ok = true;
     for (int a = 0; a < 3; ++a) { s->q0[a] = r0[a]; s->qn[a] = rn[a]; }
-    float near_ms = 0.0f;
-    cudaEventElapsedTime(&s->flux_ms, s->ev[0], s->ev[1]);
-    if (rc > 0) cudaEventElapsedTime(&near_ms, s->ev[2], s->ev[3]);
-    s->flux_ms += near_ms;
+    s->near_timed = rc > 0;
     s->T[d] = TB[d];
     if (++s->sidx == 3) {
         s->sidx = 0;
         s->t += dt;
         s->step++;
     }
-    return err_status(s, w);
+    return MB_OK;
+}
+// waits for the queued sweeps whose reports go to slots 0 .. n-1; the status
+// of the first that failed
+static mb_status finish_sweeps(mb3_sim *s, int n) {
+    const cudaError_t e = cudaStreamSynchronize(s->st);
+    if (e != cudaSuccess) {
+        s->prev_ok = false;
+        return cuda3(s, e, "mb3_sweep");
+    }
+    float far_ms = 0.0f, near_ms = 0.0f;
+    cudaEventElapsedTime(&far_ms, s->ev[0], s->ev[1]);
+    if (s->near_timed) cudaEventElapsedTime(&near_ms, s->ev[2], s->ev[3]);
+    s->flux_ms = far_ms + near_ms;
+    s->last_report = n - 1;
+    mb_status first = MB_OK;
+    for (int m = 0; m < n; ++m) {
+        const mb_status r = err_status(s, s->report[m].err);
+        if (first == MB_OK) first = r;
+    }
+    return first;
+}
+
+mb_status mb3_sweep(mb3_sim *s, int d, double dt) {
+    if (!s || d < 0 || d > 2 || !(dt > 0.0)) return MB_E_INVAL;
+    if (s->sidx > 0 && dt != s->dt_step) return fail3(s, MB_E_STATE, "the sweeps of a step must share dt");
+    const mb_status r = queue_sweep(s, d, dt, 0);
+    return r != MB_OK ? r : finish_sweeps(s, 1);
 }
 
 mb_status mb3_cfl_dt(mb3_sim *s, double *dt) {
     if (!s || !dt) return MB_E_INVAL;
-    double sm[3] = {0, 0, 0};
+    double *sm = s->smax_host;
     cudaError_t e = cudaMemsetAsync(s->D.smax, 0, 3 * sizeof(double), s->st);
     const unsigned nb = std::min(nblk(s->D.n), 152u * 8u);
     if (e == cudaSuccess && s->D.f32) mb3::k3_speeds32<<<nb, 256, 0, s->st>>>(s->D);
@@ -2131,20 +2168,24 @@ mb_status mb3_step(mb3_sim *s, double dt, double *dt_used) {
         if (r != MB_OK) return r;
     }
     if (dt_used) *dt_used = dt;
+    if (!(dt > 0.0)) return MB_E_INVAL;
+    // the three sweeps queued together: the host waits once per step
     const bool odd = s->step & 1;
-    mb_status first = MB_OK;
     for (int m = 0; m < 3; ++m) {
-        const mb_status r = mb3_sweep(s, odd ? 2 - m : m, dt);
-        if (r != MB_OK && first == MB_OK) first = r;
-        if (r == MB_E_CUDA || r == MB_E_NOMEM || r == MB_E_INVAL || r == MB_E_STATE) return r;
+        const mb_status r = queue_sweep(s, odd ? 2 - m : m, dt, m);
+        if (r != MB_OK) {
+            cudaStreamSynchronize(s->st);
+            return r;
+        }
     }
-    return first;
+    return finish_sweeps(s, 3);
 }
 
 mb_status mb3_last_sweep(mb3_sim *s, double *wall, int *merged) {
     if (!s) return MB_E_INVAL;
-    if (wall) for (int q = 0; q < NC; ++q) wall[q] = s->wall_host[q];
-    if (merged) *merged = s->merged;
+    const mb3_sim::Report &r = s->report[s->last_report];
+    if (wall) for (int q = 0; q < NC; ++q) wall[q] = r.wall[q];
+    if (merged) *merged = r.mixed;
     return MB_OK;
 }
 
