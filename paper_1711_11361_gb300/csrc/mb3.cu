@@ -281,10 +281,10 @@ struct Desc {
     float lof[3], hf[3];    // the same in FP32 (side_of only)
     float bigf[3];          // |lo| + the extent + a cell: bounds every coordinate formed
     int bc[6];
-    double gamma, U[3];
+    double gamma, g1h, U[3];   // g1h: (gamma - 1) / 2
     int gcl;
     int d;                  // the sweep's direction
-    double lam;             // dt / h_d
+    double lam, hlam;       // dt / h_d and its half
     int r0[3], rn[3];       // region R: first cell and extent per axis
     double *Q, *Qn;         // the state at the sweep's and at the step's start
     double *C;              // contents before the events (R; alpha on its way out of mb3_read_state)
@@ -709,11 +709,11 @@ __device__ __forceinline__ float vanleer(float dm, float dp) {
 template <typename T, int d> struct Flow;
 template <int d> struct Flow<double, d> {
     using S = Side<NC>;
-    double g, g1, hl;
-    __device__ __forceinline__ explicit Flow(const Desc &D) : g(D.gamma), g1(D.gamma - 1.0), hl(0.5 * D.lam) {}
+    double g, h1, hl;
+    __device__ __forceinline__ explicit Flow(const Desc &D) : g(D.gamma), h1(D.g1h), hl(D.hlam) {}
     __device__ __forceinline__ void states(const double *qm, const double *q0, const double *qp, bool lim, S &L,
                                            S &R) const {
-        evolve64<NC, d>(g1, hl, qm, q0, qp, lim, L, R);
+        evolve64<NC, d>(h1, hl, qm, q0, qp, lim, L, R);
     }
     __device__ __forceinline__ void flux(const S &L, const S &R, double *F) const { hllc64<NC, d>(g, L, R, F); }
 };
@@ -1611,7 +1611,7 @@ __global__ void __launch_bounds__(256) k3_speeds64(Desc D) {
             const long long c = c0 + u * 256 + threadIdx.x;
             double q[NC];
             for (int k = 0; k < NC; ++k) q[k] = D.Q[(size_t)k * D.n + c];
-            const double ir = rcp64(q[0]), p = press64<NC>(g - 1.0, q, ir), cs = sqrt64(g * (p * ir));
+            const double ir = rcp64(q[0]), p = press64<NC>(D.g1h, q, ir), cs = sqrt64(g * (p * ir));
             for (int a = 0; a < 3; ++a) {
                 const double x = __fma_rn(abs64(q[1 + a]), ir, cs);
                 if (pos64(x)) s[a] = max64(s[a], x);
@@ -1852,6 +1852,7 @@ mb_status mb3_create(const mb3_grid *g, double gamma, double cfl, const mb3_body
     }
     for (int q = 0; q < 6; ++q) D.bc[q] = g->bc[q];
     D.gamma = gamma;
+    D.g1h = 0.5 * (gamma - 1.0);
     D.gammaf = (float)gamma;
     D.gcl = uncover_mode == MB_UNCOVER_FLUX_GCL;
     s->cfl = cfl;
@@ -2044,6 +2045,7 @@ static mb_status queue_sweep(mb3_sim *s, int d, double dt, int slot) {
     for (int a = 0; a < 3; ++a) { D.r0[a] = r0[a]; D.rn[a] = rn[a]; }
     D.d = d;
     D.lam = dt / D.h[d];
+    D.hlam = 0.5 * D.lam;
     D.hlamf = 0.5f * (float)D.lam;
     if (e == cudaSuccess) e = cudaMemsetAsync(s->dev_report, 0, offsetof(mb3_sim::Report, err), s->st);
     if (e != cudaSuccess) return cuda3(s, e, "mb3_sweep");

@@ -271,6 +271,7 @@ static void describe_instance(int prec, int yseg, const mb_grid &g, double gamma
     I.ucov = g.uncover_mode;
     I.adv[0] = g.adv[0]; I.adv[1] = g.adv[1];
     I.gamma = gamma;
+    I.g1h = 0.5 * (gamma - 1.0);
     I.cfl = g.cfl;
     I.U[0] = m.U[0]; I.U[1] = m.U[1];
     I.pivot[0] = m.pivot[0]; I.pivot[1] = m.pivot[1];

@@ -76,6 +76,20 @@ __device__ __forceinline__ double max64(double a, double b) { return key64(a) < 
 __device__ __forceinline__ double abs64(double x) {
     return __hiloint2double(__double2hiint(x) & 0x7fffffff, __double2loint(x));
 }
+// 2 x and x / 2 by the exponent field, for 0 and 2^-1020 <= |x| <= 2^1022
+// (infinities and NaN stay; no multiplication as a second case, which the
+// compiler would issue for every x and select from)
+__device__ __forceinline__ double twice64(double x) {
+    const int hi = __double2hiint(x);
+    const bool normal = (unsigned)(hi & 0x7ff00000) - 0x100000u < 0x7fe00000u;
+    return __hiloint2double(normal ? hi + 0x100000 : hi, __double2loint(x));
+}
+__device__ __forceinline__ double half64(double x) {
+    const int hi = __double2hiint(x);
+    const bool normal = (unsigned)(hi & 0x7ff00000) - 0x100000u < 0x7fe00000u;
+    return __hiloint2double(normal ? hi - 0x100000 : hi, __double2loint(x));
+}
+
 // x rounded to float (to nearest, ties to even) by integer instructions where
 // the result is a normal float or zero, else by the conversion
 __device__ __forceinline__ float narrow32(double x) {
@@ -111,9 +125,10 @@ __device__ __forceinline__ double msq64(const double *q) {   // |m|^2
     for (int k = NC - 3; k >= 1; --k) s = __fma_rn(q[k], q[k], s);
     return s;
 }
+// pressure, h1 = (gamma - 1) / 2
 template <int NC>
-__device__ __forceinline__ double press64(double g1, const double *q, double ir) {
-    return g1 * __fma_rn(-0.5 * msq64<NC>(q), ir, q[NC - 1]);
+__device__ __forceinline__ double press64(double h1, const double *q, double ir) {
+    return h1 * __fma_rn(-msq64<NC>(q), ir, twice64(q[NC - 1]));
 }
 // rho > 0 and 2 rho E > |m|^2, in FP32 where that decides with a margin of
 // 1e-5 (its error is below 2e-6), else in FP64
@@ -132,12 +147,13 @@ __device__ __forceinline__ bool physical64(const double *q) {
     return pos64(q[0]) && 2.0 * q[0] * q[NC - 1] > msq64<NC>(q) && q[NC - 1] - q[NC - 1] == 0.0;
 }
 // MUSCL-Hancock evolved states of one cell: van Leer slopes in conserved
-// variables (none where !lim), half-step evolution (hl = dt / 2h), first order
+// variables (none where !lim), half-step evolution (hl = dt / 2h, h1 =
+// (gamma - 1) / 2), first order
 // where an evolved state is not physical.  One reciprocal of the product of
 // two densities serves both sides; the positivity tests use the pressures
 // that the Riemann solver takes.
 template <int NC, int D>
-__device__ __forceinline__ void evolve64(double g1, double hl, const double *qm, const double *q0, const double *qp,
+__device__ __forceinline__ void evolve64(double h1, double hl, const double *qm, const double *q0, const double *qp,
                                          bool lim, Side<NC> &L, Side<NC> &R) {
     constexpr int in = 1 + D, E = NC - 1;
     double l[NC], r[NC];
@@ -153,7 +169,7 @@ __device__ __forceinline__ void evolve64(double g1, double hl, const double *qm,
     }
     double rr = rcp64(l[0] * r[0]);
     const double il = r[0] * rr, ig = l[0] * rr;
-    const double pl = press64<NC>(g1, l, il), pg = press64<NC>(g1, r, ig);
+    const double pl = press64<NC>(h1, l, il), pg = press64<NC>(h1, r, ig);
     const double ul = l[in] * il, ug = r[in] * ig;
 #pragma unroll
     for (int k = 0; k < NC; ++k) {
@@ -168,13 +184,13 @@ __device__ __forceinline__ void evolve64(double g1, double hl, const double *qm,
     rr = rcp64(L.q[0] * R.q[0]);
     L.ir = R.q[0] * rr;
     R.ir = L.q[0] * rr;
-    L.p = press64<NC>(g1, L.q, L.ir);
-    R.p = press64<NC>(g1, R.q, R.ir);
+    L.p = press64<NC>(h1, L.q, L.ir);
+    R.p = press64<NC>(h1, R.q, R.ir);
     if (!(pos64(L.q[0]) && pos64(R.q[0]) && pos64(L.p) && pos64(R.p))) {
 #pragma unroll
         for (int k = 0; k < NC; ++k) L.q[k] = R.q[k] = q0[k];
         L.ir = R.ir = rcp64(q0[0]);
-        L.p = R.p = press64<NC>(g1, q0, L.ir);
+        L.p = R.p = press64<NC>(h1, q0, L.ir);
     }
 }
 // HLLC flux with Davis wave speeds (Toro, ch. 10), the star flux in the form

@@ -87,6 +87,7 @@ struct InstDesc {
     int ucov;
     double adv[2];
     double gamma, cfl;
+    double g1h;          // (gamma - 1) / 2
     void *Q[3];          // state buffers (T*), plane stride pitch*ny
     uint8_t *cls;
     int *rec;

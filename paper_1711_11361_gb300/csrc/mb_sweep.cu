@@ -388,7 +388,7 @@ struct FaceIn {
 };
 
 template <class T>
-__device__ __noinline__ void face_stab(int eq, T g, int dir, T lamT, T av0, T av1, int nc, const CellW<T> *w,
+__device__ __noinline__ void face_stab(int eq, T g, double h1, int dir, T lamT, T av0, T av1, int nc, const CellW<T> *w,
                                        const FaceIn *in, double *out) {
     for (int q = 0; q < MAXC; ++q) out[q] = 0.0;
     if (!(w[1].fluid && w[2].fluid && in->btF > 0.0)) return;
@@ -398,9 +398,9 @@ __device__ __noinline__ void face_stab(int eq, T g, int dir, T lamT, T av0, T av
         auto fluxes = [&](auto dc) {
             constexpr int DC = decltype(dc)::value;
             Side<4> x, a, b;
-            const double g1 = (double)g - 1.0, hl = 0.5 * (double)lamT;
-            evolve64<4, DC>(g1, hl, (const double *)w[0].q, (const double *)w[1].q, (const double *)w[2].q, limA, x, a);
-            evolve64<4, DC>(g1, hl, (const double *)w[1].q, (const double *)w[2].q, (const double *)w[3].q, limB, b, x);
+            const double hl = half64((double)lamT);
+            evolve64<4, DC>(h1, hl, (const double *)w[0].q, (const double *)w[1].q, (const double *)w[2].q, limA, x, a);
+            evolve64<4, DC>(h1, hl, (const double *)w[1].q, (const double *)w[2].q, (const double *)w[3].q, limB, b, x);
             hllc64<4, DC>((double)g, a, b, (double *)F);
         };
         if (dir == 0) fluxes(std::integral_constant<int, 0>());
@@ -515,12 +515,12 @@ __device__ __forceinline__ bool band_sweep_rec(const InstDesc *__restrict__ D, I
     wall_of(1, &fi.hasL, &fi.dL, fi.FBL);
     wall_of(2, &fi.hasR, &fi.dR, fi.FBR);
     double Flo[MAXC], Fhi[MAXC];
-    face_stab<T>(I.eq, g, dir, lamT, av0, av1, I.nc, &w[0], &fi, Flo);
+    face_stab<T>(I.eq, g, I.g1h, dir, lamT, av0, av1, I.nc, &w[0], &fi, Flo);
     // high face: cells k | k+1
     fi.btL = bt[1]; fi.btF = bt[2]; fi.btR = bt[3];
     wall_of(2, &fi.hasL, &fi.dL, fi.FBL);
     wall_of(3, &fi.hasR, &fi.dR, fi.FBR);
-    face_stab<T>(I.eq, g, dir, lamT, av0, av1, I.nc, &w[1], &fi, Fhi);
+    face_stab<T>(I.eq, g, I.g1h, dir, lamT, av0, av1, I.nc, &w[1], &fi, Fhi);
     for (int q = 0; q < MAXC; ++q) {
         b.Flo[q] = Flo[q];
         b.Fhi[q] = Fhi[q];
@@ -599,7 +599,7 @@ __device__ __forceinline__ void finish_warp<double>(InstDyn &y, bool last, doubl
             m0 = max(m0, __shfl_xor_sync(0xffffffffu, m0, o));
             m1 = max(m1, __shfl_xor_sync(0xffffffffu, m1, o));
         }
-        if ((threadIdx.x & 31) == 0) {
+        if ((threadIdx.x & 31) == 0 && (m0 | m1)) {
             atomicMax(&y.S[0], m0);
             atomicMax(&y.S[1], m1);
         }
@@ -622,9 +622,9 @@ __device__ __forceinline__ int find_inst_warp(const InstDesc *D, int n_inst, int
 // them (about 150 of its lane operations per cell), so what counts is that
 // every SM has some: one unit per warp spreads a 400 x 400 grid over 5600
 // warps, where a warp per row (x) or per 64 rows (y) left most SMs idle.
-// Measured per sweep, FP64 Euler, before -> after: 399 x 399, x 286 -> 76 us,
-// y 1380 -> 94 us (its two launches together); 9.8 M cells in 16 grids, x
-// 2950 -> 1604 us, y 4090 -> 1617 us, 0.85 of the FP64 pipe's rate for the 88
+// Measured per sweep, FP64 Euler, before -> after: 399 x 399, x 286 -> 73 us,
+// y 1380 -> 90 us (its two launches together); 9.8 M cells in 16 grids, x
+// 2950 -> 1428 us, y 4090 -> 1430 us, 0.86 of the FP64 pipe's rate for the 79
 // lane operations per cell this flow executes (with the division, square
 // root and comparisons of CUDA: 188 or more).
 constexpr int UNIT_CELLS = 30;
@@ -650,13 +650,14 @@ template <>
 struct Flow<double, 0> {          // Euler, FP64
     static constexpr int NC = 4;
     using S = Side<4>;
-    double g, g1, lam, hl;
+    double g, h1, lam, hl;
+    float gf, h1f;
     __device__ __forceinline__ Flow(const InstDesc &I, double l, int)
-        : g(I.gamma), g1(I.gamma - 1.0), lam(l), hl(0.5 * l) {}
+        : g(I.gamma), h1(I.g1h), lam(l), hl(half64(l)), gf(narrow32(g)), h1f(narrow32(h1)) {}
     template <int D>
     __device__ __forceinline__ void states(const double *qm, const double *q0, const double *qp, bool lim, S &L,
                                            S &R) const {
-        evolve64<4, D>(g1, hl, qm, q0, qp, lim, L, R);
+        evolve64<4, D>(h1, hl, qm, q0, qp, lim, L, R);
     }
     template <int D>
     __device__ __forceinline__ void flux(const S &L, const S &R, double *F) const { hllc64<4, D>(g, L, R, F); }
@@ -670,15 +671,28 @@ __device__ __forceinline__ void up_state(Side<4> &s) {
 template <class S>
 __device__ __forceinline__ void up_state(S &s) { s.q[0] = __shfl_up_sync(0xffffffffu, s.q[0], 1); }
 
-// new state of a lane's cell (qn), with the positivity and wave-speed checks
-// of update_cell
+// new state of a lane's cell (qn), with the positivity check and, on the
+// step's last sweep, the wave speeds s0, s1.  The speeds are first formed in
+// FP32 (error below 4e-6 where p > E / 10): only a cell within 1e-5 of the
+// instance's largest so far (m0, m1: y.S read before), or with a smaller
+// pressure, goes through FP64, so the maxima are those over every cell
 __device__ __forceinline__ void new_state(const Flow<double, 0> &f, const double *q, const double *Flo,
-                                          const double *Fhi, bool last, int ci, InstDyn &y, double *qn, double &s0,
-                                          double &s1) {
+                                          const double *Fhi, bool last, int ci, InstDyn &y, float m0, float m1,
+                                          double *qn, double &s0, double &s1) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) qn[k] = __fma_rn(f.lam, Flo[k] - Fhi[k], q[k]);
     if (last) {
-        const double ir = rcp64(qn[0]), p = press64<4>(f.g1, qn, ir);
+        bool ok = true;
+        float x[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) x[k] = near32(qn[k], ok);
+        const float ir32 = __fdividef(1.0f, x[0]);
+        const float p32 = f.h1f * fmaf(-fmaf(x[1], x[1], x[2] * x[2]), ir32, 2.0f * x[3]);
+        if (ok && x[0] > 1e-30f && x[3] < 1e30f && p32 > 0.1f * x[3]) {   // (positive with a margin)
+            const float cs = sqrtf(f.gf * p32 * ir32);
+            if (fabsf(x[1] * ir32) + cs < m0 * (1.0f - 1e-5f) && fabsf(x[2] * ir32) + cs < m1 * (1.0f - 1e-5f)) return;
+        }
+        const double ir = rcp64(qn[0]), p = press64<4>(f.h1, qn, ir);
         if (!pos64(qn[0]) || !pos64(p)) list_bulk_bad(y, ci);
         const double c = sqrt64(f.g * (p * ir));
         s0 = __fma_rn(abs64(qn[1]), ir, c);
@@ -689,7 +703,7 @@ __device__ __forceinline__ void new_state(const Flow<double, 0> &f, const double
 }
 template <class T>
 __device__ __forceinline__ void new_state(const Flow<T, 1> &f, const T *q, const T *Flo, const T *Fhi, bool, int,
-                                          InstDyn &, T *qn, T &, T &) {
+                                          InstDyn &, float, float, T *qn, T &, T &) {
     qn[0] = q[0] + f.lam * (Flo[0] - Fhi[0]);
 }
 
@@ -734,7 +748,16 @@ __device__ __forceinline__ bool unit_update(const InstDesc &I, InstDyn &y, const
         return true;
     }
     const int ci = DIR == 0 ? line * I.pitch + pos : pos * I.pitch + line;
-    new_state(f, q0, F, Fhi, last, ci, y, qn, s0, s1);
+    // the instance's largest speeds so far (they only grow during a sweep)
+    float m0 = 0.0f, m1 = 0.0f;
+    if (EQ == 0 && last) {
+        bool ok = true;
+        volatile const unsigned long long *S = y.S;
+        m0 = near32(__longlong_as_double((long long)S[0]), ok);
+        m1 = near32(__longlong_as_double((long long)S[1]), ok);
+        if (!ok) m0 = m1 = 0.0f;
+    }
+    new_state(f, q0, F, Fhi, last, ci, y, m0, m1, qn, s0, s1);
     if (EQ == 1 && last) {
         s0 = (T)fabs(I.adv[0]);
         s1 = (T)fabs(I.adv[1]);
@@ -2910,7 +2933,7 @@ __global__ void __launch_bounds__(STATE_THREADS) k_write_state(const InstDesc *_
         if (!((want >> u) & 1u)) continue;
         double q[MAXC];
         state(u, q);
-        const double ir = rcp64(q[0]), p = press64<4>(I.gamma - 1.0, q, ir), cs = sqrt64(I.gamma * (p * ir));
+        const double ir = rcp64(q[0]), p = press64<4>(I.g1h, q, ir), cs = sqrt64(I.gamma * (p * ir));
         w[u][0] = __fma_rn(abs64(q[1]), ir, cs);
         w[u][1] = __fma_rn(abs64(q[2]), ir, cs);
         if (pos64(w[u][0])) k0 = max(k0, (unsigned long long)__double_as_longlong(w[u][0]));
