@@ -29,6 +29,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "mb3.h"
@@ -744,14 +745,36 @@ template <int d> struct Flow<float, d> {
         if (!ok(L.q) || !ok(R.q))
             for (int k = 0; k < NC; ++k) { L.q[k] = q0[k]; R.q[k] = q0[k]; }
     }
-    // (fluxes are FP64 values either way, so that the update's differences
-    // F_lo - F_hi telescope as in the FP64 path)
+    __device__ __forceinline__ void flux(const S &L, const S &R, float *F) const { hllc5<d>(g, L.q, R.q, F); }
     __device__ __forceinline__ void flux(const S &L, const S &R, double *F) const {
         float f[NC];
         hllc5<d>(g, L.q, R.q, f);
         for (int k = 0; k < NC; ++k) F[k] = widen(f[k]);
     }
 };
+// the type of a face's flux: FP64 near the body, where it is stabilised
+template <typename T, bool GEN> using FluxT = std::conditional_t<GEN, double, T>;
+// F_lo - F_hi in FP64 (so that the update's differences telescope as in the
+// FP64 path).  FP32 fluxes: where all five FP32 differences are exact (their
+// rounding errors by Knuth's two-sum are zero: neighbouring fluxes mostly lie
+// within a factor of two) they are widened, else the fluxes are widened and
+// subtracted, the same values either way with five FP64 instructions fewer
+__device__ __forceinline__ void flux_diff(const double *lo, const double *hi, double *df) {
+    for (int k = 0; k < NC; ++k) df[k] = lo[k] - hi[k];
+}
+__device__ __forceinline__ void flux_diff(const float *lo, const float *hi, double *df) {
+    float s[NC];
+    bool exact = true;
+    for (int k = 0; k < NC; ++k) {
+        s[k] = lo[k] - hi[k];
+        const float b = s[k] - lo[k];
+        exact = exact && (lo[k] - (s[k] - b)) + (-hi[k] - b) == 0.0f;
+    }
+    if (exact)
+        for (int k = 0; k < NC; ++k) df[k] = widen(s[k]);
+    else
+        for (int k = 0; k < NC; ++k) df[k] = widen(lo[k]) - widen(hi[k]);
+}
 // the state array of the type T
 template <typename T> __device__ __forceinline__ const T *qsrc(const Desc &D);
 template <> __device__ __forceinline__ const double *qsrc<double>(const Desc &D) { return D.Q; }
@@ -828,8 +851,8 @@ __device__ __forceinline__ void stabilise(const Desc &D, const int *ijk, int f, 
 template <typename T, int d, bool GEN>
 __device__ __forceinline__ void line_flux(const Desc &D, const Flow<T, d> &fl, const int *line, int f, int nal,
                                           bool fluids, const typename Flow<T, d>::S &L, const typename Flow<T, d>::S &R,
-                                          double *F) {
-    if (GEN) {
+                                          FluxT<T, GEN> *F) {
+    if constexpr (GEN) {
         const bool periodic = D.bc[2 * d] == MB_BC_PERIODIC;
         int ijk[3] = {line[0], line[1], line[2]};
         ijk[d] = periodic && f == nal ? 0 : f;
@@ -845,14 +868,9 @@ __device__ __forceinline__ void line_flux(const Desc &D, const Flow<T, d> &fl, c
 }
 
 // the content update x = Q + lam (F_lo - F_hi) of a cell away from the body
-// (fused for the FP64 path; the FP32 option rounds each operation) and its
-// FP32 copy
-__device__ __forceinline__ double content(double lam, double q, double flo, double fhi, double) {
-    return __fma_rn(lam, flo - fhi, q);
-}
-__device__ __forceinline__ double content(double lam, double q, double flo, double fhi, float) {
-    return q + lam * (flo - fhi);
-}
+// (fused for the FP64 path; the FP32 option rounds each operation)
+__device__ __forceinline__ double content(double lam, double q, double df, double) { return __fma_rn(lam, df, q); }
+__device__ __forceinline__ double content(double lam, double q, double df, float) { return q + lam * df; }
 // alpha_B Q' = alpha_A Q + lam (F_lo - F_hi) + lam (beta_hi - beta_lo)(F^B -
 // w_d Q^B) (eqs. Klein2DcompleteMovingMethod2a-c) of cell m of the line
 // through ijk, index c, into Cn (in R also C and upd; elsewhere the FP32 copy
@@ -860,8 +878,9 @@ __device__ __forceinline__ double content(double lam, double q, double flo, doub
 // changes the content).  w: this thread's wall terms.
 template <typename T, int d, bool GEN>
 __device__ __forceinline__ void line_update(const Desc &D, const int *line, int m, int nal, int c, const double *Q,
-                                            const double *Flo, const double *Fhi, double *w) {
-    double v[NC];
+                                            const FluxT<T, GEN> *Flo, const FluxT<T, GEN> *Fhi, double *w) {
+    double v[NC], df[NC];
+    flux_diff(Flo, Fhi, df);
     if (GEN) {
         int ijk[3] = {line[0], line[1], line[2]};
         ijk[d] = m;
@@ -875,7 +894,7 @@ __device__ __forceinline__ void line_update(const Desc &D, const int *line, int 
             const bool wall = fl && D.whas[r] && blo != bhi;
             for (int q = 0; q < NC; ++q) {
                 v[q] = 0.0;
-                if (fl) v[q] = aA * Q[q] + D.lam * (Flo[q] - Fhi[q]);
+                if (fl) v[q] = aA * Q[q] + D.lam * df[q];
                 if (wall) {
                     const double wt = D.lam * (bhi - blo) * (D.wFB[(size_t)NC * r + q] -
                                                              D.U[d] * D.wQB[(size_t)NC * r + q]);
@@ -890,7 +909,7 @@ __device__ __forceinline__ void line_update(const Desc &D, const int *line, int 
         }
     }
     for (int q = 0; q < NC; ++q) {
-        v[q] = content(D.lam, Q[q], Flo[q], Fhi[q], T(0));
+        v[q] = content(D.lam, Q[q], df[q], T(0));
         D.Cn[(size_t)q * D.n + c] = v[q];
     }
     if (sizeof(T) == 4) {
@@ -953,11 +972,11 @@ __device__ __forceinline__ bool near_pos(const Near &N, int m, int nal) {
 // x sweep.  The line kernels keep the evolved states and the fluxes in
 // registers: per cell they read the state and write the new one (80 bytes; 120
 // with the FP32 copy), where a kernel each for the states, the fluxes, the
-// update and the new state moved 400.  FP64: bound by the FP64 pipe, 180 lane
-// operations per cell; 4 M cells per sweep, before -> after: x 2520 -> 1298
-// us, y 2400 -> 1395, z 2390 -> 1392 (0.85 of the pipe's rate).  FP32 option:
-// 15 FP64 lane operations per cell (the update) and about 700 instructions;
-// 32 M cells per sweep, 3790 -> 1002 us (x), 1104, 1133.  Rows are laid end
+// update and the new state moved 400.  FP64: bound by the FP64 pipe, 173 lane
+// operations per cell; 4 M cells per sweep, before -> after: x 2520 -> 1267
+// us, y 2400 -> 1369, z 2390 -> 1374 (0.85 of the pipe's rate).  FP32 option:
+// 10 FP64 lane operations per cell (the update) and about 700 instructions;
+// 32 M cells per sweep, 3790 -> 857 us (x), 1036, 1066.  Rows are laid end
 // to end as slots, position -1 .. nx of every row, and a warp takes 32 slots
 // from slot 30 w on: it evolves 32 positions, forms 31 fluxes and updates 30
 // cells, whatever the row length.
@@ -985,7 +1004,7 @@ __device__ __forceinline__ void row_unit(const Desc &D, bool store, int p, int j
         T *x = reinterpret_cast<T *>(&R);
         for (int m = 0; m < (int)(sizeof(R) / sizeof(T)); ++m) x[m] = __shfl_up_sync(0xffffffffu, x[m], 1);
     }
-    double F[NC], Fhi[NC];
+    FluxT<T, GEN> F[NC], Fhi[NC];
     line_flux<T, 0, GEN>(D, fl, line, max(p, 0), D.nx, fu[0] && fu[1], R, L, F);
     for (int m = 0; m < NC; ++m) Fhi[m] = __shfl_down_sync(0xffffffffu, F[m], 1);
     double w[NC] = {0, 0, 0, 0, 0};
@@ -1051,7 +1070,8 @@ __device__ __forceinline__ void march(const Desc &D, bool in, bool nearl, const 
     T qm[NC], qc[NC], qp[NC], qq[NC];
     bool um, uc, up, uq;
     S L, R, Rc;
-    double F[NC], Fp[NC], w[NC] = {0, 0, 0, 0, 0};
+    FluxT<T, GEN> F[NC], Fp[NC];
+    double w[NC] = {0, 0, 0, 0, 0};
     {
         T qa[NC];
         bool ua;
