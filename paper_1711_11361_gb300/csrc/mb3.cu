@@ -1244,7 +1244,7 @@ __global__ void k3_events(Desc D) {
 
 // safeguard seeds: non-physical new contents, and cells keeping less than
 // COLLAPSE of their volume over the sweep, in the list (cell indices)
-// (cells outside R are tested by k3_update, whose contents no later step
+// (cells outside R are tested by the line kernels, whose contents no later step
 // before the safeguard changes; this kernel runs over R, after the events)
 __global__ void k3_bad(Desc D) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;

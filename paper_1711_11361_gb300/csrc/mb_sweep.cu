@@ -7,9 +7,10 @@
 //   k_band_sweep  stabilised fluxes of every face touching a band cell
 //                 (eqs. Klein2shieldedFluxMethod2, Klein2DtotalfluxaMethod2) and
 //                 the band cells' new contents (eq. Klein2DcompleteMovingMethod2a)
-//   k_bulk        MUSCL-Hancock + HLLC standard fluxes and the conservative
-//                 update of every other cell (eq. EulerDiscreteRegular), SMEM
-//                 tiles over a persistent grid, CFL wave-speed reduction fused
+//   k_unit_x/_y   MUSCL-Hancock + HLLC standard fluxes and the conservative
+//   k_bulk_*      update of every other cell (eq. EulerDiscreteRegular), CFL
+//                 wave-speed reduction fused: scalar FP64 / FP32 units, and
+//                 FP32 Euler in cell pairs
 //   k_events      covering / uncovering redistribution, gathered per cell
 //                 (eqs. massDeficitEquation .. cutCellInitialisationDonorCellUpdate)
 //   k_mix         positivity safeguard (clusters share content by volume)
@@ -17,6 +18,7 @@
 #include "mb_internal.cuh"
 
 #include <algorithm>
+#include <climits>
 #include <type_traits>
 
 #include "mb_fp64.cuh"
@@ -2828,6 +2830,9 @@ constexpr int STATE_THREADS = 256;
 constexpr int STATE_UNROLL = 8;
 constexpr int STATE_CELLS = STATE_THREADS * STATE_UNROLL;
 
+__device__ __forceinline__ unsigned long long bits_of(double v) { return (unsigned long long)__double_as_longlong(v); }
+__device__ __forceinline__ unsigned long long bits_of(float v) { return __float_as_uint(v); }
+
 // Sources: srcs[blockIdx.y] (srcs != nullptr; a null entry skips that
 // instance) or src1.  The first step's wave speeds are the FP64 maxima over
 // the stored (T-rounded) states.  Each cell's speeds are first formed in
@@ -2836,16 +2841,19 @@ constexpr int STATE_CELLS = STATE_THREADS * STATE_UNROLL;
 // instance so far), or if its pressure is small against its energy (p <=
 // E/10, where the FP32 error could exceed 4e-6).  No skipped cell can
 // hold the maximum, so the result is that of the FP64 formula over every
-// cell.  H: the element type of the host layout (FP64 or FP32 states).
+// cell; cells in a state already taken drop out first.  H: the element type
+// of the host layout (FP64 or FP32 states).
 // 28.7 M cells whose speeds tie (the worst case): 3760 us with every cell
-// through the formula, 1185 us so; 400 x 400 cells 121 -> 40 us.
+// through the formula, 1185 us so; 400 x 400 cells 121 -> 40 us.  Uniform
+// states, whose cells a thread skipped as its last one's: 869 -> 1093 us.
 template <class T, class H>
-__global__ void __launch_bounds__(STATE_THREADS) k_write_state(const InstDesc *__restrict__ D,
+__global__ void __launch_bounds__(STATE_THREADS, 3) k_write_state(const InstDesc *__restrict__ D,
                                                                InstDyn *__restrict__ Y,
                                                                const H *const *__restrict__ srcs,
                                                                const H *__restrict__ src1, int inst0, int b) {
     __shared__ float red[2][STATE_THREADS / 32];
     __shared__ unsigned long long redk[2][STATE_THREADS / 32];
+    __shared__ int redi[STATE_THREADS / 32];
     const int inst = inst0 + blockIdx.y;
     const H *__restrict__ Qh = srcs ? srcs[blockIdx.y] : src1;
     if (!Qh) return;
@@ -2859,6 +2867,7 @@ __global__ void __launch_bounds__(STATE_THREADS) k_write_state(const InstDesc *_
     float v[STATE_UNROLL][2], m0 = 0.0f, m1 = 0.0f;
     unsigned want = 0u;
     bool fluid = false;
+    T lq[MAXC] = {T(0), T(0), T(0), T(0)};   // the thread's last distinct state (rho = 0: none)
 #pragma unroll
     for (int u = 0; u < STATE_UNROLL; ++u) {
         v[u][0] = v[u][1] = -1.0f;
@@ -2876,6 +2885,13 @@ __global__ void __launch_bounds__(STATE_THREADS) k_write_state(const InstDesc *_
         if (solid) continue;
         fluid = true;
         if (!euler) continue;
+        bool same = true;   // in a uniform region one cell per thread goes on
+#pragma unroll
+        for (int k = 0; k < MAXC; ++k) {
+            same = same && bits_of(q[k]) == bits_of(lq[k]);
+            lq[k] = q[k];
+        }
+        if (same) continue;
         bool ok = true;
         float x[MAXC];
 #pragma unroll
@@ -2918,13 +2934,43 @@ __global__ void __launch_bounds__(STATE_THREADS) k_write_state(const InstDesc *_
 #pragma unroll
     for (int u = 0; u < STATE_UNROLL; ++u)
         if (v[u][0] >= m0 * (1.0f - 1e-5f) || v[u][1] >= m1 * (1.0f - 1e-5f)) want |= 1u << u;
-    // the remaining cells' speeds by a few FP64 instructions (to 1e-15), then
-    // the formula itself for those within 1e-14 of the largest
     auto state = [&](int u, double *q) {
         const int e = e0 + u * STATE_THREADS + threadIdx.x;
 #pragma unroll
         for (int k = 0; k < MAXC; ++k) q[k] = (double)(T)Qh[(size_t)k * n + e];
     };
+    // Uniform regions: all remaining cells in the state of the first one but
+    // that one drop out, and so for the first of what is left (a shock's two
+    // sides), so that a uniform state costs one cell per CTA
+    unsigned kept = 0u;
+    for (int r = 0; r < 2; ++r) {
+        const int first = want ? e0 + (__ffs(want) - 1) * STATE_THREADS + (int)threadIdx.x : INT_MAX;
+        const int wf = __reduce_min_sync(0xffffffffu, first);
+        __syncthreads();
+        if ((threadIdx.x & 31) == 0) redi[threadIdx.x >> 5] = wf;
+        __syncthreads();
+        int ref = redi[0];
+#pragma unroll
+        for (int x = 1; x < STATE_THREADS / 32; ++x) ref = min(ref, redi[x]);
+        if (ref == INT_MAX) break;
+        T qr[MAXC];
+#pragma unroll
+        for (int k = 0; k < MAXC; ++k) qr[k] = (T)Qh[(size_t)k * n + ref];
+#pragma unroll
+        for (int u = 0; u < STATE_UNROLL; ++u) {
+            if (!((want >> u) & 1u)) continue;
+            const int e = e0 + u * STATE_THREADS + threadIdx.x;
+            bool same = true;
+#pragma unroll
+            for (int k = 0; k < MAXC; ++k) same = same && bits_of((T)Qh[(size_t)k * n + e]) == bits_of(qr[k]);
+            if (!same) continue;
+            want &= ~(1u << u);
+            if (e == ref) kept |= 1u << u;
+        }
+    }
+    want |= kept;
+    // the remaining cells' speeds by a few FP64 instructions (to 1e-15), then
+    // the formula itself for those within 1e-14 of the largest
     double w[STATE_UNROLL][2];
     unsigned long long k0 = 0ull, k1 = 0ull;
 #pragma unroll
