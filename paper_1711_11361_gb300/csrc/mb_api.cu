@@ -346,7 +346,7 @@ static size_t instance_bytes(const InstDesc &I, int prec) {
 }
 
 // rows per thread of the FP32 Euler y sweep: 64, halved down to 8 while the
-// batch's units leave fewer than 16 warps per SM.  A unit's first rows (ring
+// batch's units leave fewer than 11 warps per SM.  A unit's first rows (ring
 // fill, two rows of stencil) cost about as much as six of its own, so large
 // batches keep 64 (28.7 M cells: 32 measured slower).  400 x 400 cells: 91 us
 // per sweep with 64 rows (25 CTAs), 21 with 8; 1024 x 1024: 83 -> 19
@@ -357,7 +357,7 @@ static int auto_yseg(const mb_sim *s) {
         for (const auto &I : s->hd) u += (long long)I.tiles_x[1] * ((I.ny + g - 1) / g);
         return u;
     };
-    while (seg > 8 && units(seg) < 16LL * s->nsm) seg /= 2;
+    while (seg > 8 && units(seg) < 11LL * s->nsm) seg /= 2;
     return seg;
 }
 
@@ -398,21 +398,26 @@ static cudaError_t relayout(mb_sim *s, int old_n, const std::vector<int> &from) 
         tiles1 += I.ntiles[1];
         max_cells = std::max(max_cells, (size_t)I.nx * I.ny);
     }
-    // columns per geometry group: 2 where the groups run in one wave of three
-    // CTAs per SM, else 4, 8 or GEO_GC, the fewest that run in two.  A group's
-    // queries share its warps, so a narrow group is done sooner (400 x 400
-    // cylinder, per sweep of the whole step: 176 us with 16 columns, 142 with
-    // 8, 121 with 4, 117 with 2), while more groups repeat its gathering
-    // (940 x 376 tube: 243 us with 235 groups of 4, 247 with 470 of 2; 12 mixed
-    // grids: 16 requests in 94 ms with 16 columns, 88, 86, 93 with 8, 4, 2)
-    auto groups = [&](int w) {
+    // columns per geometry group: the fewest (2 to GEO_GC) whose groups run in
+    // one wave of three CTAs per SM.  A group's queries share its warps, so a
+    // narrow group is done sooner (400 x 400 cylinder, per sweep of the whole
+    // step: 176 us with 16 columns, 142 with 8, 121 with 4, 117 with 2), while
+    // groups beyond one wave repeat its gathering (940 x 376 tube: 243 us with
+    // 235 groups of 4, 247 with 470 of 2).  8 columns may take a second wave
+    // where a body rotates, whose queries (swept faces of moving edges) weigh
+    // more than the gathering: 12 mixed grids, 16 requests in 87 ms with 8
+    // columns, 92 with 16; 16 translating bodies, 0.468 ms per step with 550
+    // groups of 8, 0.457 with 279 of 16.  4 columns do not: the requests gain
+    // 2%, but eight such batches side by side lose 8%
+    bool rotating = false;
+    for (const auto &I : s->hd) rotating = rotating || I.rotating;
+    auto fits = [&](int w) {
         long long g = 0;
         for (const auto &I : s->hd) g += (I.gcol_max + w - 1) / w;
-        return g;
+        return g <= (w == 8 && rotating ? 6LL : 3LL) * s->nsm;
     };
     s->gcw = 2;
-    if (groups(2) > 3LL * s->nsm)
-        for (s->gcw = 4; s->gcw < GEO_GC && groups(s->gcw) > 6LL * s->nsm;) s->gcw *= 2;
+    while (s->gcw < GEO_GC && !fits(s->gcw)) s->gcw *= 2;
     // geometry groups (gcw columns, one CTA each): instances with more
     // polygon vertices first, so that the groups with the most cut cells start
     // in the first wave of CTAs
