@@ -582,9 +582,9 @@ def run_n2(args):
 
 def n3_flux_profile(precision):
     """(FP64-pipe lane operations, DRAM bytes) per face of the three-
-    dimensional flux kernel k3_flux in the given precision ("fp64" or
-    "fp32"), from the ncu captures summarised in profiles/n3_flux_ops.json;
-    None when mb3.cu has changed since."""
+    dimensional line kernels k3_row and k3_march in the given precision
+    ("fp64" or "fp32"), from the ncu captures summarised in
+    profiles/n3_flux_ops.json; None when the sources have changed since."""
     import hashlib
     try:
         d = json.load(open(os.path.join(ROOT, "profiles", "n3_flux_ops.json")))
@@ -598,13 +598,15 @@ def n3_flux_profile(precision):
         return None
 
 
-N3_FLUX_F32_BYTES = 80   # per face: two cells' FP32 evolved states (2 x 20 B) read, the FP64 flux (40 B) written
+N3_FLUX_F32_BYTES = 120   # per face (one per cell): the FP64 and FP32 states (60 B) read, the new ones written
 
 
 def n3_flux_roofline(mb3, p, rate, precision="fp64"):
-    """k3_flux, the three-dimensional path's dominant kernel: its device time
-    per sweep (CUDA events around each launch on the simulation's stream,
-    two steps' sweeps from the initial state) and faces per second.  FP64:
+    """The line kernels (k3_row, k3_march: evolved states, fluxes, update), the
+    three-dimensional path's dominant kernels: their device time per sweep
+    (CUDA events around their launches on the simulation's stream, the
+    geometry kernels running beside them; two steps' sweeps from the initial
+    state) and faces per second.  FP64:
     FP64-pipe lane operations per second against the measured FP64 rate.
     FP32 flux option: algorithmic bytes per second against the measured HBM
     copy bandwidth.  `rate` is the FP64 FMA rate."""
@@ -623,7 +625,7 @@ def n3_flux_roofline(mb3, p, rate, precision="fp64"):
     sim.close()
     faces = sum(f for f, _ in per)
     secs = sum(t for _, t in per)
-    out = {"kernel": "k3_flux", "precision": precision, "ms_per_sweep": secs / len(per) * 1e3,
+    out = {"kernel": "k3_row / k3_march", "precision": precision, "ms_per_sweep": secs / len(per) * 1e3,
            "faces_per_s": faces / secs}
     prof = n3_flux_profile(precision)
     if precision == "fp32":

@@ -625,10 +625,10 @@ __device__ __forceinline__ int find_inst_warp(const InstDesc *D, int n_inst, int
 // every SM has some: one unit per warp spreads a 400 x 400 grid over 5600
 // warps, where a warp per row (x) or per 64 rows (y) left most SMs idle.
 // Measured per sweep, FP64 Euler, before -> after: 399 x 399, x 286 -> 73 us,
-// y 1380 -> 90 us (its two launches together); 9.8 M cells in 16 grids, x
-// 2950 -> 1428 us, y 4090 -> 1430 us, 0.86 of the FP64 pipe's rate for the 79
-// lane operations per cell this flow executes (with the division, square
-// root and comparisons of CUDA: 188 or more).
+// y 1380 -> 90 us (its two launches together); 4.9 M cells in 16 grids, x
+// 2950 -> 1428 us, y 4090 -> 1430 us, 0.86 of the FP64 pipe's rate for the
+// 139 to 157 lane operations per cell this flow executes (263 in x and 289 in
+// y with CUDA's division and square root and comparisons on the FP64 pipe).
 constexpr int UNIT_CELLS = 30;
 constexpr int UNIT_COLS = 8;    // columns (lines) per CTA of the y sweep
 
