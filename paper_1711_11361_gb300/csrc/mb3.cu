@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "mb3.h"
+#include "mb3_near.h"
 #include "mb_fp64.cuh"
 
 namespace mb3 {
@@ -943,30 +944,13 @@ __device__ __forceinline__ void add_wall(const Desc &D, const double *w) {
 // Only their update reads body data: k3_row and k3_march update all other
 // cells, beside the geometry, and k3_near_row and k3_near the near ones after
 // k3_wall (few, and FP64 chains: as many threads as there are cells).
-struct Near { int a, len; bool wrap; };   // positions a .. a + len - 1 (modulo a periodic line)
 __host__ __device__ inline Near near_range(const Desc &D, int d, int nal) {
-    Near N;
-    N.a = D.r0[d] - 2;
-    N.len = D.rn[d] > 0 ? D.rn[d] + 5 : 0;
-    N.wrap = D.bc[2 * d] == MB_BC_PERIODIC;
-    if (N.wrap) {
-        if (N.len > nal) N.len = nal;
-    } else {
-        const int e = N.a + N.len < nal ? N.a + N.len : nal;
-        if (N.a < 0) N.a = 0;
-        N.len = e > N.a ? e - N.a : 0;
-    }
-    return N;
+    return near_span(D.r0[d], D.rn[d], nal, D.bc[2 * d] == MB_BC_PERIODIC);
 }
 __device__ __forceinline__ bool near_line(const Desc &D, int d, const int *ijk) {
     bool in = D.rn[0] > 0;
     for (int q = 0; q < 3; ++q) in = in && (q == d || (ijk[q] >= D.r0[q] && ijk[q] < D.r0[q] + D.rn[q]));
     return in;
-}
-__device__ __forceinline__ bool near_pos(const Near &N, int m, int nal) {
-    int r = m - N.a;
-    if (N.wrap) r += r >= nal ? -nal : r < 0 ? nal : 0;
-    return r >= 0 && r < N.len;
 }
 
 // x sweep.  The line kernels keep the evolved states and the fluxes in
