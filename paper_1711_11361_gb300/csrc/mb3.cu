@@ -1543,10 +1543,9 @@ __global__ void k3_final(Desc D) {
 // their bit patterns), in the type T of the flow arithmetic; 256-thread
 // blocks, one atomic per block and axis.
 // FP64: a block takes 2048 cells at a time and first forms their speeds in
-// FP32 (error below 4e-6 of the speed where p > E / 10); only a cell within
-// 1e-5 of the largest the block has seen along an axis, or with a smaller
-// pressure, goes through the FP64 formula, so that the result is that
-// formula's over every cell.  4 M cells: 267 us with the FP64 formula
+// FP32; only a cell within 1e-5 of the largest the block has seen along an
+// axis, or one whose FP32 speeds are not trusted (speeds32), goes through the
+// FP64 formula, so that the result is that formula's over every cell.  4 M cells: 267 us with the FP64 formula
 // throughout.
 constexpr int SPEED_CELLS = 8;   // cells per thread and turn (FP64)
 template <typename T>
@@ -1572,7 +1571,7 @@ __global__ void __launch_bounds__(256) k3_speeds64(Desc D) {
     __shared__ float redf[3][8];
     __shared__ double red[3][8];
     const double g = D.gamma;
-    const float gf = D.gammaf;
+    const float gf = D.gammaf, h1f = (float)D.g1h;
     double s[3] = {0.0, 0.0, 0.0};
     float lead[3] = {0.0f, 0.0f, 0.0f};
     for (long long c0 = (long long)blockIdx.x * 256 * SPEED_CELLS; c0 < D.n; c0 += (long long)gridDim.x * 256 * SPEED_CELLS) {
@@ -1592,10 +1591,8 @@ __global__ void __launch_bounds__(256) k3_speeds64(Desc D) {
                 x[k] = near32(q, ok);
             }
             if (!fluid) continue;
-            const float ir = __fdividef(1.0f, x[0]);
-            const float p = (gf - 1.0f) * (x[4] - 0.5f * sq3(x + 1) * ir);
-            if (!(ok && x[0] > 1e-30f && x[4] < 1e30f && p > 0.1f * x[4])) { want |= 1u << u; continue; }
-            const float cs = sqrtf(gf * p * ir);
+            float ir, cs;
+            if (!(speeds32<NC>(gf, h1f, x, ir, cs) && ok)) { want |= 1u << u; continue; }
             for (int a = 0; a < 3; ++a) {
                 v[u][a] = fabsf(x[1 + a] * ir) + cs;
                 m[a] = fmaxf(m[a], v[u][a]);

@@ -111,6 +111,25 @@ __device__ __forceinline__ float near32(double x, bool &ok) {
     return m < 0x38100000u ? 0.0f : __uint_as_float(f | (hi & 0x80000000u));
 }
 
+// Wave speeds in FP32 as a screen for the FP64 ones: 1/rho and the speed of
+// sound of a state x to 2^-22 (near32); true where every |m_a| / rho + c is
+// trusted to 3e-6.  The pressure is h1 e2, h1 = (gamma - 1) / 2, e2 = 2 E -
+// m^2 / rho: cutting the inputs, the square, the reciprocal and the difference
+// round e2 by at most 1.6e-6 E, so where e2 > E / 2 the root's relative error
+// is below 2e-6, whatever gamma is (in air that is p > E / 10).  Two cells'
+// errors stay below the 1e-5 by which a caller lets one lead.
+template <int NC>
+__device__ __forceinline__ bool speeds32(float gf, float h1f, const float *x, float &ir, float &cs) {
+    constexpr int E = NC - 1;
+    float m2 = x[E - 1] * x[E - 1];
+#pragma unroll
+    for (int k = E - 2; k >= 1; --k) m2 = fmaf(x[k], x[k], m2);
+    ir = __fdividef(1.0f, x[0]);
+    const float e2 = fmaf(-m2, ir, 2.0f * x[E]), c2 = gf * (h1f * e2) * ir;
+    cs = sqrtf(c2);
+    return x[0] > 1e-30f && x[E] < 1e30f && e2 > 0.5f * x[E] && c2 > 0.0f;
+}
+
 // ---------------------------------------------------------------------------
 // FP64 Euler arithmetic, conserved variables q[NC] = rho, momenta, E; D: the
 // momentum normal to the faces

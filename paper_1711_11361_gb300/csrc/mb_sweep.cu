@@ -675,9 +675,9 @@ __device__ __forceinline__ void up_state(S &s) { s.q[0] = __shfl_up_sync(0xfffff
 
 // new state of a lane's cell (qn), with the positivity check and, on the
 // step's last sweep, the wave speeds s0, s1.  The speeds are first formed in
-// FP32 (error below 4e-6 where p > E / 10): only a cell within 1e-5 of the
-// instance's largest so far (m0, m1: y.S read before), or with a smaller
-// pressure, goes through FP64, so the maxima are those over every cell
+// FP32: only a cell within 1e-5 of the instance's largest so far (m0, m1: y.S
+// read before), or one whose FP32 speeds are not trusted (speeds32), goes
+// through FP64, so the maxima are those over every cell
 __device__ __forceinline__ void new_state(const Flow<double, 0> &f, const double *q, const double *Flo,
                                           const double *Fhi, bool last, int ci, InstDyn &y, float m0, float m1,
                                           double *qn, double &s0, double &s1) {
@@ -688,12 +688,11 @@ __device__ __forceinline__ void new_state(const Flow<double, 0> &f, const double
         float x[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) x[k] = near32(qn[k], ok);
-        const float ir32 = __fdividef(1.0f, x[0]);
-        const float p32 = f.h1f * fmaf(-fmaf(x[1], x[1], x[2] * x[2]), ir32, 2.0f * x[3]);
-        if (ok && x[0] > 1e-30f && x[3] < 1e30f && p32 > 0.1f * x[3]) {   // (positive with a margin)
-            const float cs = sqrtf(f.gf * p32 * ir32);
-            if (fabsf(x[1] * ir32) + cs < m0 * (1.0f - 1e-5f) && fabsf(x[2] * ir32) + cs < m1 * (1.0f - 1e-5f)) return;
-        }
+        float ir32, cs;
+        // (trusted: also physical with a margin)
+        if (speeds32<4>(f.gf, f.h1f, x, ir32, cs) && ok && fabsf(x[1] * ir32) + cs < m0 * (1.0f - 1e-5f) &&
+            fabsf(x[2] * ir32) + cs < m1 * (1.0f - 1e-5f))
+            return;
         const double ir = rcp64(qn[0]), p = press64<4>(f.h1, qn, ir);
         if (!pos64(qn[0]) || !pos64(p)) list_bulk_bad(y, ci);
         const double c = sqrt64(f.g * (p * ir));
@@ -2838,11 +2837,10 @@ __device__ __forceinline__ unsigned long long bits_of(float v) { return __float_
 // the stored (T-rounded) states.  Each cell's speeds are first formed in
 // FP32; a cell goes through the FP64 formula only if one of them comes within
 // 1e-5 of the largest known along its axis (of the CTA's cells, or of the
-// instance so far), or if its pressure is small against its energy (p <=
-// E/10, where the FP32 error could exceed 4e-6).  No skipped cell can
-// hold the maximum, so the result is that of the FP64 formula over every
-// cell; cells in a state already taken drop out first.  H: the element type
-// of the host layout (FP64 or FP32 states).
+// instance so far), or if its FP32 speeds are not trusted (speeds32).  No
+// skipped cell can hold the maximum, so the result is that of the FP64 formula
+// over every cell; cells in a state already taken drop out first.  H: the
+// element type of the host layout (FP64 or FP32 states).
 // 28.7 M cells whose speeds tie (the worst case): 3760 us with every cell
 // through the formula, 1185 us so; 400 x 400 cells 121 -> 40 us.  Uniform
 // states, whose cells a thread skipped as its last one's: 869 -> 1093 us.
@@ -2863,7 +2861,7 @@ __global__ void __launch_bounds__(STATE_THREADS, 3) k_write_state(const InstDesc
     const size_t plane = (size_t)I.pitch * I.ny;
     T *Q = bufw<T>(I, b);
     const bool euler = I.eq == 0;
-    const float gf = (float)I.gamma;
+    const float gf = (float)I.gamma, h1f = (float)I.g1h;
     float v[STATE_UNROLL][2], m0 = 0.0f, m1 = 0.0f;
     unsigned want = 0u;
     bool fluid = false;
@@ -2896,13 +2894,11 @@ __global__ void __launch_bounds__(STATE_THREADS, 3) k_write_state(const InstDesc
         float x[MAXC];
 #pragma unroll
         for (int k = 0; k < MAXC; ++k) x[k] = sizeof(T) == 4 ? (float)q[k] : near32((double)q[k], ok);
-        const float ir = __fdividef(1.0f, x[0]);
-        const float p = (gf - 1.0f) * (x[3] - 0.5f * (x[1] * x[1] + x[2] * x[2]) * ir);
-        if (!(ok && x[0] > 1e-30f && x[3] < 1e30f && p > 0.1f * x[3])) {
+        float ir, cs;
+        if (!(speeds32<4>(gf, h1f, x, ir, cs) && ok)) {
             want |= 1u << u;
             continue;
         }
-        const float cs = sqrtf(gf * p * ir);
         v[u][0] = fabsf(x[1] * ir) + cs;
         v[u][1] = fabsf(x[2] * ir) + cs;
         m0 = fmaxf(m0, v[u][0]);
