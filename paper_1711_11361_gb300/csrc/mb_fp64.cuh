@@ -117,7 +117,10 @@ __device__ __forceinline__ float near32(double x, bool &ok) {
 // m^2 / rho: cutting the inputs, the square, the reciprocal and the difference
 // round e2 by at most 1.6e-6 E, so where e2 > E / 2 the root's relative error
 // is below 2e-6, whatever gamma is (in air that is p > E / 10).  Two cells'
-// errors stay below the 1e-5 by which a caller lets one lead.
+// errors stay below the 1e-5 by which a caller lets one lead.  rho E, which
+// bounds m^2, and the squared speed of sound lie far inside FP32's range: in
+// units that put them near its ends m^2 is lost (at rho about 1e-21 a cell at
+// rest counted as slower than one whose kinetic energy had underflowed).
 template <int NC>
 __device__ __forceinline__ bool speeds32(float gf, float h1f, const float *x, float &ir, float &cs) {
     constexpr int E = NC - 1;
@@ -126,8 +129,9 @@ __device__ __forceinline__ bool speeds32(float gf, float h1f, const float *x, fl
     for (int k = E - 2; k >= 1; --k) m2 = fmaf(x[k], x[k], m2);
     ir = __fdividef(1.0f, x[0]);
     const float e2 = fmaf(-m2, ir, 2.0f * x[E]), c2 = gf * (h1f * e2) * ir;
+    const float rE = x[0] * x[E];
     cs = sqrtf(c2);
-    return x[0] > 1e-30f && x[E] < 1e30f && e2 > 0.5f * x[E] && c2 > 0.0f;
+    return x[0] > 1e-30f && x[0] < 1e30f && rE > 1e-30f && rE < 1e30f && c2 > 1e-30f && c2 < 1e30f && e2 > 0.5f * x[E];
 }
 
 // ---------------------------------------------------------------------------

@@ -1,9 +1,10 @@
 """Wave speeds behind the CFL step where their FP32 screen is least accurate:
 cells whose speeds agree to 1e-7, with a pressure just above the screen's bound
 (and a tenth of the energy), the largest in a cell whose FP32 speed comes out
-lowest; adiabatic exponents from 1.1 to 20.  A written state's first step, the
-step after an update and the three-dimensional CFL step against the speeds of
-every cell in numpy: 1e-12 relative (a few FP64 roundings, amplified up to 200
+lowest; adiabatic exponents from 1.1 to 20; and units of mass that put the
+momenta's squares outside FP32's range.  A written state's first step, the step
+after an update and the three-dimensional CFL step against the speeds of every
+cell in numpy: 1e-12 relative (a few FP64 roundings, amplified up to 200
 times by 2 E - m^2 / rho, are below 1e-13; the fastest cell leads by 1e-9)."""
 import numpy as np
 import pytest
@@ -106,3 +107,27 @@ def test_three_dimensions(gamma, low, axis):
     sim = mb3.Sim3(p)
     assert abs(sim.cfl_dt() / want - 1.0) <= BAR
     sim.close()
+
+
+@pytest.mark.parametrize("scale", [1e-21, 1e-25, 1e20, 1e28], ids=str)
+def test_densities_far_from_one(scale):
+    """The same cells in other units of mass: a square of a momentum underflows or overflows in FP32."""
+    from paper_1711_11361_gb300 import mb, mb3
+    p = grid(64, 66, 1.4, True, False, 4)
+    p.Q0 *= scale
+    p.y1 = 0.2
+    # every other row at rest, with the larger speed of sound (0.26 against 0.23, and 0.47 where m^2 is lost), which
+    # sets the step along y
+    p.Q0[:, ::2] *= np.array([1.0, 0.0, 1.0, 0.3])[:, None, None]
+    sim = mb.Sim(p, mb.FP64)
+    sim.step(1e-16)
+    q = sim.read_state(0)["Q"]
+    assert abs(sim.step(0.0, report=True)[0] / first_dt(p, q) - 1.0) <= BAR
+    sim.write_state(0, p.Q0)
+    assert abs(sim.step(0.0, report=True)[0] / first_dt(p, p.Q0) - 1.0) <= BAR
+    sim.close()
+    p3 = inputs.Problem3("speeds", 64, 66, 1, hi=(1.0, 0.2, 1.0), bc=(inputs.PERIODIC,) * 6, cfl=0.4)
+    p3.Q0 = np.stack([p.Q0[0], p.Q0[1], p.Q0[2], np.zeros_like(p.Q0[0]), p.Q0[3]])[:, None]
+    sim3 = mb3.Sim3(p3)
+    assert abs(sim3.cfl_dt() / first_dt(p, p.Q0) - 1.0) <= BAR
+    sim3.close()
