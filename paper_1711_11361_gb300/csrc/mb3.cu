@@ -920,8 +920,10 @@ __device__ __forceinline__ void line_update(const Desc &D, const int *line, int 
             D.Qfn[(size_t)q * D.n + c] = x[q];
         }
         // the seed test in FP32 where that decides with a margin of 1e-5
+        // (and no product underflows)
         const float t = 2.0f * x[0] * x[4];
-        if (!(x[0] > 0.0f && x[4] > 0.0f && t < 1e38f && t - sq3(x + 1) > 1e-5f * t) && content_bad(v))
+        if (!(x[0] > 0.0f && x[4] > 0.0f && t > 1e-30f && t < 1e38f && t - sq3(x + 1) > 1e-5f * t) &&
+            content_bad(v))
             add_seed(D, c);
     } else if (!physical64<NC>(v)) {
         if (content_bad(v)) add_seed(D, c);

@@ -154,7 +154,8 @@ __device__ __forceinline__ double press64(double h1, const double *q, double ir)
     return h1 * __fma_rn(-msq64<NC>(q), ir, twice64(q[NC - 1]));
 }
 // rho > 0 and 2 rho E > |m|^2, in FP32 where that decides with a margin of
-// 1e-5 (its error is below 2e-6), else in FP64
+// 1e-5 (its error is below 2e-6 where no product underflows, which the bounds
+// on 2 rho E leave out), else in FP64
 template <int NC>
 __device__ __forceinline__ bool physical64(const double *q) {
     bool ok = true;
@@ -166,7 +167,7 @@ __device__ __forceinline__ bool physical64(const double *q) {
         m2 = fmaf(m, m, m2);
     }
     const float t = 2.0f * r * E;
-    if (ok && r > 0.0f && E > 0.0f && t < 1e38f && t - m2 > 1e-5f * t) return true;
+    if (ok && r > 0.0f && E > 0.0f && t > 1e-30f && t < 1e38f && t - m2 > 1e-5f * t) return true;
     return pos64(q[0]) && 2.0 * q[0] * q[NC - 1] > msq64<NC>(q) && q[NC - 1] - q[NC - 1] == 0.0;
 }
 // MUSCL-Hancock evolved states of one cell: van Leer slopes in conserved
