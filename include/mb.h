@@ -255,8 +255,11 @@ int mb_band_record_size(void);
  * on the device (between steps; the simulation is not changed): the CTA size
  * of each sweep direction's kernel, its register budget (registers for 4 or
  * 5 resident CTAs per SM), the depth of the x sweep's row ring and the rows
- * per thread of the y sweep.  report (optional, 8 doubles): x CTA size, y CTA
- * size, y rows per thread, the best x and y kernel times in ms, the x and y
+ * per thread of the y sweep (32, 64, 128, or the automatic choice, which goes
+ * on following the batch where it is the fastest).  report (optional, 8
+ * doubles): x CTA size, y CTA size, the best of 32, 64 and 128 y rows per
+ * thread (64 for the scalar kernels, whose units have one size), the best x
+ * and y kernel times in ms, the x and y
  * register budgets (resident CTAs per SM) and the x ring depth (chunks of 64
  * cells).  Later mb_batch_add calls use the chosen shapes. */
 mb_status mb_autotune(mb_sim *sim, double *report);

@@ -1193,19 +1193,27 @@ mb_status mb_autotune(mb_sim *sim, double *report) {
         xs.push_back(256);
         ys.push_back(256);
     }
-    const int ysegs[3] = {32, 64, 128};
-    double best_x = 1e30, best_y = 1e30;
-    int bx = sim->tune_cta[0], by = sim->tune_cta[1], bs = sim->tune_yseg ? sim->tune_yseg : 64;
+    // rows per thread of the FP32x2 y sweep (the scalar units have one size):
+    // the automatic choice (0) first, which goes on following the batch where
+    // it is the best (a small batch's 8 or 16 rows), then the other candidates
+    const int rows0 = packed ? auto_yseg(sim) : 64;
+    std::vector<int> ysegs = {0};
+    for (int r : {32, 64, 128})
+        if (packed && r != rows0) ysegs.push_back(r);
+    double best_x = 1e30, best_y = 1e30, best_c = 1e30;
+    int bx = sim->tune_cta[0], by = sim->tune_cta[1], bs = sim->tune_yseg, bc = 64;
     for (int shape : xs) {
         double t = time_bulk(0, shape);
         if (t < best_x) { best_x = t; bx = shape; }
     }
-    for (int ys_ = 0; ys_ < 3; ++ys_) {
-        e = set_yseg(sim, ysegs[ys_]);
+    for (int rows : ysegs) {
+        e = set_yseg(sim, rows);
         if (e != cudaSuccess) break;
         for (int shape : ys) {
             double t = time_bulk(1, shape);
-            if (t < best_y) { best_y = t; by = shape; bs = ysegs[ys_]; }
+            if (t < best_y) { best_y = t; by = shape; bs = rows; }
+            const int r = rows ? rows : rows0;
+            if (r >= 32 && t < best_c) { best_c = t; bc = r; }
         }
     }
     cudaEventDestroy(e0);
@@ -1219,7 +1227,7 @@ mb_status mb_autotune(mb_sim *sim, double *report) {
     if (report) {
         report[0] = bx & 1023;
         report[1] = by & 1023;
-        report[2] = bs;
+        report[2] = bc;
         report[3] = best_x;
         report[4] = best_y;
         report[5] = (bx & SHAPE_MINB4) ? 4 : 5;

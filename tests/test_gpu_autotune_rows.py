@@ -1,0 +1,37 @@
+"""mb_autotune on a small batch, where the automatic rows per thread of the FP32
+y sweep (8) are the fastest by far (400 x 400 cells: 21 us per sweep, 91 with
+64 rows): tuning leaves the bulk kernels no slower than they were.  Without the
+automatic rows among the candidates their time grows by half (two steps 0.104 to
+0.154 ms); the bar is 1.25, over
+the best of several steps."""
+import numpy as np
+import pytest
+
+from paper_1711_11361_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def _bulk_ms(sim):
+    best = 1e30
+    for _ in range(8):
+        sim.enable_timing(True)
+        sim.run(2)
+        sim.sync()
+        best = min(best, sim.kernel_time()[0])
+    sim.enable_timing(False)
+    return best
+
+
+def test_tuning_a_small_batch_keeps_its_short_units():
+    from paper_1711_11361_gb300 import mb
+    sim = mb.Sim(inputs.c2_cylinder(400), mb.FP32)
+    before = _bulk_ms(sim)
+    for _ in range(2):
+        assert sim.autotune()["y_rows"] in (32, 64, 128)
+        assert _bulk_ms(sim) <= 1.25 * before
+    # and the layout goes on following the batch
+    sim.add(inputs.small_case("cylinder", 48))
+    sim.run(2)
+    assert np.all(np.isfinite(sim.read_states()[1]))
+    sim.close()
