@@ -2047,64 +2047,65 @@ __global__ void __launch_bounds__(128, MINB) k_bulk_y_p(const InstDesc *__restri
 // reading; Sec. III.E models its open-ended tube in axisymmetric form): with
 // x axial and y the radius from the axis y = y0 = 0, every fluid cell gets
 // Q -= dt (v / r) [rho, rho u, rho v, E + p], r at the cell centre.  One thread
-// per cell (grid: x over the largest instance's cells, y over the instances);
-// instances of the batch without the flag return at once.  In
-// FP64 every operation is rounded on its own (no contraction), in the order
-// of the plain definition.
+// per cell (grid: x over the largest instance's cells, y over the instances,
+// which pass grid y's limit of 65535 by turns); instances of the batch without
+// the flag have nothing to do.  In FP64 every operation is rounded on its own
+// (no contraction), in the order of the plain definition.
 // ---------------------------------------------------------------------------
 template <class T>
 __global__ void __launch_bounds__(256) k_axisym_source(const InstDesc *__restrict__ D, InstDyn *__restrict__ Y,
-                                                       int buf) {
-    const int inst = blockIdx.y;
-    const InstDesc &I = D[inst];
-    if (!I.axisym || I.eq != 0) return;
-    InstDyn &y = Y[inst];
-    const size_t plane = (size_t)I.pitch * I.ny;
-    const double dt = y.dt;
-    bool bad = false;
-    // a warp's 32 positions lie in one row (the pitch is a multiple of 32)
-    for (size_t c = (size_t)blockIdx.x * 256 + threadIdx.x; c < plane; c += (size_t)gridDim.x * 256) {
-        const int j = (int)(c / I.pitch), i = (int)(c - (size_t)j * I.pitch);
-        if (i >= I.nx) continue;
-        const double r = __dmul_rn(__dadd_rn((double)j, 0.5), I.dy);
-        T *__restrict__ Q = (T *)I.Q[buf] + (size_t)j * I.pitch;
-        const T q0 = Q[i], q1 = Q[plane + i], q2 = Q[2 * plane + i], q3 = Q[3 * plane + i];
-        if (!(q0 == q0)) continue;   // solid
-        T n0, n1, n2, n3, pn;
-        if (sizeof(T) == 8) {
-            const double g1 = __dsub_rn(I.gamma, 1.0);
-            const double p = __dmul_rn(g1, __dsub_rn(q3, __ddiv_rn(__dmul_rn(0.5, __dadd_rn(__dmul_rn(q1, q1),
-                                                                                           __dmul_rn(q2, q2))), q0)));
-            const double f = __ddiv_rn(__dmul_rn(dt, __ddiv_rn(q2, q0)), r);
-            n0 = (T)__dsub_rn(q0, __dmul_rn(f, q0));
-            n1 = (T)__dsub_rn(q1, __dmul_rn(f, q1));
-            n2 = (T)__dsub_rn(q2, __dmul_rn(f, q2));
-            n3 = (T)__dsub_rn(q3, __dmul_rn(f, __dadd_rn(q3, p)));
-            pn = (T)__dmul_rn(g1, __dsub_rn(n3, __ddiv_rn(__dmul_rn(0.5, __dadd_rn(__dmul_rn(n1, n1),
-                                                                                  __dmul_rn(n2, n2))), n0)));
-        } else {
-            const float g1 = (float)I.gamma - 1.0f;
-            const float p = g1 * (q3 - 0.5f * (q1 * q1 + q2 * q2) / q0);
-            const float f = (float)dt * (q2 / q0) / (float)r;
-            n0 = q0 - f * q0;
-            n1 = q1 - f * q1;
-            n2 = q2 - f * q2;
-            n3 = q3 - f * (q3 + p);
-            pn = g1 * (n3 - 0.5f * (n1 * n1 + n2 * n2) / n0);
+                                                       int n_inst, int buf) {
+    for (int inst = blockIdx.y; inst < n_inst; inst += gridDim.y) {
+        const InstDesc &I = D[inst];
+        if (!I.axisym || I.eq != 0) continue;
+        InstDyn &y = Y[inst];
+        const size_t plane = (size_t)I.pitch * I.ny;
+        const double dt = y.dt;
+        bool bad = false;
+        // a warp's 32 positions lie in one row (the pitch is a multiple of 32)
+        for (size_t c = (size_t)blockIdx.x * 256 + threadIdx.x; c < plane; c += (size_t)gridDim.x * 256) {
+            const int j = (int)(c / I.pitch), i = (int)(c - (size_t)j * I.pitch);
+            if (i >= I.nx) continue;
+            const double r = __dmul_rn(__dadd_rn((double)j, 0.5), I.dy);
+            T *__restrict__ Q = (T *)I.Q[buf] + (size_t)j * I.pitch;
+            const T q0 = Q[i], q1 = Q[plane + i], q2 = Q[2 * plane + i], q3 = Q[3 * plane + i];
+            if (!(q0 == q0)) continue;   // solid
+            T n0, n1, n2, n3, pn;
+            if (sizeof(T) == 8) {
+                const double g1 = __dsub_rn(I.gamma, 1.0);
+                const double p = __dmul_rn(g1, __dsub_rn(q3, __ddiv_rn(__dmul_rn(0.5, __dadd_rn(__dmul_rn(q1, q1),
+                                                                                               __dmul_rn(q2, q2))), q0)));
+                const double f = __ddiv_rn(__dmul_rn(dt, __ddiv_rn(q2, q0)), r);
+                n0 = (T)__dsub_rn(q0, __dmul_rn(f, q0));
+                n1 = (T)__dsub_rn(q1, __dmul_rn(f, q1));
+                n2 = (T)__dsub_rn(q2, __dmul_rn(f, q2));
+                n3 = (T)__dsub_rn(q3, __dmul_rn(f, __dadd_rn(q3, p)));
+                pn = (T)__dmul_rn(g1, __dsub_rn(n3, __ddiv_rn(__dmul_rn(0.5, __dadd_rn(__dmul_rn(n1, n1),
+                                                                                      __dmul_rn(n2, n2))), n0)));
+            } else {
+                const float g1 = (float)I.gamma - 1.0f;
+                const float p = g1 * (q3 - 0.5f * (q1 * q1 + q2 * q2) / q0);
+                const float f = (float)dt * (q2 / q0) / (float)r;
+                n0 = q0 - f * q0;
+                n1 = q1 - f * q1;
+                n2 = q2 - f * q2;
+                n3 = q3 - f * (q3 + p);
+                pn = g1 * (n3 - 0.5f * (n1 * n1 + n2 * n2) / n0);
+            }
+            Q[i] = n0;
+            Q[plane + i] = n1;
+            Q[2 * plane + i] = n2;
+            Q[3 * plane + i] = n3;
+            if (!(n0 > (T)0) || !(pn > (T)0)) bad = true;
         }
-        Q[i] = n0;
-        Q[plane + i] = n1;
-        Q[2 * plane + i] = n2;
-        Q[3 * plane + i] = n3;
-        if (!(n0 > (T)0) || !(pn > (T)0)) bad = true;
+        if (bad) atomicOr(&y.err, ERR_UNSTABLE);
     }
-    if (bad) atomicOr(&y.err, ERR_UNSTABLE);
 }
 
 template <class T>
 void launch_axisym_source(const InstDesc *D, InstDyn *Y, int n_inst, size_t max_cells, int buf, cudaStream_t st) {
     const unsigned bx = (unsigned)std::min<size_t>((max_cells + 255) / 256, 1u << 20);
-    if (bx > 0 && n_inst > 0) k_axisym_source<T><<<dim3(bx, n_inst), 256, 0, st>>>(D, Y, buf);
+    if (bx > 0 && n_inst > 0) k_axisym_source<T><<<dim3(bx, std::min(n_inst, 65535)), 256, 0, st>>>(D, Y, n_inst, buf);
 }
 
 // ---------------------------------------------------------------------------

@@ -2,8 +2,7 @@
 y sweep (8) are the fastest by far (400 x 400 cells: 21 us per sweep, 91 with
 64 rows): tuning leaves the bulk kernels no slower than they were.  Without the
 automatic rows among the candidates their time grows by half (two steps 0.104 to
-0.154 ms); the bar is 1.25, over
-the best of several steps."""
+0.154 ms); the bar is 1.25, over the best of several steps."""
 import numpy as np
 import pytest
 
