@@ -2835,88 +2835,128 @@ __device__ __forceinline__ unsigned long long bits_of(float v) { return __float_
 
 // Sources: srcs[blockIdx.y] (srcs != nullptr; a null entry skips that
 // instance) or src1.  The first step's wave speeds are the FP64 maxima over
-// the stored (T-rounded) states.  Each cell's speeds are first formed in
-// FP32; a cell goes through the FP64 formula only if one of them comes within
-// 1e-5 of the largest known along its axis (of the CTA's cells, or of the
-// instance so far), or if its FP32 speeds are not trusted (speeds32).  No
-// skipped cell can hold the maximum, so the result is that of the FP64 formula
-// over every cell; cells in a state already taken drop out first.  H: the
+// the stored (T-rounded) states.  Cells in the state that their warp took last
+// drop out by their bits (a uniform region costs a cell per warp).  The others'
+// speeds are formed in FP32; a cell goes through the FP64 formula only if one
+// of them comes within 1e-5 of the largest known along its axis (of the CTA's
+// cells, or of the instance so far), or if its FP32 speeds are not trusted
+// (speeds32).  No skipped cell can hold the maximum, so the result is that of
+// the FP64 formula over every cell.  Those cells are listed, so that the FP64
+// pipe gets full warps, and where they are many, a few FP64 instructions (to
+// 1e-15) leave those within 1e-14 of the largest for the formula.  H: the
 // element type of the host layout (FP64 or FP32 states).
-// 28.7 M cells whose speeds tie (the worst case): 3760 us with every cell
-// through the formula, 1185 us so; 400 x 400 cells 121 -> 40 us.  Uniform
-// states, whose cells a thread skipped as its last one's: 869 -> 1093 us.
+// Bound by the loads in flight (a thread has four cells' under way) or, where
+// speeds tie, by the FP64 pipe.  28.7 M cells in 64 grids, FP32: shock problems
+// 250 us, uniform 214, speeds that tie 1115, random 307 (one cell after the
+// other per thread, candidates where they lie: 789, 772, 1415, 1334).
 template <class T, class H>
-__global__ void __launch_bounds__(STATE_THREADS, 3) k_write_state(const InstDesc *__restrict__ D,
+__global__ void __launch_bounds__(STATE_THREADS, 4) k_write_state(const InstDesc *__restrict__ D,
                                                                InstDyn *__restrict__ Y,
                                                                const H *const *__restrict__ srcs,
                                                                const H *__restrict__ src1, int inst0, int b) {
-    __shared__ float red[2][STATE_THREADS / 32];
-    __shared__ unsigned long long redk[2][STATE_THREADS / 32];
-    __shared__ int redi[STATE_THREADS / 32];
+    constexpr int WARPS = STATE_THREADS / 32, GROUP = 4;
+    __shared__ float red[2][WARPS];
+    __shared__ unsigned long long redk[2][WARPS];
+    __shared__ unsigned short list[STATE_CELLS];
+    __shared__ int nlist;
     const int inst = inst0 + blockIdx.y;
     const H *__restrict__ Qh = srcs ? srcs[blockIdx.y] : src1;
     if (!Qh) return;
     const InstDesc &I = D[inst];
-    const int n = I.nx * I.ny, e0 = blockIdx.x * STATE_CELLS;
+    const int nx = I.nx, n = nx * I.ny, e0 = blockIdx.x * STATE_CELLS;
     if (e0 >= n) return;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const size_t plane = (size_t)I.pitch * I.ny;
     T *Q = bufw<T>(I, b);
-    const bool euler = I.eq == 0;
-    const float gf = (float)I.gamma, h1f = (float)I.g1h;
-    float v[STATE_UNROLL][2], m0 = 0.0f, m1 = 0.0f;
-    unsigned want = 0u;
-    bool fluid = false;
-    T lq[MAXC] = {T(0), T(0), T(0), T(0)};   // the thread's last distinct state (rho = 0: none)
-#pragma unroll
-    for (int u = 0; u < STATE_UNROLL; ++u) {
-        v[u][0] = v[u][1] = -1.0f;
-        const int e = e0 + u * STATE_THREADS + threadIdx.x;
-        if (e >= n) continue;
-        const int j = e / I.nx, c = j * I.pitch + (e - j * I.nx);
-        const bool solid = I.cls[c] & CLS_SOLID;
-        T q[MAXC];
-#pragma unroll
-        for (int k = 0; k < MAXC; ++k) {
-            if (k >= I.nc) break;
-            q[k] = (T)Qh[(size_t)k * n + e];
-            Q[k * plane + c] = solid ? T(NAN) : q[k];
+    const uint8_t *__restrict__ cls = I.cls;
+    // the thread's cell e at (i, j), then the one STATE_THREADS cells on
+    int e = e0 + tid, j = e / nx, i = e - j * nx;
+    const int dj = STATE_THREADS / nx, di = STATE_THREADS - dj * nx;
+    auto next = [&]() {
+        e += STATE_THREADS;
+        i += di;
+        j += dj;
+        if (i >= nx) {
+            i -= nx;
+            ++j;
         }
-        if (solid) continue;
-        fluid = true;
-        if (!euler) continue;
-        bool same = true;   // in a uniform region one cell per thread goes on
-#pragma unroll
-        for (int k = 0; k < MAXC; ++k) {
-            same = same && bits_of(q[k]) == bits_of(lq[k]);
-            lq[k] = q[k];
+    };
+    if (I.eq != 0) {   // advection: one plane, the constant speeds
+        bool fluid = false;
+        for (int u = 0; u < STATE_UNROLL && e < n; ++u, next()) {
+            const int c = j * I.pitch + i;
+            const bool solid = cls[c] & CLS_SOLID;
+            Q[c] = solid ? T(NAN) : (T)Qh[e];
+            fluid = fluid || !solid;
         }
-        if (same) continue;
-        bool ok = true;
-        float x[MAXC];
-#pragma unroll
-        for (int k = 0; k < MAXC; ++k) x[k] = sizeof(T) == 4 ? (float)q[k] : near32((double)q[k], ok);
-        float ir, cs;
-        if (!(speeds32<4>(gf, h1f, x, ir, cs) && ok)) {
-            want |= 1u << u;
-            continue;
-        }
-        v[u][0] = fabsf(x[1] * ir) + cs;
-        v[u][1] = fabsf(x[2] * ir) + cs;
-        m0 = fmaxf(m0, v[u][0]);
-        m1 = fmaxf(m1, v[u][1]);
-    }
-    if (!euler) {   // advection: the constant speeds
-        if (__syncthreads_or(fluid) && threadIdx.x == 0) {
+        if (__syncthreads_or(fluid) && tid == 0) {
             atomic_max_pos(&Y[inst].S[0], fabs(I.adv[0]));
             atomic_max_pos(&Y[inst].S[1], fabs(I.adv[1]));
         }
         return;
     }
+    if (tid == 0) nlist = 0;
+    const float gf = (float)I.gamma, h1f = (float)I.g1h;
+    float v[STATE_UNROLL][2], m0 = 0.0f, m1 = 0.0f;
+    unsigned want = 0u;
+    T ws[4] = {T(0), T(0), T(0), T(0)};   // the warp's last distinct state (rho = 0: none)
+#pragma unroll
+    for (int g = 0; g < STATE_UNROLL; g += GROUP) {
+        T q[GROUP][4];
+        int c[GROUP];
+        uint8_t cl[GROUP];
+#pragma unroll
+        for (int u = 0; u < GROUP; ++u, next()) {
+            const bool in = e < n;
+            c[u] = in ? j * I.pitch + i : -1;
+            cl[u] = in ? cls[c[u]] : (uint8_t)CLS_SOLID;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) q[u][k] = in ? (T)Qh[(size_t)k * n + e] : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < GROUP; ++u) {
+            const bool fluid = !(cl[u] & CLS_SOLID);
+            if (c[u] >= 0) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) Q[k * plane + c[u]] = fluid ? q[u][k] : T(NAN);
+            }
+            auto same = [&]() {
+                bool s = true;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) s = s && bits_of(q[u][k]) == bits_of(ws[k]);
+                return s;
+            };
+            bool take = fluid && !same();
+            const unsigned other = __ballot_sync(0xffffffffu, take);
+            float *const vu = v[g + u];
+            vu[0] = vu[1] = -1.0f;
+            if (other) {
+                const int first = __ffs(other) - 1;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) ws[k] = __shfl_sync(0xffffffffu, q[u][k], first);
+                take = take && (lane == first || !same());
+            }
+            if (take) {
+                bool ok = true;
+                float x[4], ir, cs;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) x[k] = sizeof(T) == 4 ? (float)q[u][k] : near32((double)q[u][k], ok);
+                if (speeds32<4>(gf, h1f, x, ir, cs) && ok) {
+                    vu[0] = fabsf(x[1] * ir) + cs;
+                    vu[1] = fabsf(x[2] * ir) + cs;
+                    m0 = fmaxf(m0, vu[0]);
+                    m1 = fmaxf(m1, vu[1]);
+                } else {
+                    want |= 1u << (g + u);
+                }
+            }
+        }
+    }
     for (int o = 16; o > 0; o >>= 1) {
         m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, o));
         m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
     }
-    if ((threadIdx.x & 31) == 0) { red[0][threadIdx.x >> 5] = m0; red[1][threadIdx.x >> 5] = m1; }
+    if (lane == 0) { red[0][warp] = m0; red[1][warp] = m1; }
     __syncthreads();
     bool ok = true;
     volatile const unsigned long long *S = Y[inst].S;
@@ -2924,58 +2964,54 @@ __global__ void __launch_bounds__(STATE_THREADS, 3) k_write_state(const InstDesc
     m1 = near32(__longlong_as_double((long long)S[1]), ok);
     if (!ok) m0 = m1 = 0.0f;
 #pragma unroll
-    for (int w = 0; w < STATE_THREADS / 32; ++w) {
+    for (int w = 0; w < WARPS; ++w) {
         m0 = fmaxf(m0, red[0][w]);
         m1 = fmaxf(m1, red[1][w]);
     }
 #pragma unroll
     for (int u = 0; u < STATE_UNROLL; ++u)
         if (v[u][0] >= m0 * (1.0f - 1e-5f) || v[u][1] >= m1 * (1.0f - 1e-5f)) want |= 1u << u;
-    auto state = [&](int u, double *q) {
-        const int e = e0 + u * STATE_THREADS + threadIdx.x;
-#pragma unroll
-        for (int k = 0; k < MAXC; ++k) q[k] = (double)(T)Qh[(size_t)k * n + e];
-    };
-    // Uniform regions: all remaining cells in the state of the first one but
-    // that one drop out, and so for the first of what is left (a shock's two
-    // sides), so that a uniform state costs one cell per CTA
-    unsigned kept = 0u;
-    for (int r = 0; r < 2; ++r) {
-        const int first = want ? e0 + (__ffs(want) - 1) * STATE_THREADS + (int)threadIdx.x : INT_MAX;
-        const int wf = __reduce_min_sync(0xffffffffu, first);
-        __syncthreads();
-        if ((threadIdx.x & 31) == 0) redi[threadIdx.x >> 5] = wf;
-        __syncthreads();
-        int ref = redi[0];
-#pragma unroll
-        for (int x = 1; x < STATE_THREADS / 32; ++x) ref = min(ref, redi[x]);
-        if (ref == INT_MAX) break;
-        T qr[MAXC];
-#pragma unroll
-        for (int k = 0; k < MAXC; ++k) qr[k] = (T)Qh[(size_t)k * n + ref];
+    if (__any_sync(0xffffffffu, want)) {
+        int at = 0, tot = 0;
 #pragma unroll
         for (int u = 0; u < STATE_UNROLL; ++u) {
-            if (!((want >> u) & 1u)) continue;
-            const int e = e0 + u * STATE_THREADS + threadIdx.x;
-            bool same = true;
-#pragma unroll
-            for (int k = 0; k < MAXC; ++k) same = same && bits_of((T)Qh[(size_t)k * n + e]) == bits_of(qr[k]);
-            if (!same) continue;
-            want &= ~(1u << u);
-            if (e == ref) kept |= 1u << u;
+            const unsigned m = __ballot_sync(0xffffffffu, (want >> u) & 1u);
+            at += __popc(m & ((1u << lane) - 1u));
+            tot += __popc(m);
         }
+        int base = lane == 0 ? atomicAdd(&nlist, tot) : 0;
+        at += __shfl_sync(0xffffffffu, base, 0);
+        for (; want; want &= want - 1u) list[at++] = (unsigned short)((__ffs(want) - 1) * STATE_THREADS + tid);
     }
-    want |= kept;
-    // the remaining cells' speeds by a few FP64 instructions (to 1e-15), then
-    // the formula itself for those within 1e-14 of the largest
+    __syncthreads();
+    const int nl = nlist;
+    auto state = [&](int p, double *q) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) q[k] = (double)(T)Qh[(size_t)k * n + e0 + list[p]];
+    };
+    double s0 = 0.0, s1 = 0.0;
+    auto formula = [&](int p) {
+        double q[4];
+        state(p, q);
+        const double pr = (I.gamma - 1.0) * (q[3] - 0.5 * (q[1] * q[1] + q[2] * q[2]) / q[0]);
+        const double c2 = sqrt(I.gamma * pr / q[0]);
+        s0 = fmax(s0, fabs(q[1] / q[0]) + c2);
+        s1 = fmax(s1, fabs(q[2] / q[0]) + c2);
+    };
+    if (nl <= 32) {   // no more than a warp: the formula at once
+        if (warp != 0) return;
+        if (lane < nl) formula(lane);
+        finish_warp<double>(Y[inst], true, s0, s1);
+        return;
+    }
     double w[STATE_UNROLL][2];
     unsigned long long k0 = 0ull, k1 = 0ull;
 #pragma unroll
     for (int u = 0; u < STATE_UNROLL; ++u) {
         w[u][0] = w[u][1] = 0.0;
-        if (!((want >> u) & 1u)) continue;
-        double q[MAXC];
-        state(u, q);
+        if (u * STATE_THREADS + tid >= nl) continue;
+        double q[4];
+        state(u * STATE_THREADS + tid, q);
         const double ir = rcp64(q[0]), p = press64<4>(I.g1h, q, ir), cs = sqrt64(I.gamma * (p * ir));
         w[u][0] = __fma_rn(abs64(q[1]), ir, cs);
         w[u][1] = __fma_rn(abs64(q[2]), ir, cs);
@@ -2986,28 +3022,22 @@ __global__ void __launch_bounds__(STATE_THREADS, 3) k_write_state(const InstDesc
         k0 = max(k0, __shfl_xor_sync(0xffffffffu, k0, o));
         k1 = max(k1, __shfl_xor_sync(0xffffffffu, k1, o));
     }
-    if ((threadIdx.x & 31) == 0) { redk[0][threadIdx.x >> 5] = k0; redk[1][threadIdx.x >> 5] = k1; }
+    if (lane == 0) { redk[0][warp] = k0; redk[1][warp] = k1; }
     __syncthreads();
     k0 = S[0];
     k1 = S[1];
 #pragma unroll
-    for (int x = 0; x < STATE_THREADS / 32; ++x) {
+    for (int x = 0; x < WARPS; ++x) {
         k0 = max(k0, redk[0][x]);
         k1 = max(k1, redk[1][x]);
     }
     const double t0 = __longlong_as_double((long long)k0) * (1.0 - 1e-14);
     const double t1 = __longlong_as_double((long long)k1) * (1.0 - 1e-14);
-    double s0 = 0.0, s1 = 0.0;
 #pragma unroll
     for (int u = 0; u < STATE_UNROLL; ++u) {
         // (a speed that is no number compares false either way)
-        if (!((want >> u) & 1u) || (key64(w[u][0]) < key64(t0) && key64(w[u][1]) < key64(t1))) continue;
-        double q[MAXC];
-        state(u, q);
-        const double p = (I.gamma - 1.0) * (q[3] - 0.5 * (q[1] * q[1] + q[2] * q[2]) / q[0]);
-        const double c2 = sqrt(I.gamma * p / q[0]);
-        s0 = fmax(s0, fabs(q[1] / q[0]) + c2);
-        s1 = fmax(s1, fabs(q[2] / q[0]) + c2);
+        if (u * STATE_THREADS + tid < nl && !(key64(w[u][0]) < key64(t0) && key64(w[u][1]) < key64(t1)))
+            formula(u * STATE_THREADS + tid);
     }
     finish_warp<double>(Y[inst], true, s0, s1);
 }
