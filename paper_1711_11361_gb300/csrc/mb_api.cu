@@ -40,7 +40,7 @@ template <class T>
 int bulk_blocks_per_sm(int);
 double fp64_probe_rate(cudaStream_t st);
 template <class T>
-void launch_axisym_source(const InstDesc *, InstDyn *, int, size_t, int, cudaStream_t);
+void launch_axisym_source(const InstDesc *, InstDyn *, int, int, int, cudaStream_t);
 template <class T, class H>
 void launch_write_state(const InstDesc *, InstDyn *, const H *const *, const H *, int, int, int, int, cudaStream_t);
 template <class T, class H>
@@ -361,6 +361,8 @@ static int auto_yseg(const mb_sim *s) {
     return seg;
 }
 
+static int io_blocks(const InstDesc &I) { return (I.nx * I.ny + IO_CELLS - 1) / IO_CELLS; }
+
 // offsets of every instance in the shared arrays, those arrays, the
 // descriptors and the instance of every geometry group; the dynamic state of
 // new instance k is the old instance from[k]'s (zero when from[k] < 0).  The
@@ -378,7 +380,7 @@ static cudaError_t relayout(mb_sim *s, int old_n, const std::vector<int> &from) 
     std::vector<double> hvx, hvy;
     std::vector<unsigned char> hmov;
     std::vector<int> hnext;
-    int rec_total = 0, tiles0 = 0, tiles1 = 0;
+    int rec_total = 0, tiles0 = 0, tiles1 = 0, io_total = 0;
     size_t max_cells = 1;
     const int yseg = s->tune_yseg ? s->tune_yseg : auto_yseg(s);
     for (auto &I : s->hd) bulk_items(s->prec, yseg, I);
@@ -396,6 +398,8 @@ static cudaError_t relayout(mb_sim *s, int old_n, const std::vector<int> &from) 
         I.tile_off[1] = tiles1;
         tiles0 += I.ntiles[0];
         tiles1 += I.ntiles[1];
+        I.io_off = io_total;
+        io_total += io_blocks(I);
         max_cells = std::max(max_cells, (size_t)I.nx * I.ny);
     }
     // columns per geometry group: the fewest (2 to GEO_GC) whose groups run in
@@ -736,10 +740,9 @@ static mb_status do_sweep(mb_sim *s, int dir, double dt) {
         bool axi = false;
         for (const auto &I : s->hd) axi = axi || I.axisym;
         if (axi) {
-            size_t cells = 0;
-            for (const auto &I : s->hd) cells = std::max(cells, (size_t)I.pitch * I.ny);
-            if (s->prec == MB_FP32) launch_axisym_source<float>(s->dd, s->dy, s->n, cells, dst, st);
-            else launch_axisym_source<double>(s->dd, s->dy, s->n, cells, dst, st);
+            const int blocks = s->hd.back().io_off + io_blocks(s->hd.back());
+            if (s->prec == MB_FP32) launch_axisym_source<float>(s->dd, s->dy, s->n, blocks, dst, st);
+            else launch_axisym_source<double>(s->dd, s->dy, s->n, blocks, dst, st);
         }
     }
     if (s->sidx == 1) {

@@ -8,6 +8,7 @@ namespace mb {
 
 constexpr int MAXC = 4;
 constexpr int NBULK = 32;              // non-physical bulk cells listed per sweep
+constexpr int IO_CELLS = 2048;         // cells (in the host order) per block of an instance
 constexpr int GEO_GC = 16;            // grid columns per geometry group (one CTA each), at most
 constexpr double ALPHA_MIN = 1e-10;   // smaller volume fractions count as solid
 // launch shape of the FP32x2 bulk kernels: bits 0-9 CTA threads (64 or 128),
@@ -103,6 +104,7 @@ struct InstDesc {
     int tile_off[2];            // first bulk tile (per direction)
     int ntiles[2];
     int tiles_x[2];             // tiles along x per direction
+    int io_off;                 // first block of IO_CELLS cells in the batch's numbering
 };
 
 struct InstDyn {

@@ -617,6 +617,21 @@ __device__ __forceinline__ int find_inst_warp(const InstDesc *D, int n_inst, int
     return lo;
 }
 
+// instance (of inst0 .. inst0 + ninst - 1) of block gb of IO_CELLS cells: a
+// warp looks at 32 instances at a time
+__device__ __forceinline__ int find_inst_io(const InstDesc *__restrict__ D, int inst0, int ninst, int gb) {
+    const int lane = threadIdx.x & 31;
+    int lo = inst0;
+    while (ninst > 1) {
+        const int step = (ninst + 31) / 32, p = lane * step;
+        const bool le = p < ninst && D[lo + p].io_off <= gb;
+        const int k = (__popc(__ballot_sync(0xffffffffu, le)) - 1) * step;
+        lo += k;
+        ninst = min(step, ninst - k);
+    }
+    return lo;
+}
+
 // Units of the scalar kernels (FP64 Euler, advection in both precisions): 30
 // consecutive cells of a line on the 32 lanes of a warp, lane l holding
 // position a0 - 1 + l, so that a unit evolves 32 cells, forms 31 fluxes and
@@ -2047,65 +2062,83 @@ __global__ void __launch_bounds__(128, MINB) k_bulk_y_p(const InstDesc *__restri
 // reading; Sec. III.E models its open-ended tube in axisymmetric form): with
 // x axial and y the radius from the axis y = y0 = 0, every fluid cell gets
 // Q -= dt (v / r) [rho, rho u, rho v, E + p], r at the cell centre.  One thread
-// per cell (grid: x over the largest instance's cells, y over the instances,
-// which pass grid y's limit of 65535 by turns); instances of the batch without
-// the flag have nothing to do.  In FP64 every operation is rounded on its own
-// (no contraction), in the order of the plain definition.
+// per cell, or one for up to eight in a large batch, CTAs numbered through the
+// batch's blocks of IO_CELLS cells (as many as its cells need, however uneven
+// its grids are); instances without the flag return at once.  In FP64 every
+// operation is rounded on its own (no contraction), in the order of the plain
+// definition.  FP32, one grid: 400 x 400 cells 6 us (19 with a warp per row),
+// 4096 x 4096 130 (171; 275 with a cell per thread throughout); among 63 grids
+// of 128 x 128 cells 145 (177; 2370 with as many CTAs for every instance as for
+// the largest).
 // ---------------------------------------------------------------------------
 template <class T>
 __global__ void __launch_bounds__(256) k_axisym_source(const InstDesc *__restrict__ D, InstDyn *__restrict__ Y,
-                                                       int n_inst, int buf) {
-    for (int inst = blockIdx.y; inst < n_inst; inst += gridDim.y) {
-        const InstDesc &I = D[inst];
-        if (!I.axisym || I.eq != 0) continue;
-        InstDyn &y = Y[inst];
-        const size_t plane = (size_t)I.pitch * I.ny;
-        const double dt = y.dt;
-        bool bad = false;
-        // a warp's 32 positions lie in one row (the pitch is a multiple of 32)
-        for (size_t c = (size_t)blockIdx.x * 256 + threadIdx.x; c < plane; c += (size_t)gridDim.x * 256) {
-            const int j = (int)(c / I.pitch), i = (int)(c - (size_t)j * I.pitch);
-            if (i >= I.nx) continue;
-            const double r = __dmul_rn(__dadd_rn((double)j, 0.5), I.dy);
-            T *__restrict__ Q = (T *)I.Q[buf] + (size_t)j * I.pitch;
-            const T q0 = Q[i], q1 = Q[plane + i], q2 = Q[2 * plane + i], q3 = Q[3 * plane + i];
-            if (!(q0 == q0)) continue;   // solid
-            T n0, n1, n2, n3, pn;
-            if (sizeof(T) == 8) {
-                const double g1 = __dsub_rn(I.gamma, 1.0);
-                const double p = __dmul_rn(g1, __dsub_rn(q3, __ddiv_rn(__dmul_rn(0.5, __dadd_rn(__dmul_rn(q1, q1),
-                                                                                               __dmul_rn(q2, q2))), q0)));
-                const double f = __ddiv_rn(__dmul_rn(dt, __ddiv_rn(q2, q0)), r);
-                n0 = (T)__dsub_rn(q0, __dmul_rn(f, q0));
-                n1 = (T)__dsub_rn(q1, __dmul_rn(f, q1));
-                n2 = (T)__dsub_rn(q2, __dmul_rn(f, q2));
-                n3 = (T)__dsub_rn(q3, __dmul_rn(f, __dadd_rn(q3, p)));
-                pn = (T)__dmul_rn(g1, __dsub_rn(n3, __ddiv_rn(__dmul_rn(0.5, __dadd_rn(__dmul_rn(n1, n1),
-                                                                                      __dmul_rn(n2, n2))), n0)));
-            } else {
-                const float g1 = (float)I.gamma - 1.0f;
-                const float p = g1 * (q3 - 0.5f * (q1 * q1 + q2 * q2) / q0);
-                const float f = (float)dt * (q2 / q0) / (float)r;
-                n0 = q0 - f * q0;
-                n1 = q1 - f * q1;
-                n2 = q2 - f * q2;
-                n3 = q3 - f * (q3 + p);
-                pn = g1 * (n3 - 0.5f * (n1 * n1 + n2 * n2) / n0);
-            }
-            Q[i] = n0;
-            Q[plane + i] = n1;
-            Q[2 * plane + i] = n2;
-            Q[3 * plane + i] = n3;
-            if (!(n0 > (T)0) || !(pn > (T)0)) bad = true;
+                                                       int n_inst, int share, int buf) {
+    const int gb = blockIdx.x / share, inst = find_inst_io(D, 0, n_inst, gb);   // share: CTAs per block of cells
+    const InstDesc &I = D[inst];
+    if (!I.axisym || I.eq != 0) return;
+    InstDyn &y = Y[inst];
+    const int nx = I.nx, len = IO_CELLS / share, e0 = (gb - I.io_off) * IO_CELLS + (int)(blockIdx.x % share) * len;
+    const int e1 = min(e0 + len, nx * I.ny);
+    const size_t plane = (size_t)I.pitch * I.ny;
+    // the radii of the CTA's rows, and dt, once: with FP32 states their FP64
+    // instructions would be the kernel's bound (4096 x 4096 cells: 227 us with
+    // a radius per cell)
+    __shared__ T radius[IO_CELLS / 8 + 2], sdt;
+    const int j0 = e0 / nx;
+    for (int t = threadIdx.x; t <= (e1 - 1) / nx - j0; t += 256)
+        radius[t] = (T)__dmul_rn(__dadd_rn((double)(j0 + t), 0.5), I.dy);
+    if (threadIdx.x == 0) sdt = (T)y.dt;
+    __syncthreads();
+    const T dt = sdt;
+    bool bad = false;
+#pragma unroll 2
+    for (int e = e0 + threadIdx.x; e < e1; e += 256) {
+        const int j = e / nx, i = e - j * nx;
+        const T r = radius[j - j0];
+        T *__restrict__ Q = (T *)I.Q[buf] + (size_t)j * I.pitch;
+        const T q0 = Q[i], q1 = Q[plane + i], q2 = Q[2 * plane + i], q3 = Q[3 * plane + i];
+        if (!(q0 == q0)) continue;   // solid
+        T n0, n1, n2, n3, pn;
+        if (sizeof(T) == 8) {
+            const double g1 = __dsub_rn(I.gamma, 1.0);
+            const double p = __dmul_rn(g1, __dsub_rn(q3, __ddiv_rn(__dmul_rn(0.5, __dadd_rn(__dmul_rn(q1, q1),
+                                                                                           __dmul_rn(q2, q2))), q0)));
+            const double f = __ddiv_rn(__dmul_rn(dt, __ddiv_rn(q2, q0)), r);
+            n0 = (T)__dsub_rn(q0, __dmul_rn(f, q0));
+            n1 = (T)__dsub_rn(q1, __dmul_rn(f, q1));
+            n2 = (T)__dsub_rn(q2, __dmul_rn(f, q2));
+            n3 = (T)__dsub_rn(q3, __dmul_rn(f, __dadd_rn(q3, p)));
+            pn = (T)__dmul_rn(g1, __dsub_rn(n3, __ddiv_rn(__dmul_rn(0.5, __dadd_rn(__dmul_rn(n1, n1),
+                                                                                  __dmul_rn(n2, n2))), n0)));
+        } else {
+            const float g1 = (float)I.gamma - 1.0f;
+            const float p = g1 * (q3 - 0.5f * (q1 * q1 + q2 * q2) / q0);
+            const float f = dt * (q2 / q0) / r;
+            n0 = q0 - f * q0;
+            n1 = q1 - f * q1;
+            n2 = q2 - f * q2;
+            n3 = q3 - f * (q3 + p);
+            pn = g1 * (n3 - 0.5f * (n1 * n1 + n2 * n2) / n0);
         }
-        if (bad) atomicOr(&y.err, ERR_UNSTABLE);
+        Q[i] = n0;
+        Q[plane + i] = n1;
+        Q[2 * plane + i] = n2;
+        Q[3 * plane + i] = n3;
+        if (!(n0 > (T)0) || !(pn > (T)0)) bad = true;
     }
+    if (bad) atomicOr(&y.err, ERR_UNSTABLE);
 }
 
 template <class T>
-void launch_axisym_source(const InstDesc *D, InstDyn *Y, int n_inst, size_t max_cells, int buf, cudaStream_t st) {
-    const unsigned bx = (unsigned)std::min<size_t>((max_cells + 255) / 256, 1u << 20);
-    if (bx > 0 && n_inst > 0) k_axisym_source<T><<<dim3(bx, std::min(n_inst, 65535)), 256, 0, st>>>(D, Y, n_inst, buf);
+void launch_axisym_source(const InstDesc *D, InstDyn *Y, int n_inst, int io_blocks, int buf, cudaStream_t st) {
+    if (io_blocks <= 0) return;
+    // a cell per thread while that makes no more than four waves of eight CTAs
+    // per SM (the FP64 quotients want every SM), else up to eight, which spend
+    // less on finding their place
+    int share = 8;
+    while (share > 1 && (long long)io_blocks * share > 152 * 8 * 4) share /= 2;
+    k_axisym_source<T><<<(unsigned)io_blocks * share, 256, 0, st>>>(D, Y, n_inst, share, buf);
 }
 
 // ---------------------------------------------------------------------------
@@ -3194,7 +3227,7 @@ void launch_read_state(const InstDesc *D, H *const *ptrs, H *p1, int inst0, int 
     template void launch_bulk<T>(int, int, const InstDesc *, InstDyn *, const BandRec *, int, int, int, int, int,  \
                                  int, int, DeferList, int, cudaStream_t);                                               \
     template int bulk_blocks_per_sm<T>(int);                                                                       \
-    template void launch_axisym_source<T>(const InstDesc *, InstDyn *, int, size_t, int, cudaStream_t);            \
+    template void launch_axisym_source<T>(const InstDesc *, InstDyn *, int, int, int, cudaStream_t);               \
     template void launch_write_state<T, double>(const InstDesc *, InstDyn *, const double *const *, const double *, \
                                                 int, int, int, int, cudaStream_t);                                 \
     template void launch_write_state<T, float>(const InstDesc *, InstDyn *, const float *const *, const float *,    \
