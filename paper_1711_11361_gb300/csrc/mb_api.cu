@@ -361,7 +361,13 @@ static int auto_yseg(const mb_sim *s) {
     return seg;
 }
 
+// blocks of IO_CELLS cells: of an instance, and of cnt instances from k0 on
 static int io_blocks(const InstDesc &I) { return (I.nx * I.ny + IO_CELLS - 1) / IO_CELLS; }
+static int io_span(const mb_sim *s, int k0, int cnt) {
+    if (cnt < 1) return 0;
+    const InstDesc &last = s->hd[k0 + cnt - 1];
+    return last.io_off + io_blocks(last) - s->hd[k0].io_off;
+}
 
 // offsets of every instance in the shared arrays, those arrays, the
 // descriptors and the instance of every geometry group; the dynamic state of
@@ -740,7 +746,7 @@ static mb_status do_sweep(mb_sim *s, int dir, double dt) {
         bool axi = false;
         for (const auto &I : s->hd) axi = axi || I.axisym;
         if (axi) {
-            const int blocks = s->hd.back().io_off + io_blocks(s->hd.back());
+            const int blocks = io_span(s, 0, s->n);
             if (s->prec == MB_FP32) launch_axisym_source<float>(s->dd, s->dy, s->n, blocks, dst, st);
             else launch_axisym_source<double>(s->dd, s->dy, s->n, blocks, dst, st);
         }
@@ -891,7 +897,6 @@ static mb_status write_states(mb_sim *sim, int k0, int cnt, const H *const *Q, c
     }
     cudaStream_t st = sim->stream;
     std::vector<InstDyn> ys(cnt);
-    int max_cells = 0;
     for (int q = 0; q < cnt; ++q) {
         const InstDesc &I = sim->hd[k0 + q];
         InstDyn &y = ys[q];
@@ -900,20 +905,20 @@ static mb_status write_states(mb_sim *sim, int k0, int cnt, const H *const *Q, c
         y.X = I.U[0] * t[q];
         y.Y = I.U[1] * t[q];
         y.th = I.rotating ? I.a0 + I.a1 * std::sin(I.omega * t[q]) : 0.0;
-        max_cells = std::max(max_cells, I.nx * I.ny);
     }
     cudaError_t e = cudaMemcpyAsync(sim->dy + k0, ys.data(), cnt * sizeof(InstDyn), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_check(sim, e, "write_state copy");
-    auto launch = [&](const H *const *ptrs, const H *p1, int i0, int ni, int mc) {
-        if (sim->prec == MB_FP32) launch_write_state<float, H>(sim->dd, sim->dy, ptrs, p1, i0, ni, mc, sim->cur, st);
-        else launch_write_state<double, H>(sim->dd, sim->dy, ptrs, p1, i0, ni, mc, sim->cur, st);
+    auto launch = [&](const H *const *ptrs, const H *p1, int i0, int ni) {
+        const int nb = io_span(sim, i0, ni);
+        if (sim->prec == MB_FP32) launch_write_state<float, H>(sim->dd, sim->dy, ptrs, p1, i0, ni, nb, sim->cur, st);
+        else launch_write_state<double, H>(sim->dd, sim->dy, ptrs, p1, i0, ni, nb, sim->cur, st);
     };
     H *const stage1 = (H *)sim->stage;   // the batch buffer is taken after batch_stage (it may allocate)
     if (cnt == 1) {
         e = cudaMemcpyAsync(stage1, Q[0], state_elems(sim->hd[k0]) * sizeof(H), cudaMemcpyHostToDevice, st);
         if (e != cudaSuccess) return cuda_check(sim, e, "write_state copy");
         classify_instances(sim, k0, 1, nullptr, st);
-        launch(nullptr, stage1, k0, 1, max_cells);
+        launch(nullptr, stage1, k0, 1);
     } else {
         std::vector<size_t> off;
         e = batch_stage(sim, off);
@@ -934,7 +939,7 @@ static mb_status write_states(mb_sim *sim, int k0, int cnt, const H *const *Q, c
             e = cudaMemcpyAsync(sim->iop, ptrs.data(), cnt * sizeof(H *), cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(st, sim->ev_join, 0);
         if (e != cudaSuccess) return cuda_check(sim, e, "write_states copy");
-        launch((const H *const *)sim->iop, nullptr, k0, cnt, max_cells);
+        launch((const H *const *)sim->iop, nullptr, k0, cnt);
     }
     e = cudaStreamSynchronize(st);
     if (e == cudaSuccess) e = cudaGetLastError();
@@ -952,15 +957,16 @@ template <class H>
 static mb_status read_states(mb_sim *sim, int k0, int cnt, H *const *Q, std::vector<InstDyn> &ys) {
     cudaStream_t st = sim->stream;
     const int buf = sim->sidx == 0 ? sim->cur : (sim->qn + 1) % 3;
-    auto launch = [&](H *const *ptrs, H *p1, int i0, int ni, int max_cells) {
-        if (sim->prec == MB_FP32) launch_read_state<float, H>(sim->dd, ptrs, p1, i0, ni, max_cells, buf, st);
-        else launch_read_state<double, H>(sim->dd, ptrs, p1, i0, ni, max_cells, buf, st);
+    auto launch = [&](H *const *ptrs, H *p1, int i0, int ni) {
+        const int nb = io_span(sim, i0, ni);
+        if (sim->prec == MB_FP32) launch_read_state<float, H>(sim->dd, ptrs, p1, i0, ni, nb, buf, st);
+        else launch_read_state<double, H>(sim->dd, ptrs, p1, i0, ni, nb, buf, st);
     };
     H *const stage1 = (H *)sim->stage;   // the batch buffer is taken after batch_stage (it may allocate)
     cudaError_t e = cudaSuccess;
     if (cnt == 1) {
         if (Q[0]) {
-            launch(nullptr, stage1, k0, 1, sim->hd[k0].nx * sim->hd[k0].ny);
+            launch(nullptr, stage1, k0, 1);
             e = cudaMemcpyAsync(Q[0], stage1, state_elems(sim->hd[k0]) * sizeof(H), cudaMemcpyDeviceToHost, st);
         }
     } else {
@@ -969,14 +975,14 @@ static mb_status read_states(mb_sim *sim, int k0, int cnt, H *const *Q, std::vec
         if (e != cudaSuccess) return cuda_check(sim, e, "read_states staging");
         H *const bst = (H *)sim->bstage;
         std::vector<H *> ptrs(cnt, nullptr);
-        int max_cells = 0;
+        bool any = false;
         for (int q = 0; q < cnt; ++q) {
             if (!Q[q]) continue;
             ptrs[q] = bst + off[k0 + q];
-            max_cells = std::max(max_cells, sim->hd[k0 + q].nx * sim->hd[k0 + q].ny);
+            any = true;
         }
         e = cudaMemcpyAsync(sim->iop, ptrs.data(), cnt * sizeof(H *), cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess) launch((H *const *)sim->iop, nullptr, k0, cnt, max_cells);
+        if (e == cudaSuccess && any) launch((H *const *)sim->iop, nullptr, k0, cnt);
         for (int q = 0; q < cnt && e == cudaSuccess; ++q)
             if (Q[q])
                 e = cudaMemcpyAsync(Q[q], ptrs[q], state_elems(sim->hd[k0 + q]) * sizeof(H), cudaMemcpyDeviceToHost,

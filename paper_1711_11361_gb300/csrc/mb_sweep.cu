@@ -2853,21 +2853,22 @@ __global__ void k_finalize(const InstDesc *__restrict__ D, InstDyn *__restrict__
 
 // ---------------------------------------------------------------------------
 // state initialisation and the CFL wave speeds of a state; state read-back.
-// One CTA per STATE_CELLS consecutive cells of one instance (instance inst0 +
-// blockIdx.y) in the host order; the host layout lives in a device staging
-// buffer (one per instance, or one per batch with a pointer per instance).
+// One CTA per block of IO_CELLS consecutive cells, in the host order, of the
+// instances inst0 .. inst0 + ninst - 1 (numbered through them: an uneven batch
+// has no empty CTAs); the host layout lives in a device staging buffer (one
+// per instance, or one per batch with a pointer per instance).
 // (One CTA per 8 rows, walked one after the other, left a single instance
 // to a few CTAs: reading 400 x 400 cells back took 65 us, now 20.)
 // ---------------------------------------------------------------------------
 constexpr int STATE_THREADS = 256;
 constexpr int STATE_UNROLL = 8;
-constexpr int STATE_CELLS = STATE_THREADS * STATE_UNROLL;
+static_assert(STATE_THREADS * STATE_UNROLL == IO_CELLS, "a CTA takes a block of cells");
 
 __device__ __forceinline__ unsigned long long bits_of(double v) { return (unsigned long long)__double_as_longlong(v); }
 __device__ __forceinline__ unsigned long long bits_of(float v) { return __float_as_uint(v); }
 
-// Sources: srcs[blockIdx.y] (srcs != nullptr; a null entry skips that
-// instance) or src1.  The first step's wave speeds are the FP64 maxima over
+// Sources: srcs[k] for instance inst0 + k (srcs != nullptr; a null entry skips
+// that instance) or src1.  The first step's wave speeds are the FP64 maxima over
 // the stored (T-rounded) states.  Cells in the state that their warp took last
 // drop out by their bits (a uniform region costs a cell per warp).  The others'
 // speeds are formed in FP32; a cell goes through the FP64 formula only if one
@@ -2886,18 +2887,18 @@ template <class T, class H>
 __global__ void __launch_bounds__(STATE_THREADS, 4) k_write_state(const InstDesc *__restrict__ D,
                                                                InstDyn *__restrict__ Y,
                                                                const H *const *__restrict__ srcs,
-                                                               const H *__restrict__ src1, int inst0, int b) {
+                                                               const H *__restrict__ src1, int inst0, int ninst,
+                                                               int b) {
     constexpr int WARPS = STATE_THREADS / 32, GROUP = 4;
     __shared__ float red[2][WARPS];
     __shared__ unsigned long long redk[2][WARPS];
-    __shared__ unsigned short list[STATE_CELLS];
+    __shared__ unsigned short list[IO_CELLS];
     __shared__ int nlist;
-    const int inst = inst0 + blockIdx.y;
-    const H *__restrict__ Qh = srcs ? srcs[blockIdx.y] : src1;
+    const int gb = D[inst0].io_off + blockIdx.x, inst = find_inst_io(D, inst0, ninst, gb);
+    const H *__restrict__ Qh = srcs ? srcs[inst - inst0] : src1;
     if (!Qh) return;
     const InstDesc &I = D[inst];
-    const int nx = I.nx, n = nx * I.ny, e0 = blockIdx.x * STATE_CELLS;
-    if (e0 >= n) return;
+    const int nx = I.nx, n = nx * I.ny, e0 = (gb - I.io_off) * IO_CELLS;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const size_t plane = (size_t)I.pitch * I.ny;
     T *Q = bufw<T>(I, b);
@@ -3075,17 +3076,17 @@ __global__ void __launch_bounds__(STATE_THREADS, 4) k_write_state(const InstDesc
     finish_warp<double>(Y[inst], true, s0, s1);
 }
 
-// Destinations: dsts[blockIdx.y] (null entry: skip) or dst1; nc planes of
+// Destinations: dsts[k] (null entry: skip) or dst1; nc planes of
 // nx*ny values of type H (FP64 or FP32), solid cells NaN.
 template <class T, class H>
 __global__ void __launch_bounds__(STATE_THREADS) k_read_state(const InstDesc *__restrict__ D,
                                                               H *const *__restrict__ dsts,
-                                                              H *__restrict__ dst1, int inst0, int b) {
-    const int inst = inst0 + blockIdx.y;
-    H *__restrict__ out = dsts ? dsts[blockIdx.y] : dst1;
+                                                              H *__restrict__ dst1, int inst0, int ninst, int b) {
+    const int gb = D[inst0].io_off + blockIdx.x, inst = find_inst_io(D, inst0, ninst, gb);
+    H *__restrict__ out = dsts ? dsts[inst - inst0] : dst1;
     if (!out) return;
     const InstDesc &I = D[inst];
-    const int n = I.nx * I.ny, e0 = blockIdx.x * STATE_CELLS;
+    const int n = I.nx * I.ny, e0 = (gb - I.io_off) * IO_CELLS;
     const size_t plane = (size_t)I.pitch * I.ny;
     const T *__restrict__ Q = buf<T>(I, b);
 #pragma unroll
@@ -3206,19 +3207,17 @@ int bulk_blocks_per_sm(int dir) {
     return 1;
 }
 
-// instances inst0 .. inst0+ninst-1 (max_cells: their largest nx * ny); per-instance
-// pointers in the device array ptrs, or one pointer p1 (ninst == 1)
+// instances inst0 .. inst0+ninst-1 (blocks: their blocks of IO_CELLS cells);
+// per-instance pointers in the device array ptrs, or one pointer p1 (ninst == 1)
 template <class T, class H>
 void launch_write_state(const InstDesc *D, InstDyn *Y, const H *const *ptrs, const H *p1, int inst0, int ninst,
-                        int max_cells, int b, cudaStream_t st) {
-    const dim3 grid((max_cells + STATE_CELLS - 1) / STATE_CELLS, ninst);
-    if (ninst > 0 && max_cells > 0) k_write_state<T, H><<<grid, STATE_THREADS, 0, st>>>(D, Y, ptrs, p1, inst0, b);
+                        int blocks, int b, cudaStream_t st) {
+    if (blocks > 0) k_write_state<T, H><<<blocks, STATE_THREADS, 0, st>>>(D, Y, ptrs, p1, inst0, ninst, b);
 }
 template <class T, class H>
-void launch_read_state(const InstDesc *D, H *const *ptrs, H *p1, int inst0, int ninst, int max_cells, int b,
+void launch_read_state(const InstDesc *D, H *const *ptrs, H *p1, int inst0, int ninst, int blocks, int b,
                        cudaStream_t st) {
-    const dim3 grid((max_cells + STATE_CELLS - 1) / STATE_CELLS, ninst);
-    if (ninst > 0 && max_cells > 0) k_read_state<T, H><<<grid, STATE_THREADS, 0, st>>>(D, ptrs, p1, inst0, b);
+    if (blocks > 0) k_read_state<T, H><<<blocks, STATE_THREADS, 0, st>>>(D, ptrs, p1, inst0, ninst, b);
 }
 
 #define MB_INST(T)                                                                                                \

@@ -68,3 +68,57 @@ def test_cost_of_the_source_in_an_uneven_batch():
         t.append(_best(steps))
         sim.close()
     assert t[1] <= 2.0 * t[0], t
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("count", [2, 31, 32, 33, 65, 1030])
+def test_states_of_every_instance(count, precision):
+    """Every instance's own state in and out, some left out of the read; the first step from each one's own speeds."""
+    from paper_1711_11361_gb300 import mb
+    kinds = [_tube(nx, ny, False, k) for k, (nx, ny) in enumerate(SIZES)]
+    order = np.random.default_rng(count).integers(0, len(SIZES), count)
+    scale = 1.0 + np.arange(count) % 64 / 64.0
+    states = [kinds[k].Q0 * s for k, s in zip(order, scale)]
+    dtype = np.float32 if precision else np.float64
+    sim = mb.Sim([kinds[k] for k in order], precision, write_initial=False)
+    sim.write_states(states)
+    out = [np.full(q.shape, -7.0) for q in states]
+    ptrs = sim._ptrs(out)
+    for at in range(0, count, 3):
+        ptrs[at] = None
+    clk = np.empty((count, 4))
+    sim._check(mb.lib.mb_read_states(sim._h, ptrs, mb._dp(clk)))
+    for at in range(count):
+        assert np.array_equal(out[at], np.full(out[at].shape, -7.0) if at % 3 == 0 else states[at].astype(dtype)), at
+    got = sim.step(0.0, report=True)
+    sim.close()
+    for k in set(order.tolist()):
+        q = [states[at].astype(dtype).astype(np.float64) for at in np.where(order == k)[0]]
+        for at, x in zip(np.where(order == k)[0], q):
+            p = kinds[k]
+            c = np.sqrt(p.gamma * (p.gamma - 1.0) * (x[3] - 0.5 * (x[1] ** 2 + x[2] ** 2) / x[0]) / x[0])
+            want = p.cfl * min(p.dx / np.max(np.abs(x[1] / x[0]) + c), p.dy / np.max(np.abs(x[2] / x[0]) + c))
+            assert abs(got[at] - want) <= 1e-14 * want, at
+
+
+def test_cost_of_state_copies_in_an_uneven_batch():
+    """Writing and reading 2000 grids of 8 x 8 cells and one of 4096 x 4096 takes about as long as the small ones and
+    the large one apart (well beyond the bar where every instance got as many CTAs as the largest)."""
+    import torch
+
+    from paper_1711_11361_gb300 import mb
+
+    def cost(shapes):
+        probs = [_tube(8, 8, False) for _ in range(shapes.count(8))]
+        probs += [inputs.Problem("large", 4096, 4096, 0.0, 0.0, 1.0, 1.0) for _ in range(shapes.count(4096))]
+        bufs = [torch.empty((4, p.ny, p.nx), pin_memory=True) for p in probs]
+        for b in bufs:
+            b[:] = torch.tensor([1.0, 0.1, 0.2, 2.5])[:, None, None]
+        sim = mb.Sim(probs, mb.FP32, write_initial=False)
+        at = [b.data_ptr() for b in bufs]
+        t = _best(lambda: (sim.write_states(at, dtype=np.float32), sim.read_states(out=at, dtype=np.float32)))
+        sim.close()
+        return t
+
+    both, apart = cost([8] * 2000 + [4096]), cost([8] * 2001) + cost([4096, 8])
+    assert both <= 1.5 * apart, (both, apart)
