@@ -774,10 +774,7 @@ __device__ __forceinline__ bool unit_update(const InstDesc &I, InstDyn &y, const
         if (!ok) m0 = m1 = 0.0f;
     }
     new_state(f, q0, F, Fhi, last, ci, y, m0, m1, qn, s0, s1);
-    if (EQ == 1 && last) {
-        s0 = (T)fabs(I.adv[0]);
-        s1 = (T)fabs(I.adv[1]);
-    }
+    if (EQ == 1) s0 = T(1);   // (put_advection: the warp has a fluid cell)
     return true;
 }
 
@@ -789,6 +786,19 @@ __device__ __forceinline__ bool unit_update(const InstDesc &I, InstDyn &y, const
 // (UNITS_NEAR); both launches decide by the same test.  UNITS_ALL: one launch
 // over every unit, after the band fluxes.
 enum { UNITS_FAR = 0, UNITS_NEAR = 1, UNITS_ALL = 2 };
+
+// the wave speeds of advection, constants, for a warp with a fluid cell; an
+// atomic only until they stand (one for every warp of 4.2 M cells: 174 us for
+// an x sweep of 34)
+template <class T>
+__device__ __forceinline__ void put_advection(const InstDesc &I, InstDyn &y, bool fluid) {
+    if (!__any_sync(0xffffffffu, fluid) || (threadIdx.x & 31) != 0) return;
+    volatile const unsigned long long *S = y.S;
+    for (int d = 0; d < 2; ++d) {
+        const double v = (double)(T)fabs(I.adv[d]);
+        if (pos64(v) && (unsigned long long)__double_as_longlong(v) > S[d]) atomic_max_pos(&y.S[d], v);
+    }
+}
 
 // x sweep: one warp per unit; the three states a lane needs are plain loads
 // (the neighbours' come from L1)
@@ -843,7 +853,8 @@ __global__ void __launch_bounds__(128, 4) k_unit_x(const InstDesc *__restrict__ 
 #pragma unroll
         for (int k = 0; k < NC; ++k) Qo[k * plane] = qn[k];
     }
-    finish_warp<T>(y, last != 0, s0, s1);
+    if (EQ == 0) finish_warp<T>(y, last != 0, s0, s1);
+    else if (last) put_advection<T>(I, y, s0 > T(0));
 }
 
 // y sweep: one CTA per 8 columns and 30 rows, a warp per column with its
@@ -916,7 +927,8 @@ __global__ void __launch_bounds__(256, 2) k_unit_y(const InstDesc *__restrict__ 
         }
     }
     if (lane >= 1 && lane <= UNIT_CELLS) sst[lane - 1][w] = st;
-    finish_warp<T>(y, last != 0, s0, s1);
+    if (EQ == 0) finish_warp<T>(y, last != 0, s0, s1);
+    else if (last) put_advection<T>(I, y, s0 > T(0));
     __syncthreads();
     T *__restrict__ Qo = (T *)I.Q[dst];
     for (int e = threadIdx.x; e < UNIT_CELLS * UNIT_COLS; e += 256) {
