@@ -704,9 +704,10 @@ static mb_status do_sweep(mb_sim *s, int dir, double dt) {
                                 s->tune_cta[dir], mode, dl, any_dall ? 1 : 0, st);
     };
     // the FP32 Euler kernels always run in two passes (mb_set_overlap acts
-    // through defer_all); the scalar ones in one when the overlap is off
+    // through defer_all); the scalar ones in one when the overlap is off or no
+    // instance has a body
     const bool packed = s->prec == MB_FP32 && eq == MB_EULER;
-    const bool two_pass = packed || s->overlap;
+    const bool two_pass = packed || (s->overlap && s->total_v > 0);
     if (two_pass && !s->timing) {
         // geometry and band fluxes (FP64 pipe, latency) on the side stream
         // while the bulk pass that needs no band data (FP32 pipe, HBM) runs
@@ -731,7 +732,7 @@ static mb_status do_sweep(mb_sim *s, int dir, double dt) {
             bulk(0);
             bulk(1);
         } else {
-            bulk(2);   // every unit in one launch
+            bulk(s->total_v > 0 ? 2 : 3);   // every unit in one launch
         }
         if (s->timing) {
             cudaEventRecord(e1, st);
