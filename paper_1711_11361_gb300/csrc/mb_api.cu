@@ -34,8 +34,8 @@ template <class T>
 void launch_band_stage(int, const InstDesc *, InstDyn *, BandRec *, const double *, int *, int, int, int, int,
                        int, int, int, int, cudaStream_t);
 template <class T>
-void launch_bulk(int, int, const InstDesc *, InstDyn *, const BandRec *, int, int, int, int, int, int, int, DeferList,
-                 int, cudaStream_t);
+void launch_bulk(int, int, const InstDesc *, InstDyn *, const BandRec *, int, int, int, int, int, int, int, int,
+                 DeferList, int, cudaStream_t);
 template <class T>
 int bulk_blocks_per_sm(int);
 double fp64_probe_rate(cudaStream_t st);
@@ -91,6 +91,7 @@ struct mb_sim {
     int gcw = GEO_GC;             // grid columns per geometry group
     int *ginst = nullptr;         // instance of each geometry group
     int total_tiles[2] = {0, 0};
+    int units = 1;                // units per warp of the scalar bulk kernels
     int bulk_grid[2] = {0, 0};
     // cell pairs whose bulk update waits for the band fluxes (FP32 Euler)
     int2 *ditem = nullptr;
@@ -234,16 +235,16 @@ static const char *check_instance(const mb_grid &g, const mb_body &b, int prec, 
 
 // bulk work items.  The FP32 Euler kernels: x sweep one warp per row, y sweep
 // one warp per 64 columns (two per thread) and yseg rows.  The scalar
-// kernels: units of 30 cells (x: one warp each; y: one CTA per 8 columns and
-// 30 rows)
-static void bulk_items(int prec, int yseg, InstDesc &I) {
+// kernels: units of 30 cells, `units` of them per warp (x: one warp each; y:
+// one CTA per 8 columns each and 30 rows)
+static void bulk_items(int prec, int yseg, int units, InstDesc &I) {
     if (prec == MB_FP32 && I.eq == MB_EULER) {
         I.tiles_x[0] = 1;
         I.tiles_x[1] = (I.nx + 63) / 64;
         I.yseg = yseg;
     } else {
-        I.tiles_x[0] = (I.nx + 29) / 30;
-        I.tiles_x[1] = (I.nx + 7) / 8;
+        I.tiles_x[0] = (I.nx + 30 * units - 1) / (30 * units);
+        I.tiles_x[1] = (I.nx + 8 * units - 1) / (8 * units);
         I.yseg = 30;
     }
     I.ntiles[0] = I.tiles_x[0] * I.ny;
@@ -310,7 +311,7 @@ static void describe_instance(int prec, int yseg, const mb_grid &g, double gamma
     }
     if (I.nv == 0) gcols = 0;
     I.gcol_max = gcols;
-    bulk_items(prec, yseg, I);
+    bulk_items(prec, yseg, 1, I);
 }
 
 // descriptor and device buffers of one instance
@@ -389,7 +390,16 @@ static cudaError_t relayout(mb_sim *s, int old_n, const std::vector<int> &from) 
     int rec_total = 0, tiles0 = 0, tiles1 = 0, io_total = 0;
     size_t max_cells = 1;
     const int yseg = s->tune_yseg ? s->tune_yseg : auto_yseg(s);
-    for (auto &I : s->hd) bulk_items(s->prec, yseg, I);
+    // units per warp of the scalar kernels: advection takes UNIT_WIDE in a batch
+    // that still fills the chip so, in FP32 with 32 warps per SM (584 k cells;
+    // 1024 x 1024 with a wall body 0.196 -> 0.192 ms per step, 400 x 400 0.170
+    // -> 0.177), in FP64, where more of the time is arithmetic, from 2 M cells
+    // on (1448 x 1448 0.349 -> 0.348, 1024 x 1024 0.253 -> 0.267)
+    long long cells = 0;
+    for (const auto &I : s->hd) cells += (long long)I.nx * I.ny;
+    const bool wide = s->eq == MB_ADVECTION && cells >= 30LL * UNIT_WIDE * (s->prec == MB_FP32 ? 32 : 112) * s->nsm;
+    s->units = wide ? UNIT_WIDE : 1;
+    for (auto &I : s->hd) bulk_items(s->prec, yseg, s->units, I);
     for (int k = 0; k < n; ++k) {
         InstDesc &I = s->hd[k];
         const InstHost &h = s->ih[k];
@@ -698,10 +708,10 @@ static mb_status do_sweep(mb_sim *s, int dir, double dt) {
 
         if (s->prec == MB_FP32)
             launch_bulk<float>(dir, eq, s->dd, s->dy, s->rec, s->n, s->total_tiles[dir], src, dst, last,
-                               s->tune_cta[dir], mode, dl, any_dall ? 1 : 0, st);
+                               s->tune_cta[dir], s->units, mode, dl, any_dall ? 1 : 0, st);
         else
             launch_bulk<double>(dir, eq, s->dd, s->dy, s->rec, s->n, s->total_tiles[dir], src, dst, last,
-                                s->tune_cta[dir], mode, dl, any_dall ? 1 : 0, st);
+                                s->tune_cta[dir], s->units, mode, dl, any_dall ? 1 : 0, st);
     };
     // the FP32 Euler kernels always run in two passes (mb_set_overlap acts
     // through defer_all); the scalar ones in one when the overlap is off or no
@@ -1174,10 +1184,10 @@ mb_status mb_autotune(mb_sim *sim, double *report) {
                 if (mode == 0) cudaMemsetAsync(sim->dcount, 0, sizeof(int), sim->stream);
                 if (sim->prec == MB_FP32)
                     launch_bulk<float>(dir, sim->eq, sim->dd, sim->dy, sim->rec, sim->n, sim->total_tiles[dir], src,
-                                       dst, 0, cta, mode, dl, 0, sim->stream);
+                                       dst, 0, cta, sim->units, mode, dl, 0, sim->stream);
                 else
                     launch_bulk<double>(dir, sim->eq, sim->dd, sim->dy, sim->rec, sim->n, sim->total_tiles[dir], src,
-                                        dst, 0, cta, mode, dl, 0, sim->stream);
+                                        dst, 0, cta, sim->units, mode, dl, 0, sim->stream);
             }
         };
         go();

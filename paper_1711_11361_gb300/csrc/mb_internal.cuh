@@ -8,6 +8,7 @@ namespace mb {
 
 constexpr int MAXC = 4;
 constexpr int NBULK = 32;              // non-physical bulk cells listed per sweep
+constexpr int UNIT_WIDE = 4;           // units per warp of large advection batches (mb_sweep.cu)
 constexpr int IO_CELLS = 2048;         // cells (in the host order) per block of an instance
 constexpr int GEO_GC = 16;            // grid columns per geometry group (one CTA each), at most
 constexpr double ALPHA_MIN = 1e-10;   // smaller volume fractions count as solid

@@ -644,8 +644,15 @@ __device__ __forceinline__ int find_inst_io(const InstDesc *__restrict__ D, int 
 // 2950 -> 1428 us, y 4090 -> 1430 us, 0.86 of the FP64 pipe's rate for the
 // 139 to 157 lane operations per cell this flow executes (263 in x and 289 in
 // y with CUDA's division and square root and comparisons on the FP64 pipe).
+// Advection takes a few operations per cell, so there a unit costs little more
+// than finding its place: large batches of it give a warp UNIT_WIDE units of a
+// row in x, and as many columns in y.  FP32 without a body, ms per step, one
+// unit -> four (a warp per row or 64 rows, which also suits large grids): 1024
+// x 1024 0.067 -> 0.052 (0.082), 4096 x 4096 0.474 -> 0.238 (0.243), 8192 x
+// 8192 1.74 -> 0.78 (0.78); FP64 6.96 -> 6.53 (7.01); eight units: 0.75, 6.51,
+// and slower below 2048 x 2048.
 constexpr int UNIT_CELLS = 30;
-constexpr int UNIT_COLS = 8;    // columns (lines) per CTA of the y sweep
+constexpr int UNIT_COLS = 8;    // columns (lines) per CTA of the y sweep and unit of a warp
 
 // the flow arithmetic of a unit by type and equation
 template <class T, int EQ>
@@ -802,38 +809,39 @@ __device__ __forceinline__ void put_advection(const InstDesc &I, InstDyn &y, boo
     }
 }
 
-// x sweep: one warp per unit; the three states a lane needs are plain loads
-// (the neighbours' come from L1)
-template <class T, int EQ>
+// x sweep: one warp per K units of a row; the three states a lane needs are
+// plain loads (the neighbours' come from L1)
+template <class T, int EQ, int K>
 __global__ void __launch_bounds__(128, 4) k_unit_x(const InstDesc *__restrict__ D, InstDyn *__restrict__ Y,
-                                                   const BandRec *__restrict__ R, int n_inst, int total_units, int src,
+                                                   const BandRec *__restrict__ R, int n_inst, int total_warps, int src,
                                                    int dst, int last, int mode) {
-    constexpr int NC = Flow<T, EQ>::NC;
+    constexpr int NC = Flow<T, EQ>::NC, CELLS = K * UNIT_CELLS;
     const int lane = threadIdx.x & 31;
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (gw >= total_units) return;
+    if (gw >= total_warps) return;
     const int inst = find_inst_warp(D, n_inst, gw, 0);
     const InstDesc &I = D[inst];
     InstDyn &y = Y[inst];
     const int local = gw - I.tile_off[0], ncg = I.tiles_x[0];
-    const int j = local / ncg, a0 = (local - j * ncg) * UNIT_CELLS;
+    const int j = local / ncg, a0 = (local - j * ncg) * CELLS;
     const int n = I.nx, bclo = I.bc[0], bchi = I.bc[1];
     const uint8_t *__restrict__ cls = I.cls + (size_t)j * I.pitch;
     bool fl;
     if (mode == UNITS_FAR || mode == UNITS_NEAR) {
-        bool far = j < y.row0 || j > y.row1 || (bclo != 2 && (a0 + UNIT_CELLS + 2 < y.col0 || a0 - 3 > y.col1));
+        bool far = j < y.row0 || j > y.row1 || (bclo != 2 && (a0 + CELLS + 2 < y.col0 || a0 - 3 > y.col1));
         if (!far && !y.defer_all) {
-            int t = cls[ghost_map(a0 - 3 + lane, n, bclo, bchi, &fl)];
-            if (lane < 4) t |= cls[ghost_map(a0 + 29 + lane, n, bclo, bchi, &fl)];
+            int t = 0;
+#pragma unroll
+            for (int p = 0; p < CELLS + 6; p += 32)
+                if (p + lane < CELLS + 6) t |= cls[ghost_map(a0 - 3 + p + lane, n, bclo, bchi, &fl)];
             far = !__any_sync(0xffffffffu, t & CLS_TOUCH);
         }
         if (far != (mode == UNITS_FAR)) return;
     }
     const size_t plane = (size_t)I.pitch * I.ny;
-    const int pos = a0 - 1 + lane;
     const T *__restrict__ Q = (const T *)I.Q[src] + (size_t)j * I.pitch;
-    T qm[NC], q0[NC], qp[NC], qn[NC];
-    int cm, c0, cp;
+    T qm[K][NC], q0[K][NC], qp[K][NC], qn[NC];
+    int cm[K], c0[K], cp[K];
     auto load = [&](int a, T *q, int &c) {
         bool flip;
         const int p = ghost_map(a, n, bclo, bchi, &flip);
@@ -842,32 +850,42 @@ __global__ void __launch_bounds__(128, 4) k_unit_x(const InstDesc *__restrict__ 
         for (int k = 0; k < NC; ++k) q[k] = __ldg(Q + k * plane + p);
         if (NC == 4 && flip) q[1] = -q[1];
     };
-    load(pos - 1, qm, cm);
-    load(pos, q0, c0);
-    load(pos + 1, qp, cp);
+#pragma unroll
+    for (int u = 0; u < K; ++u) {
+        const int pos = a0 + u * UNIT_CELLS - 1 + lane;
+        load(pos - 1, qm[u], cm[u]);
+        load(pos, q0[u], c0[u]);
+        load(pos + 1, qp[u], cp[u]);
+    }
     const Flow<T, EQ> f(I, sizeof(T) == 4 ? (T)y.lamf : (T)y.lam, 0);
     T s0 = T(0), s1 = T(0);
-    const bool st = mode == UNITS_FAR || mode == UNITS_PLAIN
-        ? unit_update<T, EQ, 0, false>(I, y, R, f, j, pos, n, qm, q0, qp, cm, c0, cp, last != 0, qn, s0, s1)
-        : unit_update<T, EQ, 0, true>(I, y, R, f, j, pos, n, qm, q0, qp, cm, c0, cp, last != 0, qn, s0, s1);
-    if (st) {
-        T *__restrict__ Qo = (T *)I.Q[dst] + (size_t)j * I.pitch + pos;
 #pragma unroll
-        for (int k = 0; k < NC; ++k) Qo[k * plane] = qn[k];
+    for (int u = 0; u < K; ++u) {
+        const int pos = a0 + u * UNIT_CELLS - 1 + lane;
+        const bool st = mode == UNITS_FAR || mode == UNITS_PLAIN
+            ? unit_update<T, EQ, 0, false>(I, y, R, f, j, pos, n, qm[u], q0[u], qp[u], cm[u], c0[u], cp[u], last != 0, qn,
+                                           s0, s1)
+            : unit_update<T, EQ, 0, true>(I, y, R, f, j, pos, n, qm[u], q0[u], qp[u], cm[u], c0[u], cp[u], last != 0, qn,
+                                          s0, s1);
+        if (st) {
+            T *__restrict__ Qo = (T *)I.Q[dst] + (size_t)j * I.pitch + pos;
+#pragma unroll
+            for (int k = 0; k < NC; ++k) Qo[k * plane] = qn[k];
+        }
     }
     if (EQ == 0) finish_warp<T>(y, last != 0, s0, s1);
     else if (last) put_advection<T>(I, y, s0 > T(0));
 }
 
-// y sweep: one CTA per 8 columns and 30 rows, a warp per column with its
-// lanes along the rows; the CTA's 34 x 8 states pass through shared memory
-// both ways, so that global loads and stores are 8 consecutive columns
-template <class T, int EQ>
+// y sweep: one CTA per 8 K columns and 30 rows, K columns per warp with its
+// lanes along the rows; the CTA's states pass through shared memory both
+// ways, so that global loads and stores are 8 K consecutive columns
+template <class T, int EQ, int K>
 __global__ void __launch_bounds__(256, 2) k_unit_y(const InstDesc *__restrict__ D, InstDyn *__restrict__ Y,
                                                    const BandRec *__restrict__ R, int n_inst, int src, int dst,
                                                    int last, int mode) {
-    constexpr int NC = Flow<T, EQ>::NC;
-    constexpr int ROWS = UNIT_CELLS + 4, LD = UNIT_COLS + 1;
+    constexpr int NC = Flow<T, EQ>::NC, COLS = K * UNIT_COLS;
+    constexpr int ROWS = UNIT_CELLS + 4, LD = COLS + 1;
     __shared__ T sq[NC][ROWS][LD];
     __shared__ uint8_t sc[ROWS][LD];
     __shared__ uint8_t sst[UNIT_CELLS][LD];
@@ -876,17 +894,17 @@ __global__ void __launch_bounds__(256, 2) k_unit_y(const InstDesc *__restrict__ 
     const InstDesc &I = D[inst];
     InstDyn &y = Y[inst];
     const int local = blockIdx.x - I.tile_off[1], ncg = I.tiles_x[1];
-    const int sg = local / ncg, i0 = (local - sg * ncg) * UNIT_COLS, j0 = sg * UNIT_CELLS;
+    const int sg = local / ncg, i0 = (local - sg * ncg) * COLS, j0 = sg * UNIT_CELLS;
     const int n = I.ny, bclo = I.bc[2], bchi = I.bc[3];
     bool fl;
     if (mode == UNITS_FAR || mode == UNITS_NEAR) {
-        bool far = i0 + UNIT_COLS - 1 < y.col0 || i0 > y.col1 ||
+        bool far = i0 + COLS - 1 < y.col0 || i0 > y.col1 ||
                    (bclo != 2 && (j0 + UNIT_CELLS + 2 < y.row0 || j0 - 3 > y.row1));
         if (!far && !y.defer_all) {
             int t = 0;
-            for (int e = threadIdx.x; e < (UNIT_CELLS + 6) * UNIT_COLS; e += 256) {
-                const int i = i0 + (e & (UNIT_COLS - 1));
-                if (i < I.nx) t |= I.cls[ghost_map(j0 - 3 + (e >> 3), n, bclo, bchi, &fl) * I.pitch + i];
+            for (int e = threadIdx.x; e < (UNIT_CELLS + 6) * COLS; e += 256) {
+                const int i = i0 + e % COLS;
+                if (i < I.nx) t |= I.cls[ghost_map(j0 - 3 + e / COLS, n, bclo, bchi, &fl) * I.pitch + i];
             }
             far = !__syncthreads_or(t & CLS_TOUCH);
         }
@@ -894,8 +912,8 @@ __global__ void __launch_bounds__(256, 2) k_unit_y(const InstDesc *__restrict__ 
     }
     const size_t plane = (size_t)I.pitch * n;
     const T *__restrict__ Q = (const T *)I.Q[src];
-    for (int e = threadIdx.x; e < ROWS * UNIT_COLS; e += 256) {
-        const int r = e >> 3, c = e & (UNIT_COLS - 1);
+    for (int e = threadIdx.x; e < ROWS * COLS; e += 256) {
+        const int r = e / COLS, c = e % COLS;
         bool flip;
         const int ci = ghost_map(j0 - 2 + r, n, bclo, bchi, &flip) * I.pitch + min(i0 + c, I.nx - 1);
         sc[r][c] = I.cls[ci];
@@ -906,35 +924,39 @@ __global__ void __launch_bounds__(256, 2) k_unit_y(const InstDesc *__restrict__ 
         }
     }
     __syncthreads();
-    const int i = i0 + w, pos = j0 - 1 + lane;
+    const int pos = j0 - 1 + lane;
+    const Flow<T, EQ> f(I, sizeof(T) == 4 ? (T)y.lamf : (T)y.lam, 1);
     T s0 = T(0), s1 = T(0);
-    T qm[NC], q0[NC], qp[NC], qn[NC];
-    bool st = false;
-    if (i < I.nx) {   // whole warps
 #pragma unroll
-        for (int k = 0; k < NC; ++k) {
-            qm[k] = sq[k][lane][w];
-            q0[k] = sq[k][lane + 1][w];
-            qp[k] = sq[k][lane + 2][w];
-        }
-        const int cm = sc[lane][w], c0 = sc[lane + 1][w], cp = sc[lane + 2][w];
-        const Flow<T, EQ> f(I, sizeof(T) == 4 ? (T)y.lamf : (T)y.lam, 1);
-        st = mode == UNITS_FAR || mode == UNITS_PLAIN
-            ? unit_update<T, EQ, 1, false>(I, y, R, f, i, pos, n, qm, q0, qp, cm, c0, cp, last != 0, qn, s0, s1)
-            : unit_update<T, EQ, 1, true>(I, y, R, f, i, pos, n, qm, q0, qp, cm, c0, cp, last != 0, qn, s0, s1);
-        __syncwarp();
-        if (st) {   // a warp's column is its own
+    for (int u = 0; u < K; ++u) {
+        const int c = w + u * UNIT_COLS, i = i0 + c;
+        T qm[NC], q0[NC], qp[NC], qn[NC];
+        bool st = false;
+        if (i < I.nx) {   // whole warps
 #pragma unroll
-            for (int k = 0; k < NC; ++k) sq[k][lane + 1][w] = qn[k];
+            for (int k = 0; k < NC; ++k) {
+                qm[k] = sq[k][lane][c];
+                q0[k] = sq[k][lane + 1][c];
+                qp[k] = sq[k][lane + 2][c];
+            }
+            const int cm = sc[lane][c], c0 = sc[lane + 1][c], cp = sc[lane + 2][c];
+            st = mode == UNITS_FAR || mode == UNITS_PLAIN
+                ? unit_update<T, EQ, 1, false>(I, y, R, f, i, pos, n, qm, q0, qp, cm, c0, cp, last != 0, qn, s0, s1)
+                : unit_update<T, EQ, 1, true>(I, y, R, f, i, pos, n, qm, q0, qp, cm, c0, cp, last != 0, qn, s0, s1);
+            __syncwarp();
+            if (st) {   // a warp's columns are its own
+#pragma unroll
+                for (int k = 0; k < NC; ++k) sq[k][lane + 1][c] = qn[k];
+            }
         }
+        if (lane >= 1 && lane <= UNIT_CELLS) sst[lane - 1][c] = st;
     }
-    if (lane >= 1 && lane <= UNIT_CELLS) sst[lane - 1][w] = st;
     if (EQ == 0) finish_warp<T>(y, last != 0, s0, s1);
     else if (last) put_advection<T>(I, y, s0 > T(0));
     __syncthreads();
     T *__restrict__ Qo = (T *)I.Q[dst];
-    for (int e = threadIdx.x; e < UNIT_CELLS * UNIT_COLS; e += 256) {
-        const int r = e >> 3, c = e & (UNIT_COLS - 1);
+    for (int e = threadIdx.x; e < UNIT_CELLS * COLS; e += 256) {
+        const int r = e / COLS, c = e % COLS;
         if (!sst[r][c]) continue;
         const size_t ci = (size_t)(j0 + r) * I.pitch + i0 + c;
 #pragma unroll
@@ -3141,18 +3163,23 @@ void launch_band_stage(int stage, const InstDesc *D, InstDyn *Y, BandRec *R, con
     }
 }
 
-// the scalar kernels over total units (x: warps, y: CTAs), in the mode
-// UNITS_*
+// the scalar kernels over total work items (x: warps, y: CTAs) of units units
+// each (advection: 1 or UNIT_WIDE), in the mode UNITS_*
 template <class T>
 void launch_units(int dir, int eq, const InstDesc *D, InstDyn *Y, const BandRec *R, int n_inst, int total, int src,
-                  int dst, int last, int mode, cudaStream_t st) {
+                  int dst, int last, int units, int mode, cudaStream_t st) {
     const unsigned bx = (unsigned)((total + 3) / 4);
     if (eq == 1) {
-        if (dir == 0) k_unit_x<T, 1><<<bx, 128, 0, st>>>(D, Y, R, n_inst, total, src, dst, last, mode);
-        else k_unit_y<T, 1><<<total, 256, 0, st>>>(D, Y, R, n_inst, src, dst, last, mode);
+        if (dir == 0) {
+            if (units == 1) k_unit_x<T, 1, 1><<<bx, 128, 0, st>>>(D, Y, R, n_inst, total, src, dst, last, mode);
+            else k_unit_x<T, 1, UNIT_WIDE><<<bx, 128, 0, st>>>(D, Y, R, n_inst, total, src, dst, last, mode);
+        } else {
+            if (units == 1) k_unit_y<T, 1, 1><<<total, 256, 0, st>>>(D, Y, R, n_inst, src, dst, last, mode);
+            else k_unit_y<T, 1, UNIT_WIDE><<<total, 256, 0, st>>>(D, Y, R, n_inst, src, dst, last, mode);
+        }
     } else if constexpr (sizeof(T) == 8) {
-        if (dir == 0) k_unit_x<T, 0><<<bx, 128, 0, st>>>(D, Y, R, n_inst, total, src, dst, last, mode);
-        else k_unit_y<T, 0><<<total, 256, 0, st>>>(D, Y, R, n_inst, src, dst, last, mode);
+        if (dir == 0) k_unit_x<T, 0, 1><<<bx, 128, 0, st>>>(D, Y, R, n_inst, total, src, dst, last, mode);
+        else k_unit_y<T, 0, 1><<<total, 256, 0, st>>>(D, Y, R, n_inst, src, dst, last, mode);
     }
 }
 
@@ -3163,13 +3190,14 @@ void launch_units(int dir, int eq, const InstDesc *D, InstDyn *Y, const BandRec 
 // scalar kernels: mode is UNITS_*.
 template <class T>
 void launch_bulk(int dir, int eq, const InstDesc *D, InstDyn *Y, const BandRec *R, int n_inst, int total_warps,
-                 int src, int dst, int last, int shape, int mode, DeferList dl, int any_defer_all, cudaStream_t st) {
+                 int src, int dst, int last, int shape, int units, int mode, DeferList dl, int any_defer_all,
+                 cudaStream_t st) {
     const int cta = shape & 1023;
     const int wpc = cta / 32;   // warps per CTA of the FP32x2 kernels
     if (total_warps <= 0) return;
     const bool packed = sizeof(T) == 4 && eq == 0;   // FP32 Euler: the FP32x2 kernels
     if (!packed) {
-        launch_units<T>(dir, eq, D, Y, R, n_inst, total_warps, src, dst, last, mode, st);
+        launch_units<T>(dir, eq, D, Y, R, n_inst, total_warps, src, dst, last, units, mode, st);
         return;
     }
     const int pg = (total_warps + wpc - 1) / wpc;
@@ -3238,7 +3266,7 @@ void launch_read_state(const InstDesc *D, H *const *ptrs, H *p1, int inst0, int 
     template void launch_band_stage<T>(int, const InstDesc *, InstDyn *, BandRec *, const double *, int *,          \
                                        int, int, int, int, int, int, int, int, cudaStream_t);                     \
     template void launch_bulk<T>(int, int, const InstDesc *, InstDyn *, const BandRec *, int, int, int, int, int,  \
-                                 int, int, DeferList, int, cudaStream_t);                                               \
+                                 int, int, int, DeferList, int, cudaStream_t);                                          \
     template int bulk_blocks_per_sm<T>(int);                                                                       \
     template void launch_axisym_source<T>(const InstDesc *, InstDyn *, int, int, int, cudaStream_t);               \
     template void launch_write_state<T, double>(const InstDesc *, InstDyn *, const double *const *, const double *, \

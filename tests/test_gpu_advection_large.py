@@ -2,6 +2,7 @@
 more than moving each cell once."""
 import time
 
+import numpy as np
 import pytest
 
 from paper_1711_11361_gb300 import inputs
@@ -47,3 +48,36 @@ def test_no_body_no_second_launch(precision):
         kernels.append(sim.graph_kernels())
     assert kernels[0] == kernels[1], kernels
     sim.close()
+
+
+def test_several_units_per_warp():
+    """4096 x 4096 cells in FP32: 0.47 ms per step with a unit of 30 cells per warp, 0.24 with four (0.24 with a warp
+    per row or segment of rows)."""
+    assert _step_ms(_open(4096), 1, 20) <= 0.36
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("periodic", [False, True])
+@pytest.mark.parametrize("nx,ny", [(119, 8), (120, 31), (121, 30), (8, 257), (33, 61), (63, 29), (240, 90)])
+def test_wide_units_give_the_same_bits(nx, ny, periodic, precision):
+    """A small grid around the channel's walls in a batch large enough for four units per warp, and alone: the units'
+    ends lie elsewhere, the arithmetic per cell is the same."""
+    from paper_1711_11361_gb300 import mb
+    p = inputs.c1_advection(64)
+    p.nx, p.ny = nx, ny
+    if not periodic:
+        p.bc = (inputs.TRANSMISSIVE, inputs.TRANSMISSIVE, inputs.REFLECTIVE, inputs.TRANSMISSIVE)
+    rng = np.random.default_rng(nx + ny)
+    p.Q0 = rng.uniform(0.5, 1.5, (1, ny, nx))
+    big = _open(1500)
+    alone, batch = mb.Sim(p, precision), mb.Sim([p, big, p], precision)
+    for k in range(3):
+        dt = alone.step(0.0, report=True)[0]
+        batch.step(float(dt))
+    want = alone.read_state(0, alpha=True)
+    for k in (0, 2):
+        got = batch.read_state(k, alpha=True)
+        assert np.array_equal(got["Q"], want["Q"], equal_nan=True) and np.array_equal(got["alpha"], want["alpha"])
+    assert np.any(want["alpha"] == 0.0) and np.all(np.isfinite(want["Q"][:, want["alpha"] > 0]))
+    alone.close()
+    batch.close()
