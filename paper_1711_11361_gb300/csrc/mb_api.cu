@@ -28,6 +28,7 @@ void launch_pose(const InstDesc *, InstDyn *, const double *, const double *, co
                  double *, double *, float *, int, int, int, int, double, int *, cudaStream_t);
 void launch_geom(const InstDesc *, InstDyn *, const int *, const double *, const double *, const float *, const int *,
                  const unsigned char *, int, int, int, int, int, BandRec *, double *, cudaStream_t);
+void launch_edge_capacity(const InstDesc *, InstDyn *, const int *, const float *, int, int, int, int, cudaStream_t);
 void launch_classify(const InstDesc *, InstDyn *, const double *, const double *, const unsigned char *, double *,
                      double *, float *, const int *, int, int, int, int, double *, cudaStream_t);
 template <class T>
@@ -75,6 +76,7 @@ struct mb_sim {
     float *ebox = nullptr;        // FP32 x-bounds of every edge at the three poses
     unsigned char *vmov = nullptr;
     int *vnext = nullptr;
+    int max_nv = 0;               // most vertices of an instance
     int total_v = 0;
     BandRec *rec = nullptr;
     double *bnd = nullptr;
@@ -488,6 +490,8 @@ static cudaError_t relayout(mb_sim *s, int old_n, const std::vector<int> &from) 
     if (e != cudaSuccess) return e;
     s->n = n;
     s->total_v = (int)hvx.size();
+    s->max_nv = 0;
+    for (const auto &I : s->hd) s->max_nv = std::max(s->max_nv, I.nv);
     s->total_rec = rec_total;
     s->total_cols = col_total;
     s->total_tiles[0] = tiles0;
@@ -691,6 +695,9 @@ static mb_status do_sweep(mb_sim *s, int dir, double dt) {
             launch_band_stage<double>(stage, s->dd, s->dy, s->rec, s->bnd, s->boff, s->n, s->total_rec,
                                       dir, src, dst, qn, s->sidx, last, sx);
     };
+    auto capacity = [&]() {
+        launch_edge_capacity(s->dd, s->dy, s->ginst, s->ebox, s->total_v, s->max_nv, s->total_cols, s->gcw, st);
+    };
     auto geom_band = [&](cudaStream_t sx) {
         launch_geom(s->dd, s->dy, s->ginst, s->px, s->py, s->ebox, s->vnext, s->vmov, s->total_v, s->n, s->total_cols,
                     s->gcw, dir, s->rec, s->bnd, sx);
@@ -727,10 +734,12 @@ static mb_status do_sweep(mb_sim *s, int dir, double dt) {
         geom_band(s->side);
         band(2, s->side);   // covering / uncovering: band records only, no bulk cell
         cudaEventRecord(s->ev_join, s->side);
+        capacity();
         bulk(0);
         cudaStreamWaitEvent(st, s->ev_join, 0);
         bulk(1);
     } else {
+        capacity();
         geom_band(st);
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         if (s->timing) {

@@ -1448,6 +1448,34 @@ __device__ __forceinline__ void geom_group(int gw, const InstDesc *__restrict__ 
     if (err) atomicOr(&y.err, err);
 }
 
+// For groups narrower than GC columns: the edge capacity is one of GC columns
+// whatever the groups' width, which follows the batch, so that what one batch
+// refuses another does not take and a simulation under way meets no new limit
+// when its batch grows.  One CTA per group; the first of every GC columns
+// counts their edges at the poses that geom_group gathers.  Launched only
+// where an instance has more than EMAXG vertices, beside the geometry: counting
+// in k_geom lengthened the chain of a 1024 x 1024 grid around the aerofoil by
+// 1 to 2%, a launch before it by 6%.
+__global__ void __launch_bounds__(GEOMG_THREADS) k_edge_capacity(const InstDesc *__restrict__ D, InstDyn *__restrict__ Y,
+                                                                 const int *__restrict__ ginst,
+                                                                 const float *__restrict__ ebox, int total_v, int gcw) {
+    const InstDesc &I = D[ginst[blockIdx.x]];
+    InstDyn &y = Y[ginst[blockIdx.x]];
+    const int g = gcw * (blockIdx.x - I.gcol_off), g0 = y.col0 + g, last = min(y.col1, I.nx - 1);
+    if (I.nv <= EMAXG || g % GC != 0 || g0 > last || y.row1 < y.row0 || (y.row1 - y.row0) / 32 + 1 > NWB) return;
+    const double ad = fabs(y.delta);
+    const float fl = __double2float_rd(I.xn[g0] - ad), fr = __double2float_ru(I.xn[min(g0 + GC, last + 1)] + ad);
+    for (int P = I.rotating ? 0 : 1; P < 3; ++P) {
+        const float2 *EB = (const float2 *)(ebox + (size_t)P * total_v * 2) + I.voff;
+        int cnt = 0;
+        for (int k0 = 0; k0 < I.nv; k0 += GEOMG_THREADS) {
+            const int k = k0 + threadIdx.x;
+            cnt += __syncthreads_count(k < I.nv && EB[k].y >= fl && EB[k].x <= fr);
+        }
+        if (cnt > EMAXG && threadIdx.x == 0) atomicOr(&y.err, ERR_EDGE_CAP);
+    }
+}
+
 // One CTA per geometry group (a grid capped below the group count, looping
 // over the groups so that bulk CTAs find room beside it, measured slower).
 // Bound by latency: FP64 chains and barriers of few warps.  400 x 400 grid
@@ -1614,6 +1642,12 @@ void launch_pose(const InstDesc *D, InstDyn *Y, const double *vx, const double *
                  double dt, int *defer_count, cudaStream_t st) {
     k_pose<<<n_inst * POSE_PARTS, 256, 0, st>>>(D, Y, vx, vy, vmov, vnext, px, py, ebox, total_v, dir, sidx, dt,
                                                  defer_count);
+}
+
+void launch_edge_capacity(const InstDesc *D, InstDyn *Y, const int *ginst, const float *ebox, int total_v, int max_nv,
+                          int total_groups, int gcw, cudaStream_t st) {
+    if (total_groups > 0 && gcw < GC && max_nv > EMAXG)
+        k_edge_capacity<<<total_groups, GEOMG_THREADS, 0, st>>>(D, Y, ginst, ebox, total_v, gcw);
 }
 
 void launch_geom(const InstDesc *D, InstDyn *Y, const int *ginst, const double *px, const double *py, const float *ebox,
