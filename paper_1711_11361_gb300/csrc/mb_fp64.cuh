@@ -28,7 +28,9 @@ __device__ __forceinline__ double widen_scaled(float r, int shift) {
 // truncated significand and 2^-23 from rcp.approx), then one step of the
 // third-order hyperpower iteration y = y0 (1 + e + e^2), e = 1 - d y0.  The
 // remaining error e^3 < 2^-63 is below the last rounding: 3 FP64
-// instructions.  A zero gives infinity and a NaN NaN.
+// instructions.  A zero gives infinity, a NaN NaN, and an infinity (not 0 as
+// in 1 / d) no finite number either: a flow that overflows does not come back
+// as one that looks sound.
 __device__ __forceinline__ double rcp64(double d) {
     const int hi = __double2hiint(d), lo = __double2loint(d);
     float r;
