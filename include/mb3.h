@@ -83,10 +83,10 @@ mb_status mb3_last_sweep(mb3_sim *sim, double *wall, int *merged);
  * part and the CFL wave speeds in FP32, from an FP32 copy of the state kept
  * beside it).  Geometry, wall states and shielded fluxes, the update of the
  * contents, covering and uncovering, the safeguard and the state stay FP64,
- * and fluxes are stored in FP64, so the update stays conservative to FP64
- * rounding.  Allocates two copies (4 bytes x 5 per cell each: a sweep's old
- * and new state) on first use;
- * MB_E_STATE in the middle of a step, MB_E_INVAL for another value. */
+ * and every difference of two fluxes is the FP64 one (taken in FP32 only where
+ * it is exact), so the update stays conservative to FP64 rounding.  Allocates
+ * two copies (4 bytes x 5 per cell each: a sweep's old and new state) on first
+ * use; MB_E_STATE in the middle of a step, MB_E_INVAL for another value. */
 mb_status mb3_set_precision(mb3_sim *sim, int precision);
 /* device time (ms) of the last sweep's flow kernels (MUSCL-Hancock + HLLC +
  * stabilised flux of every face along the sweep, and the content update),

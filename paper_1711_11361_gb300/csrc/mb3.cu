@@ -66,8 +66,8 @@ struct Body3 {
 // than the margin (the rounding of the inputs and of the sums is below 12 x
 // 2^-24 of the terms' magnitudes, the margin 4e-6 of them), so a decision is
 // the FP64 tests' too.  Most of R is decided so, off the FP64 pipe (44 x 44 x
-// 24 cells, two poses: 672 us per launch with FP64 tests, 418 so; 9.9 M FP64
-// warp instructions against 4.9 M).
+// 24 cells, two poses: 672 us per launch with FP64 tests, 407 to 468 so; 9.9 M
+// FP64 warp instructions against 4.7 M).
 __device__ __forceinline__ int side_of(const Body3 &B, int f, const float *lo, const float *h, const float *big) {
     float c = B.cf[f], least = 0.0f, most = 0.0f, mag = fabsf(c);
     for (int a = 0; a < 3; ++a) {
@@ -958,14 +958,14 @@ __device__ __forceinline__ bool near_line(const Desc &D, int d, const int *ijk) 
 // x sweep.  The line kernels keep the evolved states and the fluxes in
 // registers: per cell they read the state and write the new one (80 bytes; 120
 // with the FP32 copy), where a kernel each for the states, the fluxes, the
-// update and the new state moved 400.  FP64: bound by the FP64 pipe, 173 lane
-// operations per cell; 4 M cells per sweep, before -> after: x 2520 -> 1267
-// us, y 2400 -> 1369, z 2390 -> 1374 (0.85 of the pipe's rate).  FP32 option:
-// 10 FP64 lane operations per cell (the update) and about 700 instructions;
-// 32 M cells per sweep, 3790 -> 857 us (x), 1036, 1066.  Rows are laid end
-// to end as slots, position -1 .. nx of every row, and a warp takes 32 slots
-// from slot 30 w on: it evolves 32 positions, forms 31 fluxes and updates 30
-// cells, whatever the row length.
+// update and the new state moved 400.  FP64: bound by the FP64 pipe, 153 to
+// 158 lane operations per cell; 4 M cells per sweep, before -> after: x 2520
+// -> 1161 us, y 2400 -> 1212, z 2390 -> 1225 (0.80 to 0.87 of the pipe's
+// rate).  FP32 option: 12 to 13 FP64 lane operations per cell (the update) and
+// 670 to 790 instructions; 32 M cells per sweep, 3790 -> 857 us (x), 1041,
+// 1066.  Rows are laid end to end as slots, position -1 .. nx of every row, and
+// a warp takes 32 slots from slot 30 w on: it evolves 32 positions, forms 31
+// fluxes and updates 30 cells, whatever the row length.
 template <typename T, bool GEN>
 __device__ __forceinline__ void row_unit(const Desc &D, bool store, int p, int j, int k) {
     const Flow<T, 0> fl(D);
