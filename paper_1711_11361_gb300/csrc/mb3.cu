@@ -958,11 +958,12 @@ __device__ __forceinline__ bool near_line(const Desc &D, int d, const int *ijk) 
 // x sweep.  The line kernels keep the evolved states and the fluxes in
 // registers: per cell they read the state and write the new one (80 bytes; 120
 // with the FP32 copy), where a kernel each for the states, the fluxes, the
-// update and the new state moved 400.  FP64: bound by the FP64 pipe, 153 to
-// 158 lane operations per cell; 4 M cells per sweep, before -> after: x 2520
-// -> 1161 us, y 2400 -> 1212, z 2390 -> 1225 (0.80 to 0.87 of the pipe's
-// rate).  FP32 option: 12 to 13 FP64 lane operations per cell (the update) and
-// 670 to 790 instructions; 32 M cells per sweep, 3790 -> 857 us (x), 1041,
+// update and the new state moved 400.  FP64: bound by the FP64 pipe; 4 M cells
+// whose states all vary, per sweep, before -> after: x 2520 -> 1265 us, y 2400
+// -> 1368, z 2390 -> 1373, 173 lane operations per cell at 0.85 of the pipe's
+// rate (uniform states on both sides of a shock take fewer: 153 to 158, 1161 to
+// 1225 us).  FP32 option: 12 to 13 FP64 lane operations per cell (the update)
+// and 670 to 790 instructions; 32 M cells per sweep, 3790 -> 857 us (x), 1041,
 // 1066.  Rows are laid end to end as slots, position -1 .. nx of every row, and
 // a warp takes 32 slots from slot 30 w on: it evolves 32 positions, forms 31
 // fluxes and updates 30 cells, whatever the row length.

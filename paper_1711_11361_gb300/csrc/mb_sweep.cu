@@ -641,9 +641,10 @@ __device__ __forceinline__ int find_inst_io(const InstDesc *__restrict__ D, int 
 // warps, where a warp per row (x) or per 64 rows (y) left most SMs idle.
 // Measured per sweep, FP64 Euler, before -> after: 399 x 399, x 286 -> 73 us,
 // y 1380 -> 90 us (its two launches together); 4.9 M cells in 16 grids, x
-// 2950 -> 1428 us, y 4090 -> 1430 us, 0.86 of the FP64 pipe's rate for the
-// 139 to 150 lane operations per cell this flow executes (263 in x and 289 in
-// y with CUDA's division and square root and comparisons on the FP64 pipe).
+// 2950 -> 1428 us, y 4090 -> 1430 us, 0.86 of the FP64 pipe's rate for about
+// 157 lane operations per cell where all states vary (139 in x and 150 in y
+// where most are uniform; there 263 and 289 with CUDA's division and square
+// root and comparisons on the FP64 pipe).
 // Advection takes a few operations per cell, so there a unit costs little more
 // than finding its place: large batches of it give a warp UNIT_WIDE units of a
 // row in x, and as many columns in y.  FP32 without a body, ms per step, one
